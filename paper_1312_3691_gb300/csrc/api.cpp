@@ -220,7 +220,7 @@ tpmc_status Ctx::run(const MeshRec& m, const QueryDev* h_queries, uint32_t nq, c
   if ((e = cudaMemsetAsync(s_misc.ptr, 0, 128, stream)) != cudaSuccess) return cuda_fail(e, "clear counter");
   // the set-up also clears the queries' accumulators
   if ((e = launch_setup(d_queries, nq, h_base ? (const QueryDev*)s_base.ptr : nullptr, d_dirs, d_S,
-                        h_base ? d_items : nullptr, nullptr, d_acc, nq, stream)) != cudaSuccess)
+                        h_base ? d_items : nullptr, nullptr, d_acc, nq, vn_table, stream)) != cudaSuccess)
     return cuda_fail(e, "setup kernel");
   TraceArgs a{};
   a.mesh = m.dev;
@@ -378,11 +378,11 @@ tpmc_status tpmc_create(int device, size_t mem_budget_bytes, tpmc_ctx** out) {
   if ((e = cudaMallocHost(&c->h_pinned, 4096)) != cudaSuccess) return cuda_fail(e, "cudaMallocHost");
   {
     void* t = nullptr;
-    tpmc_status st = c->alloc(&t, sizeof(float) * kVnNS * kVnNZ, "normal-speed table");
+    tpmc_status st = c->alloc(&t, sizeof(float) * kTableFloats, "start tables");
     if (st != TPMC_OK) return st;
     c->vn_table = (float*)t;
-    if ((e = launch_vn_table(c->vn_table, c->stream)) != cudaSuccess) return cuda_fail(e, "normal-speed table");
-    if ((e = cudaStreamSynchronize(c->stream)) != cudaSuccess) return cuda_fail(e, "normal-speed table");
+    if ((e = launch_tables(c->vn_table, c->stream)) != cudaSuccess) return cuda_fail(e, "start tables");
+    if ((e = cudaStreamSynchronize(c->stream)) != cudaSuccess) return cuda_fail(e, "start tables");
   }
   c->h_err_word = (int*)c->h_pinned;
   *c->h_err_word = 0;

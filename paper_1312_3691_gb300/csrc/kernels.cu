@@ -1638,87 +1638,202 @@ __global__ void __launch_bounds__(MINB > 0 ? 128 : 256, MINB > 0 ? MINB : (sizeo
 }
 
 // ---------------------------------------------------------- set-up kernel
-__device__ double latitude_cdf_d(double x, double S, double K1, double D) {
-  const double Sx = S * x;
-  return (kSqrtPiD / (4.0 * S) * (2.0 * Sx * Sx + 1.0) * erfc(-Sx) + 0.5 * x * exp(-Sx * Sx) - K1) / D;
-}
-__device__ double latitude_pdf_d(double x, double S, double D) {
-  const double Sx = S * x;
-  return (exp(-Sx * Sx) + kSqrtPiD * Sx * erfc(-Sx)) / D;
-}
-
-// Block b prepares query b.  With `base` set, query b is a copy of *base whose
+// Set-up of query blockIdx.x, spread over the chip: gridDim.y = 1 (one block
+// does it all) or kSetupParts (block y = 0: the scalars; the others: the
+// latitude start table).  With `base` set, query b is a copy of *base whose
 // direction / speed ratio come from dirs[b] / Svals[b] (when given) and whose
 // Philox stream is base->stream_id + b; with `items` set, it also writes work
 // item b = particles [0, N) of query b at work indices [b N, (b+1) N).
-__global__ void setup_kernel(QueryDev* qs, const QueryDev* base, const double* dirs, const double* Svals,
-                             ItemDev* items, const uint32_t* slots, AccStripe* acc, uint32_t acc_stride) {
+//
+// What bounds it is double-precision latency: an SM issues a double warp
+// instruction every 16 cycles or so, whether one lane is active or 32, and a
+// library function is a chain of 50 to 200 of them.  So independent functions
+// run in different warps, arguments of one function (erfc and exp at S, -S and
+// the six box faces) in the lanes of one warp, and with few queries the table
+// in blocks of its own.  The table's root searches start from a bracket and
+// two Newton steps in float, which leaves two to four double evaluations of the
+// law per knot; started at 2u - 1 it took up to 54 in the lower tail.  With that
+// start, and one thread doing the scalars, a call took 320 us for 8 queries and
+// 3.31 ms for 3,072; now 16 us and 0.33 ms.
+constexpr int kSetupThreads = 160;
+constexpr int kSetupParts = 6;
+
+__global__ void __launch_bounds__(kSetupThreads)
+    setup_kernel(QueryDev* qs, const QueryDev* base, const double* dirs, const double* Svals, ItemDev* items,
+                 const uint32_t* slots, AccStripe* acc, uint32_t acc_stride, const double* knots) {
   const uint32_t slot = slots != nullptr ? slots[blockIdx.x] : blockIdx.x;
   QueryDev& q = qs[slot];
-  // the query's sums start at zero: its kAccStripes stripes of 16 words each
-  for (uint32_t i = threadIdx.x; i < (uint32_t)kAccStripes * 16u; i += blockDim.x)
-    reinterpret_cast<unsigned long long*>(&acc[(size_t)(i >> 4) * acc_stride + slot])[i & 15u] = 0ull;
-  __shared__ int s_ok;
+  const QueryDev& in = base != nullptr ? *base : q;  // the inputs (T_inf, m, V, dir, ...)
+  const bool scalars = blockIdx.y == 0, table = gridDim.y == 1 || blockIdx.y != 0;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  __shared__ double s_V, s_S, s_c, s_cw, s_dn, s_vh[3], s_erfc[8], s_exp[8], s_erf, s_erfcx, s_D, s_K1;
+  __shared__ int s_st, s_shift_bad;
+  __shared__ float s_H[kSetupThreads];
+
+  if (scalars) {
+    // the query's sums start at zero: its kAccStripes stripes of 16 words each
+    for (uint32_t i = threadIdx.x; i < (uint32_t)kAccStripes * 16u; i += blockDim.x)
+      reinterpret_cast<unsigned long long*>(&acc[(size_t)(i >> 4) * acc_stride + slot])[i & 15u] = 0ull;
+    if (base != nullptr) {  // all of *base but the start table, which other blocks write
+      constexpr uint32_t kTab0 = offsetof(QueryDev, htab) / 4, kTab1 = kTab0 + kHTable + 1;
+      for (uint32_t i = threadIdx.x; i < sizeof(QueryDev) / 4; i += blockDim.x)
+        if (i < kTab0 || i >= kTab1) reinterpret_cast<uint32_t*>(&q)[i] = reinterpret_cast<const uint32_t*>(base)[i];
+      __syncthreads();
+    }
+  }
+  if (threadIdx.x == 0) {
+    s_c = sqrt(2.0 * kBoltz * in.T_inf / in.m);
+    s_V = Svals != nullptr ? Svals[blockIdx.x] * s_c : in.V;
+    s_S = s_V / s_c;
+    s_shift_bad = 0;
+  } else if (threadIdx.x == 32 && scalars) {
+    const double* d = dirs != nullptr ? dirs + 3 * (size_t)blockIdx.x : in.dir;
+    const double d0 = d[0], d1 = d[1], d2 = d[2];
+    s_dn = sqrt(d0 * d0 + d1 * d1 + d2 * d2);
+    s_vh[0] = d0 / s_dn;
+    s_vh[1] = d1 / s_dn;
+    s_vh[2] = d2 / s_dn;
+    if (dirs != nullptr) { q.dir[0] = d0; q.dir[1] = d1; q.dir[2] = d2; }
+  } else if (threadIdx.x == 64 && scalars) {
+    s_cw = sqrt(q.T_W / q.T_inf);
+  } else if (threadIdx.x == 96 && scalars && items != nullptr) {
+    ItemDev it;
+    it.g_begin = (uint64_t)blockIdx.x * q.N;
+    it.pid_begin = 0;
+    it.count = q.N;
+    it.query = blockIdx.x;
+    it.pad = 0;
+    items[blockIdx.x] = it;
+  }
+  __syncthreads();
   if (threadIdx.x == 0) {
     int st = TPMC_OK;
-    if (base != nullptr) {
-      q = *base;
-      q.stream_id = base->stream_id + blockIdx.x;
+    if (!(isfinite(s_V) && s_V > 0.0) || (scalars && !(isfinite(s_dn) && s_dn > 0.0))) st = TPMC_EINVAL;
+    if (!(s_S >= 0.01 && s_S <= 50.0)) st = TPMC_EINVAL;
+    s_st = st;
+    if (scalars) {
+      if (base != nullptr) q.stream_id = base->stream_id + blockIdx.x;
+      if (Svals != nullptr) q.V = s_V;
     }
-    if (items != nullptr) {
-      ItemDev it;
-      it.g_begin = (uint64_t)blockIdx.x * q.N;
-      it.pid_begin = 0;
-      it.count = q.N;
-      it.query = blockIdx.x;
-      it.pad = 0;
-      items[blockIdx.x] = it;
+  }
+  __syncthreads();
+  const bool sphere = in.cv_kind == TPMC_CV_SPHERE;
+  if (s_st != TPMC_OK) {
+    if (scalars && threadIdx.x == 0) q.status = s_st;
+    if (table && base != nullptr)
+      for (int j = threadIdx.x; j <= kHTable; j += blockDim.x) q.htab[j] = 0.0f;
+    return;
+  }
+  const double S = s_S;
+
+  // ---- functions of S and the faces' speed ratios, a warp to each function
+  if (warp == 0 && lane < 8) {
+    // lane 0: S, lane 1: -S, lanes 2-7: minus the inward-normal speed ratio of each box face
+    double a = lane == 0 ? S : -S;
+    if (lane >= 2 && scalars) {
+      const int f = lane - 2;
+      const double v = s_vh[f >> 1];
+      a = -(S * (f % 2 == 0 ? -v : v));
     }
-    if (dirs != nullptr)
-      for (int i = 0; i < 3; ++i) q.dir[i] = dirs[3 * blockIdx.x + i];
-    const double c = sqrt(2.0 * kBoltz * q.T_inf / q.m);
-    if (Svals != nullptr) q.V = Svals[blockIdx.x] * c;
-    const double dn = sqrt(q.dir[0] * q.dir[0] + q.dir[1] * q.dir[1] + q.dir[2] * q.dir[2]);
-    if (!(isfinite(q.V) && q.V > 0.0) || !(isfinite(dn) && dn > 0.0)) st = TPMC_EINVAL;
-    const double S = q.V / c;
-    if (!(S >= 0.01 && S <= 50.0)) st = TPMC_EINVAL;
-    if (st == TPMC_OK) {
-      q.S = S;
-      q.c_mp = c;
-      q.cw = sqrt(q.T_W / q.T_inf);
-      double vh[3];
-      for (int i = 0; i < 3; ++i) { vh[i] = q.dir[i] / dn; q.vhat[i] = vh[i]; }
-      // Eq. 15: rotation about u = z x Vhat by beta = acos(z . Vhat), carrying +z onto Vhat.
-      const double ux = -vh[1], uy = vh[0];  // z x Vhat = (-Vy, Vx, 0)
-      const double sb = sqrt(ux * ux + uy * uy);
-      const double cb = fmin(1.0, fmax(-1.0, vh[2]));
-      double Rm[9];
-      if (sb < 1e-12) {
-        const double sg = cb > 0.0 ? 1.0 : -1.0;  // identity, or a half turn about x
-        Rm[0] = 1; Rm[1] = 0; Rm[2] = 0; Rm[3] = 0; Rm[4] = sg; Rm[5] = 0; Rm[6] = 0; Rm[7] = 0; Rm[8] = sg;
+    s_erfc[lane] = erfc(a);
+    s_exp[lane] = exp(-a * a);
+  } else if (warp == 1 && lane == 0) {
+    s_erf = erf(S);
+  } else if (warp == 2 && lane == 0 && scalars) {
+    s_erfcx = erfcx(S);
+  } else if (warp == 3 && lane == 0 && scalars) {
+    // Eq. 15: rotation about u = z x Vhat by beta = acos(z . Vhat), carrying +z onto Vhat.
+    const double* vh = s_vh;
+    const double ux = -vh[1], uy = vh[0];  // z x Vhat = (-Vy, Vx, 0)
+    const double sb = sqrt(ux * ux + uy * uy);
+    const double cb = fmin(1.0, fmax(-1.0, vh[2]));
+    double Rm[9];
+    if (sb < 1e-12) {
+      const double sg = cb > 0.0 ? 1.0 : -1.0;  // identity, or a half turn about x
+      Rm[0] = 1; Rm[1] = 0; Rm[2] = 0; Rm[3] = 0; Rm[4] = sg; Rm[5] = 0; Rm[6] = 0; Rm[7] = 0; Rm[8] = sg;
+    } else {
+      const double kx = ux / sb, ky = uy / sb;  // unit axis (kx, ky, 0)
+      const double beta = acos(cb);
+      const double cs = cos(beta), sn = sin(beta), oc = 1.0 - cs;
+      Rm[0] = cs + kx * kx * oc; Rm[1] = kx * ky * oc;      Rm[2] = ky * sn;
+      Rm[3] = kx * ky * oc;      Rm[4] = cs + ky * ky * oc; Rm[5] = -kx * sn;
+      Rm[6] = -ky * sn;          Rm[7] = kx * sn;           Rm[8] = cs;
+    }
+    for (int i = 0; i < 9; ++i) { q.R[i] = Rm[i]; q.fc[kFcR + i] = (float)Rm[i]; }
+    for (int i = 0; i < 3; ++i) {
+      q.vhat[i] = vh[i];
+      q.fc[kFcVhat + i] = (float)vh[i];
+      q.fc[kFcCenter + i] = (float)q.center[i];
+      q.fc[kFcRef + i] = (float)q.ref[i];
+    }
+  } else if (warp == 4 && lane == 0 && scalars) {
+    // fixed point: worst case |v| <= max(S + 8, 8 c_W/c), so every int64 sum fits for
+    // N * max_bounces hits of |dv| <= 2 |v|max and lever arms <= rmax.
+    const double vmax = fmax(S + 8.0, 8.0 * s_cw);
+    const double bound = (double)q.N * (double)q.max_bounces * 2.0 * 1.7320508075688772 * vmax * fmax(1.0, q.rmax);
+    int shift = (int)floor(62.0 - log2(bound));
+    shift = min(shift, 32);
+    if (shift < 8) s_shift_bad = 1;
+    q.shift = shift;
+    q.quantum = ldexp(1.0, -shift);
+    // squared drag contributions: a particle's |dv . Vhat| <= 2 vmax max_bounces,
+    // so each quantised term stays below 2^62; the sum is a 128-bit integer
+    const double dmax = 2.0 * vmax * (double)q.max_bounces;
+    const int shift2 = max(0, min(32, (int)floor(62.0 - log2(dmax * dmax))));
+    q.shift2 = shift2;
+    q.quantum2 = ldexp(1.0, -shift2);
+    q.fc[kFcScale2] = (float)ldexp(1.0, shift2);
+    q.fc[kFcScale] = (float)ldexp(1.0, shift);
+    q.fc[kFcS] = (float)S;
+    q.fc[kFcCw] = (float)s_cw;
+    q.fc[kFcRcv] = (float)q.r_cv;
+    q.fc[kFcSqrtpi4S] = (float)(kSqrtPiD / (4.0 * S));
+    q.S = S;
+    q.c_mp = s_c;
+    q.cw = s_cw;
+    q.q_inf = 0.5 * q.n * q.m * q.V * q.V;
+  }
+  __syncthreads();
+  const double eS = s_exp[0], erS = s_erf;
+  if (threadIdx.x == 0) {
+    s_D = eS + kSqrtPiD * (1.0 + 2.0 * S * S) * erS / (2.0 * S);
+  } else if (threadIdx.x == 32) {
+    s_K1 = kSqrtPiD / (4.0 * S) * (2.0 * S * S + 1.0) * s_erfc[0] - 0.5 * eS;
+  }
+  __syncthreads();
+
+  if (scalars) {
+    if (threadIdx.x == 0) {
+      q.Dnorm = s_D;
+      q.fc[kFcDinv] = (float)(1.0 / s_D);
+      q.status = s_shift_bad ? TPMC_EINVAL : TPMC_OK;
+    } else if (threadIdx.x == 32) {
+      q.K1 = s_K1;
+      q.fc[kFcK1] = (float)s_K1;
+      // tail-mass cubics of the latitude law at the poles (see latitude_pole):
+      //   x -> +1: h(1) w - h'(1) w^2 / 2 + h''(1) w^3 / 6,  x -> -1: h(-1) w + h'(-1) w^2 / 2 + h''(-1) w^3 / 6,
+      //   h(1) = [e^{-S^2} + sqrt(pi) S erfc(-S)] / D,  h(-1) = e^{-S^2} [1 - sqrt(pi) S erfcx(S)] / D,
+      //   h'(+-1) = sqrt(pi) S erfc(-+S) / D,  h''(+-1) = 2 S^2 e^{-S^2} / D
+      q.fc[kFcPole + 0] = (float)((eS + kSqrtPiD * S * s_erfc[1]) / s_D);
+      q.fc[kFcPole + 1] = (float)(-0.5 * kSqrtPiD * S * s_erfc[1] / s_D);
+      q.fc[kFcPole + 2] = (float)(S * S * eS / (3.0 * s_D));
+    } else if (threadIdx.x == 64) {
+      q.fc[kFcPole + 3] = (float)(eS * (1.0 - kSqrtPiD * S * s_erfcx) / s_D);
+      q.fc[kFcPole + 4] = (float)(0.5 * kSqrtPiD * S * s_erfc[0] / s_D);
+      q.fc[kFcPole + 5] = (float)(S * S * eS / (3.0 * s_D));
+    } else if (threadIdx.x == 96) {
+      if (sphere) {
+        q.gamma = (kSqrtPiD * eS + (CUDART_PI / (2.0 * S) + CUDART_PI * S) * erS) * s_c * q.n * q.r_cv * q.r_cv;
       } else {
-        const double kx = ux / sb, ky = uy / sb;  // unit axis (kx, ky, 0)
-        const double beta = acos(cb);
-        const double cs = cos(beta), sn = sin(beta), oc = 1.0 - cs;
-        Rm[0] = cs + kx * kx * oc; Rm[1] = kx * ky * oc;      Rm[2] = ky * sn;
-        Rm[3] = kx * ky * oc;      Rm[4] = cs + ky * ky * oc; Rm[5] = -kx * sn;
-        Rm[6] = -ky * sn;          Rm[7] = kx * sn;           Rm[8] = cs;
-      }
-      for (int i = 0; i < 9; ++i) { q.R[i] = Rm[i]; q.fc[kFcR + i] = (float)Rm[i]; }
-      const double eS = exp(-S * S), erS = erf(S);
-      q.Dnorm = eS + kSqrtPiD * (1.0 + 2.0 * S * S) * erS / (2.0 * S);
-      q.K1 = kSqrtPiD / (4.0 * S) * (2.0 * S * S + 1.0) * erfc(S) - 0.5 * eS;
-      q.gamma = (kSqrtPiD * eS + (CUDART_PI / (2.0 * S) + CUDART_PI * S) * erS) * c * q.n * q.r_cv * q.r_cv;
-      if (q.cv_kind != TPMC_CV_SPHERE) {
         // Rectangular CV (§I, §III.A): face f receives the flat-plate number
         // flux A_f n c G(s_f), G(s) = (e^{-s^2} + sqrt(pi) s erfc(-s)) / (2 sqrt(pi)),
         // and the particle ids up to floor(N C_{f+1}), C the cumulative share.
         double flux[6], total = 0.0;
         for (int f = 0; f < 6; ++f) {
           const int ax = f / 2, a1 = (ax + 1) % 3, a2 = (ax + 2) % 3;
-          const double s_f = S * (f % 2 == 0 ? -vh[ax] : vh[ax]);
+          const double s_f = S * (f % 2 == 0 ? -s_vh[ax] : s_vh[ax]);
           const double area = (q.box_hi[a1] - q.box_lo[a1]) * (q.box_hi[a2] - q.box_lo[a2]);
-          flux[f] = area * ((exp(-s_f * s_f) + kSqrtPiD * s_f * erfc(-s_f)) / (2.0 * kSqrtPiD));
+          flux[f] = area * ((s_exp[2 + f] + kSqrtPiD * s_f * s_erfc[2 + f]) / (2.0 * kSqrtPiD));
           total += flux[f];
           q.face_s[f] = s_f;
           q.fface_s[f] = (float)s_f;
@@ -1732,74 +1847,66 @@ __global__ void setup_kernel(QueryDev* qs, const QueryDev* base, const double* d
           q.fbox_lo[i] = (float)q.box_lo[i];
           q.fbox_ext[i] = (float)(q.box_hi[i] - q.box_lo[i]);
         }
-        q.gamma = total * c * q.n;
-      }
-      q.q_inf = 0.5 * q.n * q.m * q.V * q.V;
-      // fixed point: worst case |v| <= max(S + 8, 8 c_W/c), so every int64 sum fits for
-      // N * max_bounces hits of |dv| <= 2 |v|max and lever arms <= rmax.
-      const double vmax = fmax(S + 8.0, 8.0 * q.cw);
-      const double bound = (double)q.N * (double)q.max_bounces * 2.0 * 1.7320508075688772 * vmax * fmax(1.0, q.rmax);
-      int shift = (int)floor(62.0 - log2(bound));
-      shift = min(shift, 32);
-      if (shift < 8) st = TPMC_EINVAL;
-      q.shift = shift;
-      q.quantum = ldexp(1.0, -shift);
-      // squared drag contributions: a particle's |dv . Vhat| <= 2 vmax max_bounces,
-      // so each quantised term stays below 2^62; the sum is a 128-bit integer
-      const double dmax = 2.0 * vmax * (double)q.max_bounces;
-      const int shift2 = max(0, min(32, (int)floor(62.0 - log2(dmax * dmax))));
-      q.shift2 = shift2;
-      q.quantum2 = ldexp(1.0, -shift2);
-      q.fc[kFcScale2] = (float)ldexp(1.0, shift2);
-      q.fc[kFcS] = (float)S;
-      q.fc[kFcCw] = (float)q.cw;
-      q.fc[kFcRcv] = (float)q.r_cv;
-      q.fc[kFcSqrtpi4S] = (float)(kSqrtPiD / (4.0 * S));
-      q.fc[kFcK1] = (float)q.K1;
-      q.fc[kFcDinv] = (float)(1.0 / q.Dnorm);
-      // tail-mass cubics of the latitude law at the poles (see latitude_pole):
-      //   x -> +1: h(1) w - h'(1) w^2 / 2 + h''(1) w^3 / 6,  x -> -1: h(-1) w + h'(-1) w^2 / 2 + h''(-1) w^3 / 6,
-      //   h(1) = [e^{-S^2} + sqrt(pi) S erfc(-S)] / D,  h(-1) = e^{-S^2} [1 - sqrt(pi) S erfcx(S)] / D,
-      //   h'(+-1) = sqrt(pi) S erfc(-+S) / D,  h''(+-1) = 2 S^2 e^{-S^2} / D
-      q.fc[kFcPole + 0] = (float)((eS + kSqrtPiD * S * erfc(-S)) / q.Dnorm);
-      q.fc[kFcPole + 1] = (float)(-0.5 * kSqrtPiD * S * erfc(-S) / q.Dnorm);
-      q.fc[kFcPole + 2] = (float)(S * S * eS / (3.0 * q.Dnorm));
-      q.fc[kFcPole + 3] = (float)(eS * (1.0 - kSqrtPiD * S * erfcx(S)) / q.Dnorm);
-      q.fc[kFcPole + 4] = (float)(0.5 * kSqrtPiD * S * erfc(S) / q.Dnorm);
-      q.fc[kFcPole + 5] = (float)(S * S * eS / (3.0 * q.Dnorm));
-      q.fc[kFcScale] = (float)ldexp(1.0, shift);
-      for (int i = 0; i < 3; ++i) {
-        q.fc[kFcVhat + i] = (float)vh[i];
-        q.fc[kFcCenter + i] = (float)q.center[i];
-        q.fc[kFcRef + i] = (float)q.ref[i];
+        q.gamma = total * s_c * q.n;
       }
     }
-    q.status = st;
-    s_ok = st == TPMC_OK;
   }
+  if (!table || !sphere) return;  // the latitude table serves the sphere only
+
+  // ---- latitude start table
+  const float Sf = (float)S, q4 = (float)(kSqrtPiD / (4.0 * S)), K1f = (float)s_K1, Df = (float)(1.0 / s_D);
+  s_H[threadIdx.x] = latitude_cdf<float>(-1.0f + 2.0f * (float)threadIdx.x / (float)(kSetupThreads - 1), Sf, q4, K1f, Df);
   __syncthreads();
-  if (!s_ok || q.cv_kind != TPMC_CV_SPHERE) return;  // the latitude table serves the sphere only
-  const double S = q.S, K1 = q.K1, D = q.Dnorm;
-  for (int j = threadIdx.x; j <= kHTable; j += blockDim.x) {
-    double x;
-    {
-      const double zj = kZLo + (kZHi - kZLo) * j / kHTable;
-      const double u = 0.5 * erfc(-zj * 0.70710678118654752440);  // Phi(z_j)
-      double lo = -1.0, hi = 1.0;
-      x = 2.0 * u - 1.0;
-      for (int it = 0; it < 200; ++it) {
-        const double f = latitude_cdf_d(x, S, K1, D) - u;
-        if (f == 0.0) break;
-        if (f < 0.0) lo = x; else hi = x;
-        double xn = x - f / latitude_pdf_d(x, S, D);
-        if (!(xn > lo && xn < hi)) xn = 0.5 * (lo + hi);
-        const double step = fabs(xn - x);
-        x = xn;
-        if (step < 1e-15) break;
-      }
+  const double K1 = s_K1, q4d = kSqrtPiD / (4.0 * S), Dinv = 1.0 / s_D;
+  // neighbouring knots in one warp: their arguments take the same branches of erfc
+  const int parts = gridDim.y == 1 ? 1 : (int)gridDim.y - 1, part = gridDim.y == 1 ? 0 : (int)blockIdx.y - 1;
+  const int per = (kHTable + parts) / parts;
+  const int j = part * per + (int)threadIdx.x;
+  if ((int)threadIdx.x < per && j <= kHTable) {
+    const double u = knots[j];
+    // the grid cell that brackets u, interpolated, then two steps in float (on
+    // log H in the lower tail); only a start, so float rounding does not matter
+    const float uf = (float)u;
+    int k0 = 0, k1 = kSetupThreads - 1;
+    while (k1 - k0 > 1) {
+      const int mid = (k0 + k1) >> 1;
+      if (s_H[mid] <= uf) k0 = mid; else k1 = mid;
+    }
+    const float x0 = -1.0f + 2.0f * (float)k0 / (float)(kSetupThreads - 1);
+    const float x1 = -1.0f + 2.0f * (float)k1 / (float)(kSetupThreads - 1);
+    const float h0 = s_H[k0], h1 = s_H[k1];
+    const bool tail = uf < 0.0625f && Sf > 1.0f && h0 > 0.0f && h1 > h0;
+    const float w = tail ? logf(uf / h0) / logf(h1 / h0) : (h1 > h0 ? (uf - h0) / (h1 - h0) : 0.5f);
+    float xf = x0 + (x1 - x0) * fminf(fmaxf(w, 0.0f), 1.0f);
+#pragma unroll 1
+    for (int it = 0; it < 2; ++it) {
+      const float H = latitude_cdf<float>(xf, Sf, q4, K1f, Df), h = latitude_pdf<float>(xf, Sf, Df);
+      if (!(H > 0.0f && h > 0.0f)) break;
+      const float xn = xf - (tail ? logf(H / uf) * H / h : (H - uf) / h);
+      if (xn >= x0 && xn <= x1) xf = xn;
+    }
+    double lo = -1.0, hi = 1.0, x = xf;
+#pragma unroll 1
+    for (int it = 0; it < 200; ++it) {
+      const double a = S * x, ec = erfc(-a), e = exp(-a * a);
+      const double f = (q4d * (2.0 * a * a + 1.0) * ec + 0.5 * x * e - K1) * Dinv - u;
+      const double dx = f / ((e + kSqrtPiD * a * ec) * Dinv);
+      // Newton squares the error (times at most S^2 here): below 1e-10 this step is the last
+      if (fabs(dx) < 1e-10) { x -= dx; break; }
+      if (f < 0.0) lo = x; else hi = x;
+      x -= dx;
+      if (!(x > lo && x < hi)) x = 0.5 * (lo + hi);
     }
     q.htab[j] = (float)x;
   }
+}
+
+// The latitude table's uniforms Phi(z_j) (FP64, once per context).
+__global__ void knots_kernel(double* knots) {
+  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  if (j > kHTable) return;
+  const double zj = kZLo + (kZHi - kZLo) * j / kHTable;
+  knots[j] = 0.5 * erfc(-zj * 0.70710678118654752440);  // Phi(z_j)
 }
 
 // Normal-speed start table (FP64, once per context): entry (i, j) is the
@@ -1930,14 +2037,20 @@ __global__ void panels_kernel(const QueryDev* q, const long long* panel, const d
 // ------------------------------------------------------------- launchers
 cudaError_t launch_setup(QueryDev* d_queries, uint32_t nq, const QueryDev* d_base, const double* d_dirs,
                          const double* d_S, ItemDev* d_items, const uint32_t* d_slots, AccStripe* d_acc,
-                         uint32_t acc_stride, cudaStream_t stream) {
+                         uint32_t acc_stride, const float* tables, cudaStream_t stream) {
   if (nq == 0) return cudaSuccess;
-  setup_kernel<<<nq, 160, 0, stream>>>(d_queries, d_base, d_dirs, d_S, d_items, d_slots, d_acc, acc_stride);
+  // Blocks of their own for the table as long as the chip's SMs are not all
+  // busy with other queries (152 SMs; beyond that the split only repeats the
+  // scalars the table needs).
+  const dim3 grid(nq, nq * kSetupParts <= 2 * 152 ? kSetupParts : 1);
+  setup_kernel<<<grid, kSetupThreads, 0, stream>>>(d_queries, d_base, d_dirs, d_S, d_items, d_slots, d_acc, acc_stride,
+                                                   reinterpret_cast<const double*>(tables + kVnNS * kVnNZ + 1));
   return cudaGetLastError();
 }
 
-cudaError_t launch_vn_table(float* d_table, cudaStream_t stream) {
-  vn_table_kernel<<<(kVnNS * kVnNZ + 127) / 128, 128, 0, stream>>>(d_table);
+cudaError_t launch_tables(float* d_tables, cudaStream_t stream) {
+  vn_table_kernel<<<(kVnNS * kVnNZ + 127) / 128, 128, 0, stream>>>(d_tables);
+  knots_kernel<<<(kHTable + 128) / 128, 128, 0, stream>>>(reinterpret_cast<double*>(d_tables + kVnNS * kVnNZ + 1));
   return cudaGetLastError();
 }
 

@@ -100,7 +100,7 @@ extern "C" tpmc_status tpmc_sweep_noalloc(tpmc_ctx* ctx, tpmc_mesh_id mesh, cons
   if (e == cudaSuccess) e = cudaMemsetAsync(&A->counter, 0, sizeof(unsigned long long) + 2 * sizeof(int), s);
   if (e != cudaSuccess) return cuda_fail(e, "tpmc_sweep_noalloc inputs");
   if ((e = launch_setup(A->queries, K, &A->base, h_dirs ? A->dirs : nullptr, h_S ? A->S : nullptr, A->items, nullptr,
-                        A->acc, kNoAllocMaxQueries, s)) != cudaSuccess)
+                        A->acc, kNoAllocMaxQueries, c->vn_table, s)) != cudaSuccess)
     return cuda_fail(e, "setup kernel");
   TraceArgs a{};
   a.mesh = m.dev;

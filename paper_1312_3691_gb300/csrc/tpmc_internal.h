@@ -22,6 +22,7 @@ constexpr double kZLo = -5.5, kZHi = 5.5;
 // (kVnNS rows, s in [-8, 16]) and z_j = kZLo + j kVnStep (kVnNZ columns); 69 KB.
 constexpr double kVnSLo = -8.0, kVnStep = 0.125;
 constexpr int kVnNS = 193, kVnNZ = 89;
+constexpr int kTableFloats = kVnNS * kVnNZ + 1 + 2 * (kHTable + 1);  // both tables of a context (launch_tables)
 // A queued particle keeps its id and query slot in one 64-bit word: ids
 // below 2^40 (N <= 2^34) and at most 2^24 query slots per launch.
 constexpr int kSlotPidBits = 40;
@@ -229,8 +230,10 @@ inline uint32_t node_float4s(uint32_t width) { return width == 8 ? 5u : (width =
 // their accumulator stripes in acc (stripe-major, acc_stride slots per stripe).
 cudaError_t launch_setup(QueryDev* d_queries, uint32_t nq, const QueryDev* d_base, const double* d_dirs,
                          const double* d_S, ItemDev* d_items, const uint32_t* d_slots, AccStripe* d_acc,
-                         uint32_t acc_stride, cudaStream_t stream);
-cudaError_t launch_vn_table(float* d_table, cudaStream_t stream);
+                         uint32_t acc_stride, const float* tables, cudaStream_t stream);
+// Fills a context's tables: the normal-speed start table, then (8-byte
+// aligned) the uniforms Phi(z_j) of the latitude knots as doubles.
+cudaError_t launch_tables(float* d_tables, cudaStream_t stream);
 cudaError_t launch_trace(const TraceArgs& args, uint32_t variant, const LaunchCfg& cfg, int num_sms,
                          cudaStream_t stream);
 cudaError_t launch_finalize(const QueryDev* d_queries, const AccStripe* d_acc, uint32_t acc_stride, uint32_t nq,
