@@ -53,7 +53,7 @@ FLOPS_PER_HIT = 30           # re-emission, momentum difference, torque, quantis
 BYTES_PER_TRI_TEST = 48      # three float4 vertices
 # DRAM bytes per trace launch from an ncu capture, valid only for the kernel
 # source, its build flags and the BVH builder it was taken with (keyed by the
-# SHA-256 of kernels.cu, bvh.cpp and build.py, in that order).
+# SHA-256 of trace.cuh, trace_w2.cu, kernels.cu, bvh.cpp and build.py, in that order).
 # Mean over the four bench groups of dram__bytes_read.sum + dram__bytes_write.sum
 # for one full-size launch (9.6e8 particles).
 TRACE_TRAFFIC = {"5b65220644608b79c040240ed0f05ff920b17b62b72549f59ddb14d9d7524451": 38_543_872}
@@ -61,7 +61,7 @@ TRACE_TRAFFIC = {"5b65220644608b79c040240ed0f05ff920b17b62b72549f59ddb14d9d75244
 
 def kernel_source_hash() -> str:
     h = hashlib.sha256()
-    for name in ("csrc/kernels.cu", "csrc/bvh.cpp", "build.py"):
+    for name in ("csrc/trace.cuh", "csrc/trace_w2.cu", "csrc/kernels.cu", "csrc/bvh.cpp", "build.py"):
         with open(os.path.join(ROOT, "paper_1312_3691_gb300", name), "rb") as f:
             h.update(f.read())
     return h.hexdigest()

@@ -19,15 +19,15 @@ LIB = os.path.join(HERE, "libtpmc.so")
 CUDA_HOME = os.environ.get("CUDA_HOME", "/usr/local/cuda")
 NVCC = os.path.join(CUDA_HOME, "bin", "nvcc")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-CU_SOURCES = ["kernels.cu", "noalloc.cu", "ceilings.cu"]
+CU_SOURCES = ["trace_w2.cu", "trace_w4.cu", "trace_w8.cu", "kernels.cu", "noalloc.cu", "ceilings.cu"]
 CPP_SOURCES = ["api.cpp", "bvh.cpp", "serve.cpp", "tune.cpp"]
-HEADERS = ["tpmc_internal.h", "runtime.h", os.path.join("..", "..", "include", "tpmc.h")]
-# kernels.cu: float division and square root by the hardware approximations
+HEADERS = ["trace.cuh", "tpmc_internal.h", "runtime.h", os.path.join("..", "..", "include", "tpmc.h")]
+# The trace and set-up kernels: float division and square root by the hardware approximations
 # (within two units in the last place) instead of the correctly rounded
 # sequences, which cost 7-10 % of the trace kernel's throughput in the seeding
 # and re-emission arithmetic.  Double precision is unaffected, and so are the
 # explicitly rounded intrinsics the watertight triangle test uses.
-CU_FLAGS = {"kernels.cu": ["-prec-div=false", "-prec-sqrt=false"]}
+CU_FLAGS = {src: ["-prec-div=false", "-prec-sqrt=false"] for src in CU_SOURCES if src.startswith(("trace_w", "kernels"))}
 
 
 def _newest(paths):

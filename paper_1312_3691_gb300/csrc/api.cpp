@@ -30,10 +30,21 @@ tpmc_status cuda_fail(cudaError_t e, const char* where) {
 tpmc_status Ctx::alloc(void** p, size_t bytes, const char* what) {
   *p = nullptr;
   if (bytes == 0) return TPMC_OK;
+  // the pool gives way to everything else (cudaFree waits for the kernels that read it)
+  if (used + bytes > budget && s_pool.ptr) {
+    release(s_pool.ptr);
+    s_pool = Scratch();
+  }
   if (used + bytes > budget)
     return fail(TPMC_ENOMEM, std::string(what) + ": memory budget exceeded (" + std::to_string(used + bytes) +
                                  " > " + std::to_string(budget) + " bytes)");
   cudaError_t e = cudaMalloc(p, bytes);
+  if (e != cudaSuccess && s_pool.ptr) {
+    cudaGetLastError();
+    release(s_pool.ptr);
+    s_pool = Scratch();
+    e = cudaMalloc(p, bytes);
+  }
   if (e != cudaSuccess) {
     cudaGetLastError();
     *p = nullptr;
@@ -157,7 +168,7 @@ tpmc_status fill_query(const MeshRec& m, const tpmc_params* p, uint64_t N, Query
 
 LaunchCfg Ctx::schedule(const MeshRec& m, uint32_t variant, uint64_t total) {
   LaunchCfg cfg;
-  const uint64_t key = tune_key(m.dev.n_tri, variant);
+  const uint64_t key = tune_key(m.dev.n_tri, variant & ~kVariantPool);
   auto it = tuned.find(key);
   if (manual_launch) cfg = manual;
   else if (it != tuned.end()) cfg = it->second;
@@ -174,6 +185,9 @@ LaunchCfg Ctx::schedule(const MeshRec& m, uint32_t variant, uint64_t total) {
     cfg.chunk = 0;
   }
   cfg.smem_nodes = m.dev.width > 2 ? 0u : std::min<uint32_t>(cfg.smem_nodes, m.dev.n_nodes);  // wide: none staged
+  // the kernel's own fixed shared memory comes out of the largest staging
+  const size_t smem = trace_smem_bytes(cfg, m.dev.n_nodes, variant);
+  if (smem <= 227 * 1024 && smem + kTraceStaticSmem > 227 * 1024) cfg.smem_nodes -= kTraceStaticSmem / 32;
   // A traversal round ends once this many lanes have finished their rays.
   // Same-box sweeps with the current kernel: 16 to 28 are equal on the plate
   // and the cylinder; on the satellite 16 is 3 % faster than 24 and 2 % than 20.
@@ -187,6 +201,76 @@ LaunchCfg Ctx::schedule(const MeshRec& m, uint32_t variant, uint64_t total) {
     cfg.chunk = (uint32_t)std::min<uint64_t>(1024, std::max<uint64_t>(32, ch));
   }
   return cfg;
+}
+
+// Entries for `batch` particles (a multiple of 32) and a count for each segment of 32 or more.
+static size_t pool_bytes(uint64_t batch) {
+  return (size_t)batch * kPoolEntryBytes + (size_t)(batch / 32) * sizeof(uint32_t) + 256;
+}
+
+// The pool for launches of `total` particles: twice the entries of a batch and a
+// count for each of its segments.  It takes at most half of the memory the context's
+// budget leaves and halves the batch until that holds; false when less than a
+// small batch fits (the launch then seeds inside the trace kernel).
+bool Ctx::grow_pool(uint64_t total) {
+  const size_t left = budget - std::min(budget, used - s_pool.cap);
+  uint64_t batch = std::min<uint64_t>(kPoolBatch, (total + 31) / 32 * 32);
+  while (batch > kPoolSmallest && 2 * pool_bytes(batch) > left / 2) batch = (batch / 2 + 31) / 32 * 32;
+  const size_t need = 2 * pool_bytes(batch);
+  if (need > left / 2) return false;
+  const std::string last = g_last_error;
+  if (grow(s_pool, need, "seeded particles") == TPMC_OK) return true;
+  g_last_error = last;  // not the caller's failure
+  return false;
+}
+
+// Traces a launch through the pool: batches of half of it, seed_kernel then
+// trace_kernel, in turn on the context's stream and on a second one, which joins
+// it again at the end.  A batch ends in a tail of its longest paths (up to 0.6 ms
+// on the satellite: 64 bounces, one after the other); the other stream's next
+// kernels fill it.  One stream and batches of 2^26, 2^27 particles: the attitude
+// sweep 236 and 226 ms; two streams of 2^26: 217 (of 2^27: 211, for
+// twice the memory).
+cudaError_t Ctx::trace_pool(TraceArgs a, uint32_t variant, const LaunchCfg& cfg) {
+  cudaError_t e = cudaSuccess;
+  if (!side_stream) e = cudaStreamCreateWithFlags(&side_stream, cudaStreamNonBlocking);
+  for (cudaEvent_t* ev : {&fork, &join})
+    if (e == cudaSuccess && !*ev) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
+  if (e != cudaSuccess) return e;
+  const uint64_t total = a.total;
+  uint64_t batch = std::min<uint64_t>(kPoolBatch, (s_pool.cap - 512) / (2 * (32 * kPoolEntryBytes + sizeof(uint32_t))) * 32);
+  // Segments: 512 work indices, fewer where that would not give every warp of
+  // the grid about eight.
+  const uint64_t warps = (uint64_t)num_sms * cfg.blocks_per_sm * (cfg.block / 32);
+  const uint64_t per_warp = std::min(batch, total) / (8 * std::max<uint64_t>(1, warps));
+  a.segment = per_warp >= 512 ? 512u : (per_warp >= 256 ? 256u : (per_warp >= 128 ? 128u : (per_warp >= 64 ? 64u : 32u)));
+  batch = batch / a.segment * a.segment;
+  bool forked = false;
+  uint64_t i = 0;
+  for (a.g0 = 0; a.g0 < total && e == cudaSuccess; a.g0 += batch, ++i) {
+    const bool side = (i & 1) != 0;
+    if (side && !forked) {
+      // the second stream starts where the set-up left the first
+      if ((e = cudaStreamWaitEvent(side_stream, fork, 0)) != cudaSuccess) break;
+      forked = true;
+    }
+    if (i == 0 && total > batch && (e = cudaEventRecord(fork, stream)) != cudaSuccess) break;
+    TraceArgs b = a;
+    b.total = std::min(total, a.g0 + batch);
+    b.n_seg = (uint32_t)((b.total - a.g0 + a.segment - 1) / a.segment);
+    char* half = (char*)s_pool.ptr + (side ? (s_pool.cap / 2) & ~(size_t)255 : 0);
+    b.pool = half;
+    b.seg_count = (uint32_t*)(half + batch * kPoolEntryBytes);
+    b.counter = a.counter + (side ? 1 : 0);
+    const cudaStream_t st = side ? side_stream : stream;
+    if ((e = launch_seed(b, st)) == cudaSuccess) e = launch_trace(b, variant, cfg, num_sms, st);
+  }
+  if (forked) {  // also after an error: what was enqueued ends before anything else on the stream
+    cudaError_t e2 = cudaEventRecord(join, side_stream);
+    if (e2 == cudaSuccess) e2 = cudaStreamWaitEvent(stream, join, 0);
+    if (e == cudaSuccess) e = e2;
+  }
+  return e;
 }
 
 // One batched run: nq queries prepared on the device from `base` (+ dirs/S)
@@ -235,12 +319,15 @@ tpmc_status Ctx::run(const MeshRec& m, const QueryDev* h_queries, uint32_t nq, c
   a.count_work = counters ? 1u : 0u;
   a.vn_table = vn_table;
   if (rec) a.rec = *rec;
+  const bool pooled = !counters && !rec && (variant & 1u) == TPMC_FP32 && total >= kPoolMin && grow_pool(total);
+  if (pooled) variant |= kVariantPool;
   const LaunchCfg cfg = schedule(m, variant, total);
   a.chunk = cfg.chunk;
   a.smem_nodes = cfg.smem_nodes;
   a.refill_at = cfg.refill_at;
   last_cfg = cfg;
-  if (total > 0 && (e = launch_trace(a, variant, cfg, num_sms, stream)) != cudaSuccess) return cuda_fail(e, "trace kernel");
+  if (total > 0 && (e = pooled ? trace_pool(a, variant, cfg) : launch_trace(a, variant, cfg, num_sms, stream)) != cudaSuccess)
+    return cuda_fail(e, "trace kernel");
   if ((e = launch_finalize(d_queries, d_acc, nq, nq, nullptr, d_out, stream)) != cudaSuccess)
     return cuda_fail(e, "finalize kernel");
   if ((e = cudaMemcpyAsync(h_err_word, d_err, sizeof(int), cudaMemcpyDeviceToHost, stream)) != cudaSuccess)
@@ -315,13 +402,12 @@ tpmc_status Ctx::upload_mesh(const double* xyz, uint32_t n_vert, const uint32_t*
   m.dev.width = b.width;
   m.dev.depth = b.depth;
   for (int k = 0; k < 3; ++k) {
-    // the padded root box (empty when there is no mesh): binary trees test it
-    // in their grid's units, wide trees in metres
-    m.dev.box_lo[k] = b.width == 2 ? b.qroot_lo[k] : b.root_lo[k];
-    m.dev.box_hi[k] = b.width == 2 ? b.qroot_hi[k] : b.root_hi[k];
     m.dev.qorigin[k] = b.qorigin[k];
     m.dev.qstep[k] = b.qstep[k];
   }
+  m.dev.n_front = b.n_front;
+  std::memcpy(m.dev.front_reach, b.front_reach, sizeof(b.front_reach));
+  std::memcpy(m.dev.front, b.front, sizeof(b.front));
   m.dev.n_tri = n_tri;
   m.dev.n_tri_leaf = b.n_leaf_tris;
   m.dev.scene_radius = (float)b.radius;
@@ -342,10 +428,13 @@ Ctx::~Ctx() {
   if (serve) stop_serving(this);
   for (auto& kv : panels) release(kv.second.d_panel);
   for (auto& kv : meshes) release(kv.second.d_block);
-  for (Scratch* s : {&s_queries, &s_acc, &s_items, &s_misc, &s_base, &s_out, &s_in})
+  for (Scratch* s : {&s_queries, &s_acc, &s_items, &s_misc, &s_base, &s_out, &s_in, &s_pool})
     release(s->ptr);
   release(vn_table);
   if (h_pinned) cudaFreeHost(h_pinned);
+  if (side_stream) cudaStreamDestroy(side_stream);
+  for (cudaEvent_t ev : {fork, join})
+    if (ev) cudaEventDestroy(ev);
   if (own_stream) cudaStreamDestroy(own_stream);
 }
 

@@ -47,6 +47,16 @@ struct ServeState;  // serve.cpp
 // BVH width of mesh loads that neither tpmc_set_launch nor tpmc_tune decided.
 constexpr uint32_t kDefaultBvhWidth = 2;
 
+// FP32 launches of at least this many particles go through the pool.  Below, the
+// second launch and two tails cost more than the leaner kernels save.  One
+// attitude at S = 7, us through the pool / fused, at 2^22, 2^23 and 2^24
+// particles: plate 261/219, 363/356, 574/640; icosphere 1075/1189, 1966/2283,
+// 3769/4463; cylinder 717/705, 1169/1319, 2119/2493; hemisphere 3475/3769,
+// 6495/7152, 12500/13919; satellite 1001/929, 1316/1381, 1731/1928.
+constexpr uint64_t kPoolMin = 1u << 23;
+// Particles of a batch, at most and at least (32 bytes each, two batches).
+constexpr uint64_t kPoolBatch = 1ull << 26, kPoolSmallest = 1ull << 20;
+
 tpmc_status fill_query(const MeshRec& m, const tpmc_params* p, uint64_t N, QueryDev* q);
 
 inline uint64_t tune_key(uint32_t n_tri, uint32_t variant) {
@@ -61,6 +71,9 @@ struct Ctx {
   int num_sms = 1;
   cudaStream_t own_stream = nullptr;
   cudaStream_t stream = nullptr;
+  // trace_pool: the second stream of a launch, and where it leaves and rejoins the first
+  cudaStream_t side_stream = nullptr;
+  cudaEvent_t fork = nullptr, join = nullptr;
   size_t budget = 0, used = 0;
   uint64_t n_allocs = 0;       // device allocations made since creation
   std::map<void*, size_t> sizes;
@@ -78,6 +91,7 @@ struct Ctx {
   LaunchCfg last_cfg;
   std::map<uint64_t, LaunchCfg> tuned;
   Scratch s_queries, s_acc, s_items, s_misc, s_base, s_out, s_in;
+  Scratch s_pool;              // seeded particles of a batch (grow_pool); released when other allocations need room
   float* vn_table = nullptr;   // start tables (normal speed, latitude knots), built once at creation
   void* h_pinned = nullptr;
   int* h_err_word = nullptr;
@@ -93,6 +107,8 @@ struct Ctx {
   tpmc_status run(const MeshRec& m, const QueryDev* h_queries, uint32_t nq, const QueryDev* h_base,
                   const double* d_dirs, const double* d_S, const ItemDev* h_items, uint32_t n_items,
                   uint64_t total, uint32_t variant, tpmc_result* d_out, const RecordsDev* rec);
+  bool grow_pool(uint64_t total);
+  cudaError_t trace_pool(TraceArgs a, uint32_t variant, const LaunchCfg& cfg);
   tpmc_status check_error_word();
   ~Ctx();
 };

@@ -70,6 +70,10 @@ constexpr int kWideLeafMax = 4;
 constexpr int kMaxStackW = 32;     // wide traversal stack (the builder keeps the depth below)
 constexpr uint32_t kWide4Corner[4] = {0u, 3u, 5u, 6u};
 
+// The front: up to kMaxFront boxes high in the tree that together hold the whole
+// mesh.  A seeded particle that meets none of them misses the mesh.
+constexpr int kMaxFront = 8;
+
 struct MeshDev {
   const float4* nodes = nullptr;    // binary: [n_nodes][4]; wide: [n_nodes][width == 8 ? 5 : 4]
   const float4* tris = nullptr;     // [n_tri_leaf][3]: (v0, id bits), (v1, 0), (v2, 0)
@@ -82,8 +86,13 @@ struct MeshDev {
   uint32_t width = 2;               // 2: binary nodes; 4 or 8: compressed wide nodes
   uint32_t depth = 0;               // levels below the root (bounds the wide traversal's stack)
   float scene_radius = 1.0f;
-  // padded root box (empty: no mesh); binary trees: in grid units 2^23 + q
-  float box_lo[3] = {0.0f, 0.0f, 0.0f}, box_hi[3] = {-1.0f, -1.0f, -1.0f};
+  // front boxes as (centre, half extent) in the units of the tree's slab tests
+  // (binary: grid units 2^23 + q; wide: metres), n_front = 0: no mesh.  A ray
+  // that starts more than front_reach of those units from their zero along an
+  // axis is not tested against them: its rounding could exceed the padding.
+  uint32_t n_front = 0;
+  float front_reach[3] = {0.0f, 0.0f, 0.0f};
+  float front[kMaxFront][6] = {};
   float qorigin[3] = {0.0f, 0.0f, 0.0f}, qstep[3] = {1.0f, 1.0f, 1.0f};  // grid of binary trees' boxes
 };
 
@@ -196,8 +205,15 @@ struct TraceArgs {
   unsigned long long* counter;  // global work counter (zeroed before launch)
   int* error;                 // device error word (stack overflow)
   const float* vn_table;      // [kVnNS][kVnNZ] normal-speed start table
+  // pool path (kVariantPool): the particles of work indices g0 ... total - 1,
+  // seeded beforehand in n_seg segments of `segment` indices
+  void* pool = nullptr;           // Seeded<float>[n_seg][segment]: a segment's particles that may hit, closed up
+  uint32_t* seg_count = nullptr;  // [n_seg] how many
+  uint32_t n_seg = 0, segment = 0;
+  uint64_t g0 = 0;
   RecordsDev rec;
 };
+constexpr size_t kPoolEntryBytes = 32;
 
 struct LaunchCfg {
   uint32_t block = 128;
@@ -219,6 +235,8 @@ struct LaunchCfg {
 constexpr uint32_t kVariantCll = 2u;
 constexpr uint32_t kVariantWide4 = 4u, kVariantWide8 = 8u;
 constexpr uint32_t kVariantCount = 16u;
+// kVariantPool: the particles come from the pool (Ctx::trace_pool); FP32, not with kVariantCount.
+constexpr uint32_t kVariantPool = 32u;
 inline uint32_t trace_variant(const tpmc_params* p, const MeshDev& m) {
   return p->precision | (p->gsi_model == TPMC_GSI_CLL ? kVariantCll : 0u) |
          (m.width == 8 ? kVariantWide8 : (m.width == 4 ? kVariantWide4 : 0u));
@@ -234,6 +252,16 @@ cudaError_t launch_setup(QueryDev* d_queries, uint32_t nq, const QueryDev* d_bas
 // Fills a context's tables: the normal-speed start table, then (8-byte
 // aligned) the uniforms Phi(z_j) of the latitude knots as doubles.
 cudaError_t launch_tables(float* d_tables, cudaStream_t stream);
+using TraceKernel = void (*)(TraceArgs);
+// Kernels by BVH width (trace_w2.cu, trace_w4.cu, trace_w8.cu).
+TraceKernel trace_kernel_w2(uint32_t variant, uint32_t block, uint32_t blocks_per_sm);
+TraceKernel trace_kernel_w4(uint32_t variant, uint32_t block, uint32_t blocks_per_sm);
+TraceKernel trace_kernel_w8(uint32_t variant, uint32_t block, uint32_t blocks_per_sm);
+cudaError_t launch_seed_w2(const TraceArgs& args, cudaStream_t stream);
+cudaError_t launch_seed_w4(const TraceArgs& args, cudaStream_t stream);
+cudaError_t launch_seed_w8(const TraceArgs& args, cudaStream_t stream);
+// Seeds a batch into its pool.
+cudaError_t launch_seed(const TraceArgs& args, cudaStream_t stream);
 cudaError_t launch_trace(const TraceArgs& args, uint32_t variant, const LaunchCfg& cfg, int num_sms,
                          cudaStream_t stream);
 cudaError_t launch_finalize(const QueryDev* d_queries, const AccStripe* d_acc, uint32_t acc_stride, uint32_t nq,
@@ -241,6 +269,7 @@ cudaError_t launch_finalize(const QueryDev* d_queries, const AccStripe* d_acc, u
 cudaError_t launch_panels(const QueryDev* d_query, const long long* d_panel, const float4* frames,
                           const double* frames64, uint32_t n_tri, double* d_pressure, double* d_shear,
                           cudaStream_t stream);
+constexpr uint32_t kTraceStaticSmem = 384;  // the trace kernel's fixed shared memory (front, counts of misses), at most
 size_t trace_smem_bytes(const LaunchCfg& cfg, uint32_t n_nodes, uint32_t variant);
 int trace_max_blocks_per_sm(uint32_t variant, const LaunchCfg& cfg, uint32_t n_nodes);
 
@@ -250,9 +279,10 @@ struct BvhBuild {
   uint32_t width = 2;        // children per node: 2 (binary layout) or 4, 8 (compressed wide layout)
   uint32_t node_bytes = 64;  // bytes per node in `nodes`
   float root_lo[3] = {0.0f, 0.0f, 0.0f}, root_hi[3] = {-1.0f, -1.0f, -1.0f};  // padded root box (empty: no mesh)
-  // binary layout: the boxes' grid, and the root box in grid units 2^23 + q
+  // binary layout: the boxes' grid
   float qorigin[3] = {0.0f, 0.0f, 0.0f}, qstep[3] = {1.0f, 1.0f, 1.0f};
-  float qroot_lo[3] = {0.0f, 0.0f, 0.0f}, qroot_hi[3] = {-1.0f, -1.0f, -1.0f};
+  uint32_t n_front = 0;      // front boxes (see MeshDev)
+  float front_reach[3] = {0.0f, 0.0f, 0.0f}, front[kMaxFront][6] = {};
   uint32_t depth = 0, leaf_max = 0, n_skipped = 0;
   uint32_t n_exposed = 0;    // triangle sides the whole mesh lies behind
   // host copies ready for upload

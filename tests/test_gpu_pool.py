@@ -1,0 +1,125 @@
+"""Particles seeded into the pool against particles seeded inside the trace kernel, and the front boxes, on the GPU.
+
+A counting launch (tpmc_set_counters) always seeds inside the trace kernel, so it is the reference for the pool: the
+sums are integers over the same particles, so they are compared bit for bit.
+"""
+import numpy as np
+import pytest
+
+from tpmc_inputs import meshes as M
+from tpmc_inputs import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+KEYS = ("sum_dv_q", "sum_rdv_q", "n_particles", "n_hits", "n_hit_particles", "n_truncated", "CD_sigma", "status")
+
+
+@pytest.fixture(scope="module")
+def T():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1312_3691_gb300.build import build
+
+    build()
+    from paper_1312_3691_gb300 import tpmc
+
+    return tpmc
+
+
+def _base(T, **kw):
+    return T.make_params(**{**W.base_state(S=6.0), "dir": (0.3, -0.2, 1.0), "eps_diffuse": 0.9, "A_ref": 1.0,
+                            "max_bounces": 64, "seed": 99, **kw})
+
+
+# (items, particles each): just over the pool's smallest launch; several items a batch with ragged ends; over two
+# batches of 2^26 (both streams, and the first pool again); many items inside one segment of 256 work indices
+@pytest.mark.parametrize("K,N", [(1, (1 << 23) + 1), (3, 12_000_017), (7, 25_000_003), (400_000, 97)])
+@pytest.mark.parametrize("width", [2, 4, 8])
+@pytest.mark.parametrize("gsi", ["maxwell", "cll"])
+def test_pool_gives_the_fused_sums(T, K, N, width, gsi):
+    xyz, tri = M.satellite(3_000)
+    kw = dict(gsi_model=T.TPMC_GSI_CLL, alpha_n=0.9, sigma_t=0.8) if gsi == "cll" else {}
+    dirs = np.random.default_rng(1).normal(size=(K, 3))
+    c = T.tpmc_create(0)
+    try:
+        T.tpmc_set_launch(c, block=0, bvh_width=width)
+        mesh = T.tpmc_mesh_load(c, xyz, tri)
+        import torch
+
+        d = torch.from_numpy(dirs).cuda()
+
+        def swept(counting):
+            T.tpmc_set_counters(c, counting)
+            out = torch.zeros(K * T.RESULT_BYTES // 8, dtype=torch.int64, device="cuda")
+            torch.cuda.synchronize()
+            T.tpmc_sweep_device(c, mesh, _base(T, **kw), d, None, K, N, out)
+            torch.cuda.synchronize()
+            rows = out.view(K, -1).cpu()
+            return torch.cat([rows[:, :35], rows[:, 39:]], dim=1)  # all but the work counters, the id and ms
+
+        pooled, fused = swept(False), swept(True)
+        assert T.tpmc_memory_info(c)["used"] > (1 << 23) * 32  # the pool was there
+        assert bool((pooled == fused).all())
+        assert bool((pooled[:, 31] == N).all())  # n_particles: 25 doubles and six sums before it
+    finally:
+        T.tpmc_destroy(c)
+
+
+@pytest.mark.parametrize("budget_mib", [24, 80, 300, 2048])
+def test_pool_yields_to_the_memory_budget(T, budget_mib):
+    """A pool of any size gives the same sums; meshes loaded after it find the room they would have had."""
+    xyz, tri = M.cylinder(0.5, 2.0, 32, 7)
+    N = (1 << 25) + 4097
+    c = T.tpmc_create(0, budget_mib << 20)
+    try:
+        mesh = T.tpmc_mesh_load(c, xyz, tri)
+        r = T.tpmc_trace(c, mesh, _base(T), N)
+        assert T.tpmc_memory_info(c)["used"] <= budget_mib << 20
+        T.tpmc_set_counters(c, True)
+        f = T.tpmc_trace(c, mesh, _base(T), N)
+        assert [r[k] for k in KEYS] == [f[k] for k in KEYS]
+        big = M.satellite(60_000)  # 16 MB on the device
+        extra = [T.tpmc_mesh_load(c, *big) for _ in range(1 if budget_mib < 80 else 3)]
+        T.tpmc_set_counters(c, False)
+        again = T.tpmc_trace(c, mesh, _base(T), N)
+        assert [again[k] for k in KEYS] == [f[k] for k in KEYS]
+        assert len(extra) > 0
+    finally:
+        T.tpmc_destroy(c)
+
+
+@pytest.mark.parametrize("r_cv", [0.75, 40.0, 3000.0])
+@pytest.mark.parametrize("name", ["plate", "cylinder"])
+@pytest.mark.parametrize("width", [2, 8])
+def test_front_rejects_no_particle_that_hits(T, orc, name, r_cv, width):
+    """Control volumes from tight to thousands of bodies wide (beyond the front boxes' reach): the oracle's hits."""
+    xyz, tri = M.plate(1.0) if name == "plate" else M.cylinder(0.3, 0.8, 12, 2)
+    # aim: particles are seeded on the far volume, so the flow is cold and few of them meet the body
+    N = 20_000 if r_cv < 1 else 400_000
+    kw = dict(**W.base_state(S=8.0), dir=(0.02, 0.01, -1.0), eps_diffuse=0.9, A_ref=1.0, r_cv=r_cv, max_bounces=16, seed=3)
+    c = T.tpmc_create(0)
+    try:
+        T.tpmc_set_launch(c, block=0, bvh_width=width)
+        mesh = T.tpmc_mesh_load(c, xyz, tri)
+        r = T.tpmc_trace(c, mesh, T.make_params(**kw), N)
+    finally:
+        T.tpmc_destroy(c)
+    o = orc.trace(orc.Mesh(xyz, tri), orc.make_params(**kw), N)[0]
+    assert r["n_particles"] == N
+    # float positions are off by 6e-8 r_cv: particles that near to a silhouette edge may fall on either side
+    edge = 8.0 * 6e-8 * r_cv / 0.5 * max(1.0, float(o["n_hits"]))
+    assert abs(int(r["n_hits"]) - int(o["n_hits"])) <= 2 + edge, (r["n_hits"], o["n_hits"])
+    if r_cv < 1:
+        assert r["n_hits"] > 1000 and abs(r["CD"] - o["CD"]) <= 1e-4 * abs(o["CD"]) + 3 * o["CD_sigma"]
+
+
+def test_empty_mesh_counts_every_particle(T):
+    c = T.tpmc_create(0)
+    try:
+        mesh = T.tpmc_mesh_load(c, np.zeros((0, 3)), np.zeros((0, 3), np.uint32))
+        for N in (1, 33, (1 << 25) + 5):
+            r = T.tpmc_trace(c, mesh, _base(T, r_cv=1.0), N)
+            assert r["n_particles"] == N and r["n_hits"] == 0 and r["CD"] == 0.0
+    finally:
+        T.tpmc_destroy(c)
