@@ -231,7 +231,13 @@ bool Ctx::grow_pool(uint64_t total) {
 // kernels fill it.  One stream and batches of 2^26, 2^27 particles: the attitude
 // sweep 236 and 226 ms; two streams of 2^26: 217 (of 2^27: 211, for
 // twice the memory).
-cudaError_t Ctx::trace_pool(TraceArgs a, uint32_t variant, const LaunchCfg& cfg) {
+cudaError_t Ctx::trace_pool(TraceArgs a, uint32_t variant, const LaunchCfg& cfg, float cv_area) {
+  // Rough rays first where at most a quarter of the particles is expected to
+  // meet the front (its mean projected area over the control volume's).  They
+  // cost 59 % of an exact seeding: the satellite (12 % pass) 6.74 -> 6.26 ms for
+  // 1e8 particles; the plate sweep (36 %) 33.7 -> 33.6, the cylinder's (55 %) 98.7
+  // -> 101.9, so those seed exactly at once.
+  a.prefilter = a.mesh.front_area < 0.25f * cv_area ? 1u : 0u;
   cudaError_t e = cudaSuccess;
   if (!side_stream) e = cudaStreamCreateWithFlags(&side_stream, cudaStreamNonBlocking);
   for (cudaEvent_t* ev : {&fork, &join})
@@ -319,6 +325,10 @@ tpmc_status Ctx::run(const MeshRec& m, const QueryDev* h_queries, uint32_t nq, c
   a.count_work = counters ? 1u : 0u;
   a.vn_table = vn_table;
   if (rec) a.rec = *rec;
+  // mean projected area of the control volume over pi
+  const QueryDev& bq = h_base ? *h_base : *h_queries;
+  const double bx = bq.box_hi[0] - bq.box_lo[0], by = bq.box_hi[1] - bq.box_lo[1], bz = bq.box_hi[2] - bq.box_lo[2];
+  const float cv_area = (float)(bq.cv_kind == TPMC_CV_SPHERE ? bq.r_cv * bq.r_cv : (bx * by + by * bz + bz * bx) / 6.283185307179586);
   const bool pooled = !counters && !rec && (variant & 1u) == TPMC_FP32 && total >= kPoolMin && grow_pool(total);
   if (pooled) variant |= kVariantPool;
   const LaunchCfg cfg = schedule(m, variant, total);
@@ -326,7 +336,7 @@ tpmc_status Ctx::run(const MeshRec& m, const QueryDev* h_queries, uint32_t nq, c
   a.smem_nodes = cfg.smem_nodes;
   a.refill_at = cfg.refill_at;
   last_cfg = cfg;
-  if (total > 0 && (e = pooled ? trace_pool(a, variant, cfg) : launch_trace(a, variant, cfg, num_sms, stream)) != cudaSuccess)
+  if (total > 0 && (e = pooled ? trace_pool(a, variant, cfg, cv_area) : launch_trace(a, variant, cfg, num_sms, stream)) != cudaSuccess)
     return cuda_fail(e, "trace kernel");
   if ((e = launch_finalize(d_queries, d_acc, nq, nq, nullptr, d_out, stream)) != cudaSuccess)
     return cuda_fail(e, "finalize kernel");
@@ -406,6 +416,7 @@ tpmc_status Ctx::upload_mesh(const double* xyz, uint32_t n_vert, const uint32_t*
     m.dev.qstep[k] = b.qstep[k];
   }
   m.dev.n_front = b.n_front;
+  m.dev.front_area = b.front_area;
   std::memcpy(m.dev.front_reach, b.front_reach, sizeof(b.front_reach));
   std::memcpy(m.dev.front, b.front, sizeof(b.front));
   m.dev.n_tri = n_tri;

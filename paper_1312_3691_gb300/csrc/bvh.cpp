@@ -206,10 +206,9 @@ constexpr double kExposedEps = 1e-12;
 // lanes active.  A convex body keeps its root box alone; the box satellite
 // with its panels and dish takes 6 to 8 boxes, which let 12 % of the particles
 // through instead of 29 % (10 % hit).
-std::vector<Box> choose_front(const std::vector<BNode>& bn) {
+std::vector<Box> choose_front(const std::vector<BNode>& bn, float* area) {
   std::vector<Box> best;
   if (bn.empty()) return best;
-  if (bn[0].left < 0) return {bn[0].box};
   constexpr int kLines = 512;
   constexpr double kBoxCost = 15.0, kPassCost = 1500.0;
   const Box& root = bn[0].box;
@@ -274,6 +273,7 @@ std::vector<Box> choose_front(const std::vector<BNode>& bn) {
     const double cost = kBoxCost * (double)front.size() + kPassCost * pass / kLines;
     if (cost < least) {
       least = cost;
+      *area = (float)(r2 * pass / kLines);  // lines of the disc of radius r
       best.clear();
       for (const Part& f : front) best.push_back(bn[f.node].box);
     }
@@ -872,7 +872,7 @@ bool build_bvh(const double* xyz, uint32_t n_vert, const uint32_t* tri, uint32_t
       out->root_lo[a] = pad_down(bn[0].box.lo[a], scale);
       out->root_hi[a] = pad_up(bn[0].box.hi[a], scale);
     }
-  const std::vector<Box> front = choose_front(bn);
+  const std::vector<Box> front = choose_front(bn, &out->front_area);
   out->width = 2;
   out->node_bytes = 64;
   if (width > 2 && !bn.empty() && layout_wide(bn, leaf_refs, prims, xyz, tri, width, scale, out)) {

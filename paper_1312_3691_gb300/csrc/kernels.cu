@@ -159,6 +159,21 @@ __global__ void __launch_bounds__(kSetupThreads)
     q.fc[kFcScale2] = (float)ldexp(1.0, shift2);
     q.fc[kFcScale] = (float)ldexp(1.0, shift);
     q.fc[kFcS] = (float)S;
+    // Rough rays (may_hit): off by `da` radians on the CV, their velocity by da |v|
+    // + dv + S dc; emulated over the uniforms, da and dc are at most 1.6e-3 for S
+    // below 3.5 and 4.4e-4 above (tests/test_rough_rays.py), dv 2.6e-3.  They pass the body within two CV radii
+    // (or the box's diagonal) of the start.  Half as much again is added.
+    const double vmin = fmax(0.5, 0.5 * S), da = S < 4.0 ? 1.7e-3 : 4.5e-4, dv = 2.6e-3;
+    double margin;
+    if (q.cv_kind == TPMC_CV_SPHERE) {
+      margin = 1.5 * q.r_cv * (da + 2.0 * (da + (dv + S * da) / vmin));
+    } else {
+      double d2 = 0.0;
+      for (int i = 0; i < 3; ++i) d2 += (q.box_hi[i] - q.box_lo[i]) * (q.box_hi[i] - q.box_lo[i]);
+      margin = 1.5 * sqrt(d2) * (1e-5 + dv / vmin);
+    }
+    q.fc[kFcPreMargin] = S <= 15.9 && q.cv_kind != TPMC_CV_BOX_MAXWELL ? (float)margin : 0.0f;
+    q.fc[kFcPreV2] = (float)(vmin * vmin);
     q.fc[kFcCw] = (float)s_cw;
     q.fc[kFcRcv] = (float)q.r_cv;
     q.fc[kFcSqrtpi4S] = (float)(kSqrtPiD / (4.0 * S));

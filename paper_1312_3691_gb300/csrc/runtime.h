@@ -108,7 +108,7 @@ struct Ctx {
                   const double* d_dirs, const double* d_S, const ItemDev* h_items, uint32_t n_items,
                   uint64_t total, uint32_t variant, tpmc_result* d_out, const RecordsDev* rec);
   bool grow_pool(uint64_t total);
-  cudaError_t trace_pool(TraceArgs a, uint32_t variant, const LaunchCfg& cfg);
+  cudaError_t trace_pool(TraceArgs a, uint32_t variant, const LaunchCfg& cfg, float cv_area);
   tpmc_status check_error_word();
   ~Ctx();
 };

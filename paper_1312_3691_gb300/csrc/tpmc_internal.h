@@ -91,6 +91,7 @@ struct MeshDev {
   // that starts more than front_reach of those units from their zero along an
   // axis is not tested against them: its rounding could exceed the padding.
   uint32_t n_front = 0;
+  float front_area = 0.0f;  // their mean projected area over pi, m^2
   float front_reach[3] = {0.0f, 0.0f, 0.0f};
   float front[kMaxFront][6] = {};
   float qorigin[3] = {0.0f, 0.0f, 0.0f}, qstep[3] = {1.0f, 1.0f, 1.0f};  // grid of binary trees' boxes
@@ -105,7 +106,9 @@ enum : int {
   kFcCenter = 16, kFcVhat = 19, kFcRef = 22,          // [3] each
   kFcPole = 25,                                       // [6] latitude tail-mass cubics at x = +1, then -1
   kFcScale2 = 31,                                     // fixed-point scale of the squared drag contributions
-  kFcCount = 32
+  kFcPreMargin = 32, kFcPreV2 = 33,                   // rough rays (may_hit): how far off they pass, m (0: not used), for
+                                                      // speeds squared of at least this
+  kFcCount = 36
 };
 
 // One query: inputs copied from tpmc_params, derived values written by the
@@ -135,7 +138,7 @@ struct QueryDev {
   int32_t status;         // tpmc_status of the set-up
   int32_t pad2;
   // FP32 copies of the query constants (kFc* indices)
-  float fc[kFcCount];
+  alignas(16) float fc[kFcCount];
   float htab[kHTable + 1];
   // box CV (cv_kind != sphere): face f = 2a + k is x_a = hi_a (k = 0) or lo_a
   // (k = 1) and owns particle ids [face_end[f-1], face_end[f]); s_f is its
@@ -210,6 +213,7 @@ struct TraceArgs {
   void* pool = nullptr;           // Seeded<float>[n_seg][segment]: a segment's particles that may hit, closed up
   uint32_t* seg_count = nullptr;  // [n_seg] how many
   uint32_t n_seg = 0, segment = 0;
+  uint32_t prefilter = 0;         // 1: rough rays first (may_hit)
   uint64_t g0 = 0;
   RecordsDev rec;
 };
@@ -282,6 +286,7 @@ struct BvhBuild {
   // binary layout: the boxes' grid
   float qorigin[3] = {0.0f, 0.0f, 0.0f}, qstep[3] = {1.0f, 1.0f, 1.0f};
   uint32_t n_front = 0;      // front boxes (see MeshDev)
+  float front_area = 0.0f;
   float front_reach[3] = {0.0f, 0.0f, 0.0f}, front[kMaxFront][6] = {};
   uint32_t depth = 0, leaf_max = 0, n_skipped = 0;
   uint32_t n_exposed = 0;    // triangle sides the whole mesh lies behind

@@ -55,9 +55,21 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint2 k) {
 }
 
 // (k + 1/2) 2^-23 for the top 23 bits k: exact in float and double.
+// In float from the bits: 1 + k 2^-23 less (1 - 2^-24), an exact difference,
+// spares the conversion its quarter-rate pipe.
 template <typename R>
 __device__ __forceinline__ R uniform(uint32_t w) {
+  if constexpr (sizeof(R) == 4) return __uint_as_float(0x3F800000u | (w >> 9)) - 0.999999940395355224609375f;
   return (R)(w >> 9) * (R)1.1920928955078125e-07 + (R)5.9604644775390625e-08;
+}
+
+// floor(f) for |f| < 2^21, as an integer and as a float: adding 1.5 2^23 rounded
+// down leaves it in the low bits (two additions where two conversions take the
+// quarter-rate pipe twice).
+__device__ __forceinline__ int floor_bits(float f, float& as_float) {
+  const float r = __fadd_rd(f, 12582912.0f);
+  as_float = r - 12582912.0f;
+  return __float_as_int(r) - 0x4B400000;
 }
 
 __device__ __forceinline__ uint4 draws(const QueryDev& q, uint64_t pid, uint32_t block) {
@@ -153,8 +165,9 @@ __device__ __forceinline__ R latitude_pdf(R x, R S, R Dinv) {
 // Interpolated start from a table laid out in z = Phi^-1(u).
 __device__ __forceinline__ float z_table_start(const float* tab, int n, float z, float z_lo, float z_step) {
   const float f = (z - z_lo) / z_step;
-  const int j = min(max((int)floorf(f), 0), n - 2);
-  const float w = fminf(fmaxf(f - (float)j, 0.0f), 1.0f);
+  float fl;
+  const int j = min(max(floor_bits(f, fl), 0), n - 2);
+  const float w = fminf(fmaxf(f - fminf(fmaxf(fl, 0.0f), (float)(n - 2)), 0.0f), 1.0f);
   return (1.0f - w) * __ldg(&tab[j]) + w * __ldg(&tab[j + 1]);
 }
 
@@ -333,11 +346,12 @@ __device__ __forceinline__ float normal_speed_start(const float* tab, float s, f
     const float zs = 1.0f - 1.77245385f * a * erfcxf(a);  // e^{s^2} Z
     return fmaxf(sqrtf(u * fmaxf(zs, 1e-30f)), 1e-30f);
   }
-  const int i = min((int)fs, kVnNS - 2);
-  const float a = fminf(fs - (float)i, 1.0f);
+  float fi, fj;
+  const int i = min(floor_bits(fs, fi), kVnNS - 2);
+  const float a = fminf(fs - fminf(fi, (float)(kVnNS - 2)), 1.0f);
   const float fz = (z - (float)kZLo) / (float)kVnStep;
-  const int j = min(max((int)floorf(fz), 0), kVnNZ - 2);
-  const float b = fminf(fmaxf(fz - (float)j, 0.0f), 1.0f);
+  const int j = min(max(floor_bits(fz, fj), 0), kVnNZ - 2);
+  const float b = fminf(fmaxf(fz - fminf(fmaxf(fj, 0.0f), (float)(kVnNZ - 2)), 0.0f), 1.0f);
   const float* r0 = tab + i * kVnNZ + j;
   const float* r1 = r0 + kVnNZ;
   const float x = (1.0f - a) * ((1.0f - b) * __ldg(r0) + b * __ldg(r0 + 1)) + a * ((1.0f - b) * __ldg(r1) + b * __ldg(r1 + 1));
@@ -474,13 +488,16 @@ __device__ __forceinline__ void seed_box(const QueryDev& q, const QC<R>& c, cons
   }
 }
 
+// One Philox block seeds a particle: u_x, u_theta, u_vn, u_r from the top 23 bits
+// of its words, u_a (Box-Muller angle) from 23 low bits they leave unused.
+__device__ __forceinline__ uint32_t angle_word(const uint4& w0) {
+  return ((w0.x & 0x1FFu) | ((w0.y & 0x1FFu) << 9) | ((w0.z & 0x1Fu) << 18)) << 9;
+}
+
 template <typename R>
 __device__ __forceinline__ void seed_particle(const QueryDev& q, const QC<R>& c, const float* vn_table, uint64_t pid,
-                                              R pos[3], R vel[3]) {
-  // one Philox block: u_x, u_theta, u_vn, u_r from the top 23 bits of its
-  // words, u_a (Box-Muller angle) from 23 low bits they leave unused
-  const uint4 w0 = draws(q, pid, 0);
-  const uint32_t w_a = ((w0.x & 0x1FFu) | ((w0.y & 0x1FFu) << 9) | ((w0.z & 0x1Fu) << 18)) << 9;
+                                              const uint4& w0, R pos[3], R vel[3]) {
+  const uint32_t w_a = angle_word(w0);
   if (q.cv_kind != TPMC_CV_SPHERE) {
     seed_box<R>(q, c, vn_table, pid, w0, w_a, pos, vel);
     return;
@@ -1308,7 +1325,7 @@ __device__ __forceinline__ void add_missed(const TraceArgs& a, int q, uint32_t n
 // misses every triangle: the boxes are padded beyond the rounding (tpmc_internal.h).
 template <int W, typename R>
 __device__ __forceinline__ bool meets_front(const MeshDev& m, const float* __restrict__ front, const R pos[3],
-                                            const R vel[3]) {
+                                            const R vel[3], float margin = 0.0f) {
   float inv[3], oi[3], ainv[3];
   bool far = false;
 #pragma unroll
@@ -1327,17 +1344,87 @@ __device__ __forceinline__ bool meets_front(const MeshDev& m, const float* __res
     far = far || !(fabsf(oi[i]) <= m.front_reach[i] * ainv[i]);
   }
   if (far) return m.n_front > 0;
+  // the boxes wider by `margin` metres
+  float w[3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) w[i] = W == 2 ? margin / m.qstep[i] : margin;
   bool meet = false;
   for (uint32_t k = 0; k < m.n_front; ++k) {
     const float* f = front + 8 * k;
     const float4 c = *reinterpret_cast<const float4*>(f);
     const float2 h = *reinterpret_cast<const float2*>(f + 4);
     const float tx = fmaf(c.x, inv[0], -oi[0]), ty = fmaf(c.y, inv[1], -oi[1]), tz = fmaf(c.z, inv[2], -oi[2]);
-    const float tn = max3(fmaf(-c.w, ainv[0], tx), fmaf(-h.x, ainv[1], ty), fmaf(-h.y, ainv[2], tz));
-    const float tf = min3(fmaf(c.w, ainv[0], tx), fmaf(h.x, ainv[1], ty), fmaf(h.y, ainv[2], tz));
+    const float hx = c.w + w[0], hy = h.x + w[1], hz = h.y + w[2];
+    const float tn = max3(fmaf(-hx, ainv[0], tx), fmaf(-hy, ainv[1], ty), fmaf(-hz, ainv[2], tz));
+    const float tf = min3(fmaf(hx, ainv[0], tx), fmaf(hy, ainv[1], ty), fmaf(hz, ainv[2], tz));
     meet = meet || (tn <= tf && tf >= 0.0f);
   }
   return meet;
+}
+
+// Phi^-1(u) to 4.5e-4 (Hastings' rational approximation; Abramowitz & Stegun
+// 26.2.23), with hardware logarithm and square root.
+__device__ __forceinline__ float rough_quantile(float u) {
+  const float p = fminf(u, 1.0f - u);
+  const float t = sqrtf(-2.0f * __logf(p));
+  const float n = fmaf(fmaf(0.010328f, t, 0.802853f), t, 2.515517f);
+  const float d = fmaf(fmaf(fmaf(0.001308f, t, 0.189269f), t, 1.432788f), t, 1.0f);
+  return copysignf(t - __fdividef(n, d), u - 0.5f);
+}
+
+// Whether the particle may hit, from a rough copy of its ray: the starts of the
+// two inverse-CDF solves without their Newton steps, quantiles to 4.5e-4,
+// hardware sines.  The position is off by at most 1.6e-3 CV radii (in arc), the
+// normal speed by 2e-3, the tangential radius by 6e-4 (units of c_mp), so the ray
+// passes within fc[kFcPreMargin] (set-up) of the true one as long as its speed
+// squared is at least fc[kFcPreV2]; slower ones are kept, as is what the start
+// table does not cover.  440 instructions with the Philox block and the loop
+// around it (156 of them), where the exact seeding takes 745.
+template <int W>
+__device__ __forceinline__ bool may_hit(const QueryDev& q, const TraceArgs& a, const float* front, uint64_t pid,
+                                        const uint4& w0) {
+  const float margin = q.fc[kFcPreMargin];
+  if (!(margin > 0.0f)) return true;
+  const float rad = sqrtf(fmaxf(-__logf(uniform<float>(w0.w)), 0.0f));
+  const float an = (uniform<float>(angle_word(w0)) - 0.5f) * 6.28318531f;  // the angle less pi
+  const float sa = -__sinf(an), ca = -__cosf(an);
+  const float uv = uniform<float>(w0.z), zv = rough_quantile(uv);
+  float pos[3], vel[3], s;
+  if (q.cv_kind == TPMC_CV_SPHERE) {
+    const float ux = uniform<float>(w0.x);
+    const float x = z_table_start(q.htab, kHTable + 1, rough_quantile(ux), (float)kZLo, (float)((kZHi - kZLo) / kHTable));
+    const float cphi = sqrtf(fmaxf((1.0f - x) * (1.0f + x), 0.0f));
+    const float th = (uniform<float>(w0.y) - 0.5f) * 6.28318531f;
+    const float st = -__sinf(th), ct = -__cosf(th);
+    s = q.fc[kFcS] * x;
+    const float vn = normal_speed_start(a.vn_table, s, zv, uv);
+    const float vt1 = q.fc[kFcS] * cphi + rad * ca, vt2 = rad * sa;
+    const float ps[3] = {cphi * ct, cphi * st, -x};
+    const float vr = vt1 * x - vn * cphi;
+    const float vs[3] = {vr * ct + vt2 * st, vr * st - vt2 * ct, vn * x + vt1 * cphi};
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      const float* R = &q.fc[kFcR + 3 * i];
+      pos[i] = q.fc[kFcCenter + i] + q.fc[kFcRcv] * (R[0] * ps[0] + R[1] * ps[1] + R[2] * ps[2]);
+      vel[i] = R[0] * vs[0] + R[1] * vs[1] + R[2] * vs[2];
+    }
+  } else {
+    int f = 0;
+#pragma unroll
+    for (int k = 0; k < 5; ++k) f += pid >= q.face_end[k] ? 1 : 0;
+    const int ax = f >> 1, a1 = ax == 2 ? 0 : ax + 1;
+    s = q.fface_s[f];
+    const float vn = normal_speed_start(a.vn_table, s, zv, uv);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      const float at = i == ax ? ((f & 1) == 0 ? 1.0f : 0.0f) : uniform<float>(i == a1 ? w0.x : w0.y);
+      pos[i] = fmaf(at, q.fbox_ext[i], q.fbox_lo[i]);
+      vel[i] = i == ax ? ((f & 1) == 0 ? -vn : vn) : fmaf(q.fc[kFcS], q.fc[kFcVhat + i], rad * (i == a1 ? ca : sa));
+    }
+  }
+  const float v2 = vel[0] * vel[0] + vel[1] * vel[1] + vel[2] * vel[2];
+  if (!(v2 >= q.fc[kFcPreV2]) || !(s >= -7.9f)) return true;
+  return meets_front<W, float>(a.mesh, front, pos, vel, margin);
 }
 
 // First half of the pool path: a warp seeds one segment of the batch, a.segment
@@ -1351,50 +1438,101 @@ __device__ __forceinline__ bool meets_front(const MeshDev& m, const float* __res
 // stall cycles per issue, now 0.3).  Here every lane seeds, 750 instructions a
 // particle at 85 % of the issue slots: 3.9e10 particles/s, where the fused
 // kernel on an empty mesh reaches 3.2e10.
-template <int W, typename R>
+//
+// PRE: a rough ray (may_hit) decides first, and only the particles that it lets
+// through, gathered in shared memory until they fill a warp, are seeded exactly.
+// The host takes it when it expects that few pass (Ctx::trace_pool): 6.8e10
+// particles/s when none does.
+template <int W, typename R, bool PRE>
 __global__ void __launch_bounds__(128, 8) seed_kernel(const __grid_constant__ TraceArgs a) {
   __shared__ __align__(16) float s_front[kMaxFront * 8];
+  struct Cand {  // a particle that may hit: its Philox block, id and query
+    uint4 w0;
+    uint64_t pq;
+    uint64_t pad;
+  };
+  __shared__ Cand s_cand[PRE ? 4 * 64 : 1];
   for (uint32_t i = threadIdx.x; i < (uint32_t)kMaxFront * 6u; i += blockDim.x)
     s_front[8 * (i / 6) + i % 6] = a.mesh.front[0][i];
   __syncthreads();
   const uint32_t seg = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31u;
+  const uint32_t lt_mask = (1u << lane) - 1u;
   if (seg == 0 && lane == 0) *a.counter = 0;  // the trace kernel's segment counter
   if (seg >= a.n_seg) return;
   const uint64_t first = a.g0 + (uint64_t)seg * a.segment;
-  const uint64_t end = min(first + a.segment, a.total);
+  const uint32_t n_idx = (uint32_t)(min(first + a.segment, a.total) - first);
   Seeded<R>* out = reinterpret_cast<Seeded<R>*>(a.pool) + (size_t)seg * a.segment;
-  uint32_t n_kept = 0, missed = 0;
-  uint64_t it_end = 0, it_off = 0;  // the lane's work item: end of its work range, pid - g
+  Cand* cand = s_cand + (PRE ? (threadIdx.x >> 5) * 64u : 0u);
+  uint32_t n_kept = 0, n_cand = 0, missed = 0;
+  // the lane's work item: where it ends and its particle id 0, both from the segment's first index
+  uint32_t it_end = 0;
+  uint64_t it_pid = 0;
   int it_q = -1;
-  for (uint64_t gb = first; gb < end; gb += 32) {
-    const uint64_t g = gb + lane;
+  // seeds the lane's particle exactly (when it has one) and keeps it if it may hit
+  auto seed = [&](bool active, uint64_t pid, int qi, const uint4& w0) {
     bool keep = false;
     R pos[3], vel[3];
+    if (active) {
+      const QueryDev& q = a.queries[qi];
+      QC<R> c;
+      c.load(q);
+      seed_particle<R>(q, c, a.vn_table, pid, w0, pos, vel);
+      keep = meets_front<W, R>(a.mesh, s_front, pos, vel);
+    }
+    const unsigned kept = __ballot_sync(kFull, keep);
+    if (keep) slot_store<R>(out[n_kept + __popc(kept & lt_mask)], pos, vel, pid | ((uint64_t)qi << kSlotPidBits));
+    n_kept += __popc(kept);
+    return keep;
+  };
+  for (uint32_t i0 = 0; i0 < n_idx || (PRE && n_cand > 0); i0 += 32) {
+    const uint32_t i = i0 + lane;
+    const bool active = i < n_idx;
     uint64_t pid = 0;
-    if (g < end) {
-      if (g >= it_end) {
-        const ItemDev item = a.items[find_item(a.items, a.n_items, g)];
-        it_end = item.g_begin + item.count;
-        it_off = item.pid_begin - item.g_begin;
+    uint4 w0 = make_uint4(0u, 0u, 0u, 0u);
+    if (active) {
+      if (i >= it_end) {
+        const ItemDev item = a.items[find_item(a.items, a.n_items, first + i)];
+        it_end = (uint32_t)min(item.g_begin + item.count - first, (uint64_t)n_idx);
+        it_pid = item.pid_begin - item.g_begin + first;
         if ((int)item.query != it_q) {
           add_missed(a, it_q, missed, acc_stripe());
           missed = 0;
           it_q = (int)item.query;
         }
       }
-      const QueryDev& q = a.queries[it_q];
-      QC<R> c;
-      c.load(q);
-      pid = g + it_off;
-      seed_particle<R>(q, c, a.vn_table, pid, pos, vel);
-      keep = meets_front<W, R>(a.mesh, s_front, pos, vel);
-      missed += keep ? 0u : 1u;
+      pid = it_pid + i;
+      w0 = draws(a.queries[it_q], pid, 0);
     }
-    const unsigned kept = __ballot_sync(kFull, keep);
-    if (keep)
-      slot_store<R>(out[n_kept + __popc(kept & ((1u << lane) - 1u))], pos, vel,
-                    pid | ((uint64_t)it_q << kSlotPidBits));
-    n_kept += __popc(kept);
+    if constexpr (PRE) {
+      const bool may = active && may_hit<W>(a.queries[it_q], a, s_front, pid, w0);
+      const unsigned m = __ballot_sync(kFull, may);
+      if (may) {
+        Cand& e = cand[n_cand + __popc(m & lt_mask)];
+        e.w0 = w0;
+        e.pq = pid | ((uint64_t)it_q << kSlotPidBits);
+      }
+      missed += active && !may ? 1u : 0u;
+      n_cand += __popc(m);
+      __syncwarp();
+      if (n_cand >= 32u || i0 + 32 >= n_idx) {
+        const uint32_t n = min(n_cand, 32u);
+        const Cand e = cand[lane];
+        const int qi = (int)(e.pq >> kSlotPidBits);
+        const bool keep = seed(lane < n, e.pq & ((1ull << kSlotPidBits) - 1), qi, e.w0);
+        // a miss counts for its own query, which need not be the lane's item
+        if (lane < n && !keep) {
+          if (qi == it_q) ++missed;
+          else add_missed(a, qi, 1, acc_stripe());
+        }
+        n_cand -= n;
+        __syncwarp();
+        if (lane < n_cand) cand[lane] = cand[32u + lane];
+        __syncwarp();
+      }
+    } else {
+      const bool keep = seed(active, pid, it_q, w0);
+      missed += active && !keep ? 1u : 0u;
+    }
   }
   // the misses are particles of their queries all the same
   const int q0 = __shfl_sync(kFull, it_q, 0);
@@ -1419,7 +1557,7 @@ __device__ __noinline__ unsigned seed_into(const TraceArgs& a, uint32_t qi, uint
   QC<R> c;
   c.load(q);
   R pos[3], vel[3];
-  seed_particle<R>(q, c, a.vn_table, pid, pos, vel);
+  seed_particle<R>(q, c, a.vn_table, pid, draws(q, pid, 0), pos, vel);
   const bool keep = meets_front<W, R>(a.mesh, front, pos, vel);
   const unsigned kept = __ballot_sync(mask, keep);
   if (keep)
@@ -1805,7 +1943,8 @@ TraceFn pick_trace_w(uint32_t variant, uint32_t block, uint32_t blocks_per_sm) {
 template <int W>
 cudaError_t launch_seed_w(const TraceArgs& a, cudaStream_t stream) {
   const uint32_t grid = (a.n_seg + 3) / 4;
-  seed_kernel<W, float><<<grid, 128, 0, stream>>>(a);
+  if (a.prefilter) seed_kernel<W, float, true><<<grid, 128, 0, stream>>>(a);
+  else seed_kernel<W, float, false><<<grid, 128, 0, stream>>>(a);
   return cudaGetLastError();
 }
 

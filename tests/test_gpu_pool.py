@@ -66,6 +66,34 @@ def test_pool_gives_the_fused_sums(T, K, N, width, gsi):
         T.tpmc_destroy(c)
 
 
+@pytest.mark.parametrize("cv", ["tight", "wide", "box", "maxwell box"])
+@pytest.mark.parametrize("body", ["satellite", "cylinder", "plate"])
+def test_rough_rays_drop_no_particle_that_hits(T, body, cv):
+    """S over its whole range (rough rays are not used above 15.9), 1e6 particles each, in control volumes that make
+    most particles miss (rough rays first) or not: the fused kernel, which seeds every particle exactly, as reference."""
+    xyz, tri = {"satellite": lambda: M.satellite(3_000), "cylinder": lambda: M.cylinder(0.5, 2.0, 24, 5),
+                "plate": lambda: M.plate(1.0)}[body]()
+    S = np.array([0.01, 0.1, 0.35, 0.7, 1.0, 1.5, 2.0, 2.5, 2.8, 3.2, 3.9, 4.0, 5.0, 6.0, 7.0, 8.0, 9.5, 11.0, 13.0,
+                  15.8, 15.9, 16.0, 25.0, 50.0])
+    centre, radius = M.bounding_sphere(xyz)
+    kw = dict(center=tuple(centre), r_cv=radius * (1.02 if cv == "tight" else 3.0))
+    if "box" in cv:
+        kw = dict(cv_kind=T.TPMC_CV_BOX_MAXWELL if "maxwell" in cv else T.TPMC_CV_BOX_FLUX,
+                  box_lo=tuple(xyz.min(axis=0) - 3.0), box_hi=tuple(xyz.max(axis=0) + 4.0))
+    c = T.tpmc_create(0)
+    try:
+        mesh = T.tpmc_mesh_load(c, xyz, tri)
+        dirs = np.random.default_rng(5).normal(size=(len(S), 3))
+        got = []
+        for counting in (False, True):
+            T.tpmc_set_counters(c, counting)
+            got.append(T.tpmc_sweep(c, mesh, _base(T, **kw), dirs, S, 1_000_000))
+        for pooled, fused in zip(*got):
+            assert [pooled[k] for k in KEYS] == [fused[k] for k in KEYS]
+    finally:
+        T.tpmc_destroy(c)
+
+
 @pytest.mark.parametrize("budget_mib", [24, 80, 300, 2048])
 def test_pool_yields_to_the_memory_budget(T, budget_mib):
     """A pool of any size gives the same sums; meshes loaded after it find the room they would have had."""
