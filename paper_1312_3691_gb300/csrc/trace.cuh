@@ -706,6 +706,27 @@ constexpr int kDone = (int)0x80000000;  // no valid leaf code: first + count wou
 template <typename R> struct StackE;
 template <> struct __align__(8) StackE<float> { int node; float t; };
 template <> struct __align__(16) StackE<double> { double t; int node; int pad; };
+// The pool kernel's stack: its first kSharedStack entries in shared memory, a
+// column of the warp's block for each lane (so lanes at different depths use
+// different banks), the rest in local memory.  Most pushes and pops of a lane
+// are within the first four, and they no longer miss the L1 or write lines of
+// the 90 MB that the grid's local stacks span back through the L2: cylinder
+// sweep 97.4 -> 96.4 ms, hemisphere 7.17 -> 7.00, attitude sweep 197.3 -> 195.7
+// (6 and 8 entries take the L1 as much as they save).
+constexpr int kSharedStack = 4;
+struct SplitStack {
+  int2* shared;
+  StackE<float>* local;
+};
+__device__ __forceinline__ void stack_put(SplitStack s, int i, int node, float t) {
+  if (i < kSharedStack) s.shared[i * 32] = make_int2(node, __float_as_int(t));
+  else *reinterpret_cast<int2*>(s.local + i) = make_int2(node, __float_as_int(t));
+}
+__device__ __forceinline__ void stack_get(SplitStack s, int i, int& node, float& t) {
+  const int2 v = i < kSharedStack ? s.shared[i * 32] : *reinterpret_cast<const int2*>(s.local + i);
+  node = v.x;
+  t = __int_as_float(v.y);
+}
 __device__ __forceinline__ void stack_put(StackE<float>* s, int i, int node, float t) {
   *reinterpret_cast<int2*>(s + i) = make_int2(node, __float_as_int(t));
 }
@@ -742,8 +763,8 @@ __device__ __forceinline__ void trav_begin(Trav<R>& t) {
 }
 
 // Next stacked candidate whose entry distance is still below the best hit.
-template <typename R>
-__device__ __forceinline__ int trav_pop(Trav<R>& t, const StackE<R>* stack) {
+template <typename R, typename SP>
+__device__ __forceinline__ int trav_pop(Trav<R>& t, SP stack) {
   while (t.sp > 0) {
     --t.sp;
     int node;
@@ -757,9 +778,9 @@ __device__ __forceinline__ int trav_pop(Trav<R>& t, const StackE<R>* stack) {
 // One inner node: test both children, continue with the nearer hit child,
 // stack the farther one; the first leaf reached is postponed.  STAGE: nodes
 // below n_stage come from the copy in shared memory.
-template <typename R, bool STAGE>
+template <typename R, bool STAGE, typename SP>
 __device__ __forceinline__ void trav_inner(const MeshDev& m, const float4* __restrict__ s_nodes, uint32_t n_stage,
-                                           const Ray<R>& r, Trav<R>& t, StackE<R>* stack, uint32_t& n_nodes,
+                                           const Ray<R>& r, Trav<R>& t, SP stack, uint32_t& n_nodes,
                                            int* err) {
   ++n_nodes;
   float4 n0, n1;
@@ -813,9 +834,9 @@ __device__ __forceinline__ void trav_inner(const MeshDev& m, const float4* __res
 
 // The postponed leaf: test its triangles; then a leaf found meanwhile becomes
 // the postponed one.  Returns true when the ray's traversal is finished.
-template <typename R>
+template <typename R, typename SP>
 __device__ __forceinline__ bool trav_leaf(const MeshDev& m, const Ray<R>& r, uint32_t last, Trav<R>& t,
-                                          const StackE<R>* stack, uint32_t& n_tris) {
+                                          SP stack, uint32_t& n_tris) {
   const uint32_t code = ~(uint32_t)t.leaf;
   const uint32_t first = code & 0xFFFFFFu, count = code >> 24;
   const Shear<R> sh = make_shear<R>(r.d);
@@ -1283,12 +1304,20 @@ static_assert(sizeof(Seeded<float>) == 32, "a float queue slot is two 16-byte ve
 // Float slots are written and read as two 16-byte vectors: eight lanes'
 // 16-byte accesses at a 32-byte stride take two shared-memory wavefronts,
 // where 4-byte fields at that stride would conflict eight ways.
-template <typename R>
+// STREAM: pool entries, written once and read once (they leave the L2 to the mesh).
+template <typename R, bool STREAM = false>
 __device__ __forceinline__ void slot_store(Seeded<R>& e, const R pos[3], const R vel[3], uint64_t pq) {
   if constexpr (sizeof(R) == 4) {
     float4* v = reinterpret_cast<float4*>(&e);
-    v[0] = make_float4(pos[0], pos[1], pos[2], vel[0]);
-    v[1] = make_float4(vel[1], vel[2], __uint_as_float((uint32_t)pq), __uint_as_float((uint32_t)(pq >> 32)));
+    const float4 v0 = make_float4(pos[0], pos[1], pos[2], vel[0]);
+    const float4 v1 = make_float4(vel[1], vel[2], __uint_as_float((uint32_t)pq), __uint_as_float((uint32_t)(pq >> 32)));
+    if constexpr (STREAM) {
+      __stcs(v, v0);
+      __stcs(v + 1, v1);
+    } else {
+      v[0] = v0;
+      v[1] = v1;
+    }
   } else {
 #pragma unroll
     for (int i = 0; i < 3; ++i) { e.pos[i] = pos[i]; e.vel[i] = vel[i]; }
@@ -1296,11 +1325,11 @@ __device__ __forceinline__ void slot_store(Seeded<R>& e, const R pos[3], const R
   }
 }
 
-template <typename R>
+template <typename R, bool STREAM = false>
 __device__ __forceinline__ uint64_t slot_load(const Seeded<R>& e, R pos[3], R vel[3]) {
   if constexpr (sizeof(R) == 4) {
     const float4* v = reinterpret_cast<const float4*>(&e);
-    const float4 a = v[0], b = v[1];
+    const float4 a = STREAM ? __ldcs(v) : v[0], b = STREAM ? __ldcs(v + 1) : v[1];
     pos[0] = a.x; pos[1] = a.y; pos[2] = a.z;
     vel[0] = a.w; vel[1] = b.x; vel[2] = b.y;
     return (uint64_t)__float_as_uint(b.z) | ((uint64_t)__float_as_uint(b.w) << 32);
@@ -1480,7 +1509,7 @@ __global__ void __launch_bounds__(128, 8) seed_kernel(const __grid_constant__ Tr
       keep = meets_front<W, R>(a.mesh, s_front, pos, vel);
     }
     const unsigned kept = __ballot_sync(kFull, keep);
-    if (keep) slot_store<R>(out[n_kept + __popc(kept & lt_mask)], pos, vel, pid | ((uint64_t)qi << kSlotPidBits));
+    if (keep) slot_store<R, true>(out[n_kept + __popc(kept & lt_mask)], pos, vel, pid | ((uint64_t)qi << kSlotPidBits));
     n_kept += __popc(kept);
     return keep;
   };
@@ -1654,7 +1683,14 @@ __global__ void __launch_bounds__(MINB > 0 ? 128 : 256, MINB > 0 ? MINB : (sizeo
   using TV = std::conditional_t<(W > 2), TravW<R>, Trav<R>>;
   using SE = std::conditional_t<(W > 2), uint2, StackE<R>>;
   TV tv{};
-  SE stack[W > 2 ? kMaxStackW : kMaxStack];
+  SE local_stack[W > 2 ? kMaxStackW : kMaxStack];
+  constexpr bool kSplit = POOL && W == 2 && sizeof(R) == 4 && MINB > 0;
+  __shared__ int2 s_stack[kSplit ? 4 * kSharedStack * 32 : 1];
+  std::conditional_t<kSplit, SplitStack, SE*> stack;
+  if constexpr (kSplit)
+    stack = SplitStack{s_stack + (threadIdx.x >> 5) * kSharedStack * 32 + (threadIdx.x & 31u), local_stack};
+  else
+    stack = local_stack;
   uint32_t n_nodes = 0, n_tris = 0;
 
   for (;;) {
@@ -1821,7 +1857,7 @@ __global__ void __launch_bounds__(MINB > 0 ? 128 : 256, MINB > 0 ? MINB : (sizeo
       }
       if (((need >> lane) & 1u) && rank < take) {
         R pos[3], vel[3];
-        const uint64_t pq = slot_load<R>(POOL ? reinterpret_cast<const Seeded<R>*>(a.pool)[q_head + rank]
+        const uint64_t pq = slot_load<R, POOL>(POOL ? reinterpret_cast<const Seeded<R>*>(a.pool)[q_head + rank]
                                               : queue[(q_head + rank) & (kQueue - 1)], pos, vel);
         const uint64_t pid = pq & ((1ull << kSlotPidBits) - 1);
         const int nq = (int)(pq >> kSlotPidBits);
@@ -1887,7 +1923,13 @@ __global__ void __launch_bounds__(MINB > 0 ? 128 : 256, MINB > 0 ? MINB : (sizeo
     for (;;) {
       // without staged nodes, the shared-memory check leaves the node loop
       if (n_stage == 0) {
-        while (__any_sync(kFull, has && !tdone && tv.cur >= 0 && tv.leaf == 0)) {
+        for (;;) {
+          const unsigned searching = __ballot_sync(kFull, has && !tdone && tv.cur >= 0 && tv.leaf == 0);
+          if (searching == 0u) break;
+          // the last few lanes wait while as many others test their leaves: cylinder
+          // sweep 98.3 -> 97.5 ms, hemisphere 7.38 -> 7.17, attitude sweep 204.5 -> 197.4
+          // (6 lanes: 98.9, 7.14, 197.4; 8: 101.0, 7.21, 198.7)
+          if (__popc(searching) < 4 && __popc(__ballot_sync(kFull, has && !tdone && tv.leaf != 0)) >= 4) break;
           if (has && !tdone && tv.cur >= 0)
             trav_inner<R, false>(a.mesh, s_nodes, n_stage, ray, tv, stack, n_nodes, a.error);
         }
