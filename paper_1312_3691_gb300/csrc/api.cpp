@@ -234,7 +234,7 @@ bool Ctx::grow_pool(uint64_t total) {
 cudaError_t Ctx::trace_pool(TraceArgs a, uint32_t variant, const LaunchCfg& cfg, float cv_area) {
   // Rough rays first where at most a quarter of the particles is expected to
   // meet the front (its mean projected area over the control volume's).  They
-  // cost 59 % of an exact seeding: the satellite (12 % pass) 6.74 -> 6.26 ms for
+  // cost 55 % of an exact seeding: the satellite (12 % pass) 6.74 -> 6.09 ms for
   // 1e8 particles; the plate sweep (36 %) 33.7 -> 33.6, the cylinder's (55 %) 98.7
   // -> 101.9, so those seed exactly at once.
   a.prefilter = a.mesh.front_area < 0.25f * cv_area ? 1u : 0u;
@@ -414,6 +414,7 @@ tpmc_status Ctx::upload_mesh(const double* xyz, uint32_t n_vert, const uint32_t*
   for (int k = 0; k < 3; ++k) {
     m.dev.qorigin[k] = b.qorigin[k];
     m.dev.qstep[k] = b.qstep[k];
+    m.dev.qinv[k] = 1.0f / b.qstep[k];
   }
   m.dev.n_front = b.n_front;
   m.dev.front_area = b.front_area;

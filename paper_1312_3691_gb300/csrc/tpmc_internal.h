@@ -95,6 +95,7 @@ struct MeshDev {
   float front_reach[3] = {0.0f, 0.0f, 0.0f};
   float front[kMaxFront][6] = {};
   float qorigin[3] = {0.0f, 0.0f, 0.0f}, qstep[3] = {1.0f, 1.0f, 1.0f};  // grid of binary trees' boxes
+  float qinv[3] = {1.0f, 1.0f, 1.0f};   // 1 / qstep (exact: a power of two)
 };
 
 // ------------------------------------------------------------- query (device)

@@ -1352,7 +1352,8 @@ __device__ __forceinline__ void add_missed(const TraceArgs& a, int q, uint32_t n
 // distances about a box's centre (one FMA for the centre, two for the planes),
 // so that only the final comparisons use the ALU pipe.  A ray rejected here
 // misses every triangle: the boxes are padded beyond the rounding (tpmc_internal.h).
-template <int W, typename R>
+// WIDER: of the boxes widened by `margin` metres.
+template <int W, bool WIDER, typename R>
 __device__ __forceinline__ bool meets_front(const MeshDev& m, const float* __restrict__ front, const R pos[3],
                                             const R vel[3], float margin = 0.0f) {
   float inv[3], oi[3], ainv[3];
@@ -1373,19 +1374,24 @@ __device__ __forceinline__ bool meets_front(const MeshDev& m, const float* __res
     far = far || !(fabsf(oi[i]) <= m.front_reach[i] * ainv[i]);
   }
   if (far) return m.n_front > 0;
-  // the boxes wider by `margin` metres
-  float w[3];
+  [[maybe_unused]] float w[3];  // the margin in distances along the ray
 #pragma unroll
-  for (int i = 0; i < 3; ++i) w[i] = W == 2 ? margin / m.qstep[i] : margin;
+  for (int i = 0; i < 3; ++i) w[i] = W == 2 ? margin * (ainv[i] * m.qinv[i]) : margin * ainv[i];
   bool meet = false;
   for (uint32_t k = 0; k < m.n_front; ++k) {
     const float* f = front + 8 * k;
     const float4 c = *reinterpret_cast<const float4*>(f);
     const float2 h = *reinterpret_cast<const float2*>(f + 4);
     const float tx = fmaf(c.x, inv[0], -oi[0]), ty = fmaf(c.y, inv[1], -oi[1]), tz = fmaf(c.z, inv[2], -oi[2]);
-    const float hx = c.w + w[0], hy = h.x + w[1], hz = h.y + w[2];
-    const float tn = max3(fmaf(-hx, ainv[0], tx), fmaf(-hy, ainv[1], ty), fmaf(-hz, ainv[2], tz));
-    const float tf = min3(fmaf(hx, ainv[0], tx), fmaf(hy, ainv[1], ty), fmaf(hz, ainv[2], tz));
+    float tn, tf;
+    if constexpr (WIDER) {
+      const float hx = fmaf(c.w, ainv[0], w[0]), hy = fmaf(h.x, ainv[1], w[1]), hz = fmaf(h.y, ainv[2], w[2]);
+      tn = max3(tx - hx, ty - hy, tz - hz);
+      tf = min3(tx + hx, ty + hy, tz + hz);
+    } else {
+      tn = max3(fmaf(-c.w, ainv[0], tx), fmaf(-h.x, ainv[1], ty), fmaf(-h.y, ainv[2], tz));
+      tf = min3(fmaf(c.w, ainv[0], tx), fmaf(h.x, ainv[1], ty), fmaf(h.y, ainv[2], tz));
+    }
     meet = meet || (tn <= tf && tf >= 0.0f);
   }
   return meet;
@@ -1401,13 +1407,26 @@ __device__ __forceinline__ float rough_quantile(float u) {
   return copysignf(t - __fdividef(n, d), u - 0.5f);
 }
 
+// Entry of the normal-speed table at (s, z), s in its range: normal_speed_start without the cases beyond it.
+__device__ __forceinline__ float rough_normal_speed(const float* tab, float s, float z) {
+  float fi, fj;
+  const float fs = fmaf(s, (float)(1.0 / kVnStep), (float)(-kVnSLo / kVnStep));
+  const float fz = fmaf(z, (float)(1.0 / kVnStep), (float)(-kZLo / kVnStep));
+  const int i = min(max(floor_bits(fs, fi), 0), kVnNS - 2), j = min(max(floor_bits(fz, fj), 0), kVnNZ - 2);
+  const float a = fs - fi, b = fz - fj;
+  const float* r = tab + i * kVnNZ + j;
+  const float lo = fmaf(b, __ldg(r + 1) - __ldg(r), __ldg(r));
+  const float hi = fmaf(b, __ldg(r + kVnNZ + 1) - __ldg(r + kVnNZ), __ldg(r + kVnNZ));
+  return fmaf(a, hi - lo, lo);
+}
+
 // Whether the particle may hit, from a rough copy of its ray: the starts of the
 // two inverse-CDF solves without their Newton steps, quantiles to 4.5e-4,
 // hardware sines.  The position is off by at most 1.6e-3 CV radii (in arc), the
 // normal speed by 2e-3, the tangential radius by 6e-4 (units of c_mp), so the ray
 // passes within fc[kFcPreMargin] (set-up) of the true one as long as its speed
 // squared is at least fc[kFcPreV2]; slower ones are kept, as is what the start
-// table does not cover.  440 instructions with the Philox block and the loop
+// table does not cover.  About 410 instructions with the Philox block and the loop
 // around it (156 of them), where the exact seeding takes 745.
 template <int W>
 __device__ __forceinline__ bool may_hit(const QueryDev& q, const TraceArgs& a, const float* front, uint64_t pid,
@@ -1417,16 +1436,19 @@ __device__ __forceinline__ bool may_hit(const QueryDev& q, const TraceArgs& a, c
   const float rad = sqrtf(fmaxf(-__logf(uniform<float>(w0.w)), 0.0f));
   const float an = (uniform<float>(angle_word(w0)) - 0.5f) * 6.28318531f;  // the angle less pi
   const float sa = -__sinf(an), ca = -__cosf(an);
-  const float uv = uniform<float>(w0.z), zv = rough_quantile(uv);
+  const float zv = rough_quantile(uniform<float>(w0.z));
   float pos[3], vel[3], s;
   if (q.cv_kind == TPMC_CV_SPHERE) {
     const float ux = uniform<float>(w0.x);
-    const float x = z_table_start(q.htab, kHTable + 1, rough_quantile(ux), (float)kZLo, (float)((kZHi - kZLo) / kHTable));
+    const float f = fmaf(rough_quantile(ux), (float)(kHTable / (kZHi - kZLo)), (float)(-kZLo * kHTable / (kZHi - kZLo)));
+    float fl;
+    const int j = min(max(floor_bits(f, fl), 0), kHTable - 1);
+    const float x0 = __ldg(&q.htab[j]), x = fmaf(f - fl, __ldg(&q.htab[j + 1]) - x0, x0);
     const float cphi = sqrtf(fmaxf((1.0f - x) * (1.0f + x), 0.0f));
     const float th = (uniform<float>(w0.y) - 0.5f) * 6.28318531f;
     const float st = -__sinf(th), ct = -__cosf(th);
     s = q.fc[kFcS] * x;
-    const float vn = normal_speed_start(a.vn_table, s, zv, uv);
+    const float vn = rough_normal_speed(a.vn_table, s, zv);
     const float vt1 = q.fc[kFcS] * cphi + rad * ca, vt2 = rad * sa;
     const float ps[3] = {cphi * ct, cphi * st, -x};
     const float vr = vt1 * x - vn * cphi;
@@ -1443,7 +1465,7 @@ __device__ __forceinline__ bool may_hit(const QueryDev& q, const TraceArgs& a, c
     for (int k = 0; k < 5; ++k) f += pid >= q.face_end[k] ? 1 : 0;
     const int ax = f >> 1, a1 = ax == 2 ? 0 : ax + 1;
     s = q.fface_s[f];
-    const float vn = normal_speed_start(a.vn_table, s, zv, uv);
+    const float vn = rough_normal_speed(a.vn_table, s, zv);
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
       const float at = i == ax ? ((f & 1) == 0 ? 1.0f : 0.0f) : uniform<float>(i == a1 ? w0.x : w0.y);
@@ -1453,7 +1475,7 @@ __device__ __forceinline__ bool may_hit(const QueryDev& q, const TraceArgs& a, c
   }
   const float v2 = vel[0] * vel[0] + vel[1] * vel[1] + vel[2] * vel[2];
   if (!(v2 >= q.fc[kFcPreV2]) || !(s >= -7.9f)) return true;
-  return meets_front<W, float>(a.mesh, front, pos, vel, margin);
+  return meets_front<W, true, float>(a.mesh, front, pos, vel, margin);
 }
 
 // First half of the pool path: a warp seeds one segment of the batch, a.segment
@@ -1470,7 +1492,7 @@ __device__ __forceinline__ bool may_hit(const QueryDev& q, const TraceArgs& a, c
 //
 // PRE: a rough ray (may_hit) decides first, and only the particles that it lets
 // through, gathered in shared memory until they fill a warp, are seeded exactly.
-// The host takes it when it expects that few pass (Ctx::trace_pool): 6.8e10
+// The host takes it when it expects that few pass (Ctx::trace_pool): 7.3e10
 // particles/s when none does.
 template <int W, typename R, bool PRE>
 __global__ void __launch_bounds__(128, 8) seed_kernel(const __grid_constant__ TraceArgs a) {
@@ -1506,7 +1528,7 @@ __global__ void __launch_bounds__(128, 8) seed_kernel(const __grid_constant__ Tr
       QC<R> c;
       c.load(q);
       seed_particle<R>(q, c, a.vn_table, pid, w0, pos, vel);
-      keep = meets_front<W, R>(a.mesh, s_front, pos, vel);
+      keep = meets_front<W, false, R>(a.mesh, s_front, pos, vel);
     }
     const unsigned kept = __ballot_sync(kFull, keep);
     if (keep) slot_store<R, true>(out[n_kept + __popc(kept & lt_mask)], pos, vel, pid | ((uint64_t)qi << kSlotPidBits));
@@ -1587,7 +1609,7 @@ __device__ __noinline__ unsigned seed_into(const TraceArgs& a, uint32_t qi, uint
   c.load(q);
   R pos[3], vel[3];
   seed_particle<R>(q, c, a.vn_table, pid, draws(q, pid, 0), pos, vel);
-  const bool keep = meets_front<W, R>(a.mesh, front, pos, vel);
+  const bool keep = meets_front<W, false, R>(a.mesh, front, pos, vel);
   const unsigned kept = __ballot_sync(mask, keep);
   if (keep)
     slot_store<R>(queue[(at + __popc(kept & ((1u << (threadIdx.x & 31u)) - 1u))) & (kQueue - 1)], pos, vel,
