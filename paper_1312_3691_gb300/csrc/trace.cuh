@@ -220,8 +220,12 @@ __device__ R latitude_inverse(R u, const QueryDev& q, const QC<R>& c, R* cphi) {
     const R lu = logmode ? Fn<R>::log(u) : (R)0;
 #pragma unroll 1
     for (int it = 0; it < Fn<R>::kIter; ++it) {
-      const R H = latitude_cdf<R>(x, c.S, c.sqrtpi_4S, c.K1, c.Dinv);
-      const R h = latitude_pdf<R>(x, c.S, c.Dinv);
+      // the law and its density from one erfc and one exp: each is a chain of
+      // branches in double, which the compiler does not merge by itself
+      const R Sx = c.S * x;
+      const R ec = Fn<R>::erfc(-Sx), ex = Fn<R>::exp(-Sx * Sx);
+      const R H = (c.sqrtpi_4S * ((R)2 * Sx * Sx + (R)1) * ec + (R)0.5 * x * ex - c.K1) * c.Dinv;
+      const R h = (ex + (R)kSqrtPiD * Sx * ec) * c.Dinv;
       R f, dx;
       if (logmode) {
         if (!(H > (R)0)) { lo = x; x = (R)0.5 * (lo + hi); continue; }
@@ -272,43 +276,31 @@ __device__ R normal_speed_inverse_adaptive(R u, R s, R x_start) {
   for (int it = 0; it < Fn<R>::kIter; ++it) {
     const R y = x - s;
     R T, p;
+    // x near 0 below the median: F by 4-point Gauss-Legendre of p on [0, x]
+    const bool quad = !upper && x < xq;
+    R e, q1 = (R)0;
     if (s >= (R)0) {
-      const R e = Fn<R>::exp(-y * y);
+      // erfc(y) above the median, erfc(-y) below: one evaluation for both
+      e = Fn<R>::exp(-y * y);
+      const R ec = Fn<R>::erfc(upper ? y : s - x);
       p = (R)2 * x * e / Z;
-      if (upper) {
-        T = (e + sp * Fn<R>::erfc(y)) / Z;
-      } else if (x < xq) {
-        const R gx[4] = {(R)0.06943184420297371, (R)0.33000947820757187, (R)0.6699905217924281, (R)0.9305681557970262};
-        const R gw[4] = {(R)0.17392742256872692, (R)0.3260725774312731, (R)0.3260725774312731, (R)0.17392742256872692};
-        R acc = 0;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const R t = x * gx[k];
-          acc += gw[k] * (R)2 * t * Fn<R>::exp(-(t - s) * (t - s));
-        }
-        T = x * acc / Z;
-      } else {
-        const R w = s - x;
-        T = ((sp * Fn<R>::erfc(w) - Fn<R>::exp(-w * w)) - g_s) / Z;
-      }
+      T = upper ? (e + sp * ec) / Z : ((sp * ec - e) - g_s) / Z;
     } else {
-      const R e = Fn<R>::exp(-x * (x - (R)2 * s));
+      e = Fn<R>::exp(-x * (x - (R)2 * s));
       p = (R)2 * x * e / Zs;
-      if (upper) {
-        T = e * ((R)1 + sp * Fn<R>::erfcx(y)) / Zs;
-      } else if (x < xq) {
-        const R gx[4] = {(R)0.06943184420297371, (R)0.33000947820757187, (R)0.6699905217924281, (R)0.9305681557970262};
-        const R gw[4] = {(R)0.17392742256872692, (R)0.3260725774312731, (R)0.3260725774312731, (R)0.17392742256872692};
-        R acc = 0;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const R t = x * gx[k];
-          acc += gw[k] * (R)2 * t * Fn<R>::exp(-t * (t - (R)2 * s));
-        }
-        T = x * acc / Zs;
-      } else {
-        T = (Zs - e * ((R)1 + sp * Fn<R>::erfcx(y))) / Zs;
+      q1 = e * ((R)1 + sp * Fn<R>::erfcx(y));
+      T = upper ? q1 / Zs : (Zs - q1) / Zs;
+    }
+    if (quad) {
+      const R gx[4] = {(R)0.06943184420297371, (R)0.33000947820757187, (R)0.6699905217924281, (R)0.9305681557970262};
+      const R gw[4] = {(R)0.17392742256872692, (R)0.3260725774312731, (R)0.3260725774312731, (R)0.17392742256872692};
+      R acc = 0;
+#pragma unroll 1
+      for (int k = 0; k < 4; ++k) {
+        const R t = x * gx[k];
+        acc += gw[k] * (R)2 * t * Fn<R>::exp(s >= (R)0 ? -(t - s) * (t - s) : -t * (t - (R)2 * s));
       }
+      T = x * acc / (s >= (R)0 ? Z : Zs);
     }
     if (!(T > (R)0)) {
       // underflow or cancellation: x lies deep in the solved tail
