@@ -423,6 +423,7 @@ tpmc_status Ctx::upload_mesh(const double* xyz, uint32_t n_vert, const uint32_t*
   m.dev.n_tri = n_tri;
   m.dev.n_tri_leaf = b.n_leaf_tris;
   m.dev.scene_radius = (float)b.radius;
+  for (int i = 0; i < 3; ++i) m.dev.centre[i] = (float)b.center[i];
   for (int i = 0; i < 3; ++i) m.center[i] = b.center[i];
   m.radius = b.radius;
   m.depth = b.depth;

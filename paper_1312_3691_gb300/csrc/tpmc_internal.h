@@ -85,7 +85,7 @@ struct MeshDev {
   uint32_t n_tri_leaf = 0;          // triangles referenced by leaves (zero-area ones dropped)
   uint32_t width = 2;               // 2: binary nodes; 4 or 8: compressed wide nodes
   uint32_t depth = 0;               // levels below the root (bounds the wide traversal's stack)
-  float scene_radius = 1.0f;
+  float scene_radius = 1.0f, centre[3] = {0.0f, 0.0f, 0.0f};  // a sphere that holds the mesh
   // front boxes as (centre, half extent) in the units of the tree's slab tests
   // (binary: grid units 2^23 + q; wide: metres), n_front = 0: no mesh.  A ray
   // that starts more than front_reach of those units from their zero along an
