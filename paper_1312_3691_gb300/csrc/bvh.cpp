@@ -561,7 +561,11 @@ bool build_bvh(const double* xyz, uint32_t n_vert, const uint32_t* tri, uint32_t
   Box all;
   for (uint64_t i = 0; i < (uint64_t)n_tri * 3; ++i) all.grow(xyz + 3 * (uint64_t)tri[i]);
   if (!all.empty()) {
-    for (int a = 0; a < 3; ++a) out->center[a] = 0.5 * (all.lo[a] + all.hi[a]);
+    for (int a = 0; a < 3; ++a) {
+      out->center[a] = 0.5 * (all.lo[a] + all.hi[a]);
+      out->lo[a] = all.lo[a];
+      out->hi[a] = all.hi[a];
+    }
     double r2 = 0;
     for (uint64_t i = 0; i < (uint64_t)n_tri * 3; ++i) {
       const double* p = xyz + 3 * (uint64_t)tri[i];

@@ -23,7 +23,7 @@ struct MeshRec {
   MeshDev dev;
   void* d_block = nullptr;     // one device allocation holding every mesh array
   size_t bytes = 0;
-  double center[3] = {0, 0, 0}, radius = 0;
+  double center[3] = {0, 0, 0}, radius = 0, lo[3] = {0, 0, 0}, hi[3] = {0, 0, 0};
   uint32_t depth = 0, leaf_max = 0, n_skipped = 0, n_vert = 0, n_exposed = 0, node_bytes = 64;
   std::vector<double> h_xyz;   // host copy for the control-volume containment check
   std::vector<uint32_t> h_tri;
@@ -90,6 +90,7 @@ struct Ctx {
   LaunchCfg manual;
   LaunchCfg last_cfg;
   std::map<uint64_t, LaunchCfg> tuned;
+  std::map<uint64_t, int> max_blocks;  // trace_max_blocks_per_sm by variant, block and shared memory
   Scratch s_queries, s_acc, s_items, s_misc, s_base, s_out, s_in;
   Scratch s_pool;              // seeded particles of a batch (grow_pool); released when other allocations need room
   float* vn_table = nullptr;   // start tables (normal speed, latitude knots), built once at creation

@@ -299,6 +299,7 @@ struct BvhBuild {
   double* frames64 = nullptr;// [n_tri * 8]: n, area, t1, exposed-side bits (as a double in word 7)
   uint32_t n_leaf_tris = 0;
   double center[3] = {0, 0, 0}, radius = 0;
+  double lo[3] = {0, 0, 0}, hi[3] = {0, 0, 0};  // of the referenced vertices
   void release();
 };
 

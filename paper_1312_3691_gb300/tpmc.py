@@ -10,6 +10,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import struct
 
 import numpy as np
 
@@ -51,11 +52,24 @@ class tpmc_result(ctypes.Structure):
     ]
 
     def as_dict(self) -> dict:
-        out = {}
-        for name, _ in self._fields_:
-            v = getattr(self, name)
-            out[name] = list(v) if isinstance(v, ctypes.Array) else v
-        return out
+        return _result_dicts(self)[0]
+
+
+# one unpacking for a whole record (a getattr for each field takes 6 us a record)
+_RESULT = struct.Struct("=25d6q7Qdii")
+_RESULT_AT = []  # (name, first value, end or None for a single one)
+for _name, _type in tpmc_result._fields_:
+    _at = _RESULT_AT[-1][3] if _RESULT_AT else 0
+    _n = getattr(_type, "_length_", 0)
+    _RESULT_AT.append((_name, _at, _at + _n if _n else None, _at + max(_n, 1)))
+_RESULT_AT = [(name, at, end) for name, at, end, _ in _RESULT_AT]
+assert _RESULT.size == ctypes.sizeof(tpmc_result)
+
+
+def _result_dicts(results) -> list:
+    """Each record of a buffer of results as a dict."""
+    return [{name: v[at] if end is None else list(v[at:end]) for name, at, end in _RESULT_AT}
+            for v in _RESULT.iter_unpack(results)]
 
 
 class tpmc_records(ctypes.Structure):
@@ -281,7 +295,7 @@ def tpmc_sweep(ctx, mesh: int, base: tpmc_params, dirs, S, N_each: int):
     out = (tpmc_result * K)()
     _check(lib().tpmc_sweep(ctx, int(mesh), ctypes.byref(base), _pd(D), _pd(Sv), K, int(N_each), out),
            "tpmc_sweep", ctx)
-    return [o.as_dict() for o in out]
+    return _result_dicts(out)
 
 
 def tpmc_sweep_device(ctx, mesh: int, base: tpmc_params, d_dirs, d_S, K: int, N_each: int, d_out):
@@ -297,15 +311,14 @@ def tpmc_sweep_noalloc(ctx, mesh: int, base: tpmc_params, dirs, S, N_each: int):
     out = (tpmc_result * K)()
     _check(lib().tpmc_sweep_noalloc(ctx, int(mesh), ctypes.byref(base), _pd(D), _pd(Sv), K, int(N_each), out),
            "tpmc_sweep_noalloc", ctx)
-    return [o.as_dict() for o in out]
+    return _result_dicts(out)
 
 
 RESULT_BYTES = ctypes.sizeof(tpmc_result)
 
 
 def results_from_bytes(buf: bytes, K: int):
-    arr = (tpmc_result * K).from_buffer_copy(buf)
-    return [a.as_dict() for a in arr]
+    return _result_dicts((tpmc_result * K).from_buffer_copy(buf))
 
 
 def tpmc_submit(ctx, mesh: int, params: tpmc_params, N: int) -> int:

@@ -67,3 +67,29 @@ def test_rejected_items_report_their_status(T):
         assert r[0]["sum_dv_q"] == ok[0]["sum_dv_q"] and r[3]["sum_dv_q"] == ok[3]["sum_dv_q"]
     finally:
         T.tpmc_destroy(c)
+
+
+@pytest.mark.parametrize("offset", [0.0, 0.3])
+def test_containment_at_its_limit(T, offset):
+    """A control volume is accepted exactly when its radius exceeds the farthest vertex's distance."""
+    xyz, tri = M.cylinder(0.4, 1.3, 9, 2)
+    centre = np.array([offset, -offset, 0.1])
+    far = np.sqrt(((xyz[np.unique(tri)] - centre) ** 2).sum(axis=1)).max()
+    kw = dict(**W.base_state(S=7.0), dir=(0, 0, 1), eps_diffuse=1.0, A_ref=1.0, max_bounces=8, seed=5, center=tuple(centre))
+    lo, hi = xyz.min(axis=0), xyz.max(axis=0)
+    box = {k: v for k, v in kw.items() if k != "center"}
+    c = T.tpmc_create(0)
+    try:
+        mesh = T.tpmc_mesh_load(c, xyz, tri)
+        for grow, ok in ((-1e-6, False), (-1e-12, False), (1e-12, True), (1e-6, True), (1.0, True)):
+            params = [T.make_params(**kw, r_cv=far * (1 + grow)),
+                      T.make_params(**box, cv_kind=T.TPMC_CV_BOX_FLUX, box_lo=tuple(lo - max(grow, 0)), box_hi=tuple(hi + grow))]
+            for p in params:
+                if ok:
+                    assert T.tpmc_trace(c, mesh, p, 100)["n_particles"] == 100
+                else:
+                    with pytest.raises(T.TpmcError) as e:
+                        T.tpmc_trace(c, mesh, p, 100)
+                    assert e.value.status == T.TPMC_EINVAL
+    finally:
+        T.tpmc_destroy(c)
