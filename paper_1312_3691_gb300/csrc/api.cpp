@@ -30,19 +30,13 @@ tpmc_status cuda_fail(cudaError_t e, const char* where) {
 tpmc_status Ctx::alloc(void** p, size_t bytes, const char* what) {
   *p = nullptr;
   if (bytes == 0) return TPMC_OK;
-  // the pool gives way to everything else (cudaFree waits for the kernels that read it)
-  if (used + bytes > budget && s_pool.ptr) {
-    release(s_pool.ptr);
-    s_pool = Scratch();
-  }
+  if (used + bytes > budget) release_pools();
   if (used + bytes > budget)
     return fail(TPMC_ENOMEM, std::string(what) + ": memory budget exceeded (" + std::to_string(used + bytes) +
                                  " > " + std::to_string(budget) + " bytes)");
   cudaError_t e = cudaMalloc(p, bytes);
-  if (e != cudaSuccess && s_pool.ptr) {
+  if (e != cudaSuccess && release_pools()) {
     cudaGetLastError();
-    release(s_pool.ptr);
-    s_pool = Scratch();
     e = cudaMalloc(p, bytes);
   }
   if (e != cudaSuccess) {
@@ -214,20 +208,59 @@ static size_t pool_bytes(uint64_t batch) {
   return (size_t)batch * kPoolEntryBytes + (size_t)(batch / 32) * sizeof(uint32_t) + 256;
 }
 
-// The pool for launches of `total` particles: twice the entries of a batch and a
-// count for each of its segments.  It takes at most half of the memory the context's
-// budget leaves and halves the batch until that holds; false when less than a
-// small batch fits (the launch then seeds inside the trace kernel).
-bool Ctx::grow_pool(uint64_t total) {
-  const size_t left = budget - std::min(budget, used - s_pool.cap);
-  uint64_t batch = std::min<uint64_t>(kPoolBatch, (total + 31) / 32 * 32);
+// Mean projected area over pi, m^2, of a query's control volume.
+float cv_area(const QueryDev& q) {
+  if (q.cv_kind == TPMC_CV_SPHERE) return (float)(q.r_cv * q.r_cv);
+  const double x = q.box_hi[0] - q.box_lo[0], y = q.box_hi[1] - q.box_lo[1], z = q.box_hi[2] - q.box_lo[2];
+  return (float)((x * y + y * z + z * x) / 6.283185307179586);
+}
+
+// A pool for launches of `total` particles: twice the entries of a batch (at most
+// max_batch) and a count for each of its segments.  It takes at most half of the
+// memory the context's budget leaves and halves the batch until that holds; false
+// when less than a small batch fits (the launch then seeds inside the trace kernel).
+bool Ctx::grow_pool(Pool& pool, uint64_t total, uint64_t max_batch) {
+  const size_t left = budget - std::min(budget, used - pool.cap);
+  uint64_t batch = std::min<uint64_t>(max_batch, (total + 31) / 32 * 32);
   while (batch > kPoolSmallest && 2 * pool_bytes(batch) > left / 2) batch = (batch / 2 + 31) / 32 * 32;
   const size_t need = 2 * pool_bytes(batch);
   if (need > left / 2) return false;
+  if (pool.cap >= need) return true;
+  release_pool(pool);
   const std::string last = g_last_error;
-  if (grow(s_pool, need, "seeded particles") == TPMC_OK) return true;
+  if (alloc(&pool.ptr, need, "seeded particles") == TPMC_OK) {
+    pool.cap = need;
+    return true;
+  }
   g_last_error = last;  // not the caller's failure
   return false;
+}
+
+// Frees a pool once the kernels that use it are done.
+void Ctx::release_pool(Pool& pool) {
+  if (!pool.ptr) return;
+  if (pool.done) cudaEventSynchronize(pool.done);
+  release(pool.ptr);
+  pool.ptr = nullptr;
+  pool.cap = 0;
+}
+
+// Pools give way to everything else that needs the memory.
+bool Ctx::release_pools() {
+  bool any = false;
+  for (Pool* p : pools) {
+    any = any || p->ptr;
+    release_pool(*p);
+  }
+  return any;
+}
+
+void Ctx::destroy_pool(Pool& pool) {
+  release_pool(pool);
+  if (pool.side) cudaStreamDestroy(pool.side);
+  for (cudaEvent_t ev : {pool.fork, pool.join, pool.done})
+    if (ev) cudaEventDestroy(ev);
+  pool = Pool();
 }
 
 // Traces a launch through the pool: batches of half of it, seed_kernel then
@@ -237,20 +270,22 @@ bool Ctx::grow_pool(uint64_t total) {
 // kernels fill it.  One stream and batches of 2^26, 2^27 particles: the attitude
 // sweep 236 and 226 ms; two streams of 2^26: 217 (of 2^27: 211, for
 // twice the memory).
-cudaError_t Ctx::trace_pool(TraceArgs a, uint32_t variant, const LaunchCfg& cfg, float cv_area) {
+// a.counter: two counters.
+cudaError_t Ctx::trace_pool(Pool& pool, cudaStream_t stream, TraceArgs a, uint32_t variant, const LaunchCfg& cfg,
+                            float area) {
   // Rough rays first where at most a quarter of the particles is expected to
   // meet the front (its mean projected area over the control volume's).  They
   // cost 55 % of an exact seeding: the satellite (12 % pass) 6.74 -> 6.09 ms for
   // 1e8 particles; the plate sweep (36 %) 33.7 -> 33.6, the cylinder's (55 %) 98.7
   // -> 101.9, so those seed exactly at once.
-  a.prefilter = a.mesh.front_area < 0.25f * cv_area ? 1u : 0u;
+  a.prefilter = a.mesh.front_area < 0.25f * area ? 1u : 0u;
   cudaError_t e = cudaSuccess;
-  if (!side_stream) e = cudaStreamCreateWithFlags(&side_stream, cudaStreamNonBlocking);
-  for (cudaEvent_t* ev : {&fork, &join})
+  if (!pool.side) e = cudaStreamCreateWithFlags(&pool.side, cudaStreamNonBlocking);
+  for (cudaEvent_t* ev : {&pool.fork, &pool.join, &pool.done})
     if (e == cudaSuccess && !*ev) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
   if (e != cudaSuccess) return e;
   const uint64_t total = a.total;
-  uint64_t batch = std::min<uint64_t>(kPoolBatch, (s_pool.cap - 512) / (2 * (32 * kPoolEntryBytes + sizeof(uint32_t))) * 32);
+  uint64_t batch = std::min<uint64_t>(kPoolBatch, (pool.cap - 512) / (2 * (32 * kPoolEntryBytes + sizeof(uint32_t))) * 32);
   // Segments: 512 work indices, fewer where that would not give every warp of
   // the grid about eight.
   const uint64_t warps = (uint64_t)num_sms * cfg.blocks_per_sm * (cfg.block / 32);
@@ -263,25 +298,27 @@ cudaError_t Ctx::trace_pool(TraceArgs a, uint32_t variant, const LaunchCfg& cfg,
     const bool side = (i & 1) != 0;
     if (side && !forked) {
       // the second stream starts where the set-up left the first
-      if ((e = cudaStreamWaitEvent(side_stream, fork, 0)) != cudaSuccess) break;
+      if ((e = cudaStreamWaitEvent(pool.side, pool.fork, 0)) != cudaSuccess) break;
       forked = true;
     }
-    if (i == 0 && total > batch && (e = cudaEventRecord(fork, stream)) != cudaSuccess) break;
+    if (i == 0 && total > batch && (e = cudaEventRecord(pool.fork, stream)) != cudaSuccess) break;
     TraceArgs b = a;
     b.total = std::min(total, a.g0 + batch);
     b.n_seg = (uint32_t)((b.total - a.g0 + a.segment - 1) / a.segment);
-    char* half = (char*)s_pool.ptr + (side ? (s_pool.cap / 2) & ~(size_t)255 : 0);
+    char* half = (char*)pool.ptr + (side ? (pool.cap / 2) & ~(size_t)255 : 0);
     b.pool = half;
     b.seg_count = (uint32_t*)(half + batch * kPoolEntryBytes);
     b.counter = a.counter + (side ? 1 : 0);
-    const cudaStream_t st = side ? side_stream : stream;
+    const cudaStream_t st = side ? pool.side : stream;
     if ((e = launch_seed(b, st)) == cudaSuccess) e = launch_trace(b, variant, cfg, num_sms, st);
   }
   if (forked) {  // also after an error: what was enqueued ends before anything else on the stream
-    cudaError_t e2 = cudaEventRecord(join, side_stream);
-    if (e2 == cudaSuccess) e2 = cudaStreamWaitEvent(stream, join, 0);
+    cudaError_t e2 = cudaEventRecord(pool.join, pool.side);
+    if (e2 == cudaSuccess) e2 = cudaStreamWaitEvent(stream, pool.join, 0);
     if (e == cudaSuccess) e = e2;
   }
+  const cudaError_t e3 = cudaEventRecord(pool.done, stream);
+  if (e == cudaSuccess) e = e3;
   return e;
 }
 
@@ -331,18 +368,14 @@ tpmc_status Ctx::run(const MeshRec& m, const QueryDev* h_queries, uint32_t nq, c
   a.count_work = counters ? 1u : 0u;
   a.vn_table = vn_table;
   if (rec) a.rec = *rec;
-  // mean projected area of the control volume over pi
-  const QueryDev& bq = h_base ? *h_base : *h_queries;
-  const double bx = bq.box_hi[0] - bq.box_lo[0], by = bq.box_hi[1] - bq.box_lo[1], bz = bq.box_hi[2] - bq.box_lo[2];
-  const float cv_area = (float)(bq.cv_kind == TPMC_CV_SPHERE ? bq.r_cv * bq.r_cv : (bx * by + by * bz + bz * bx) / 6.283185307179586);
-  const bool pooled = !counters && !rec && (variant & 1u) == TPMC_FP32 && total >= kPoolMin && grow_pool(total);
+  const bool pooled = !counters && !rec && (variant & 1u) == TPMC_FP32 && total >= kPoolMin && grow_pool(pool, total, kPoolBatch);
   if (pooled) variant |= kVariantPool;
   const LaunchCfg cfg = schedule(m, variant, total);
   a.chunk = cfg.chunk;
   a.smem_nodes = cfg.smem_nodes;
   a.refill_at = cfg.refill_at;
   last_cfg = cfg;
-  if (total > 0 && (e = pooled ? trace_pool(a, variant, cfg, cv_area) : launch_trace(a, variant, cfg, num_sms, stream)) != cudaSuccess)
+  if (total > 0 && (e = pooled ? trace_pool(pool, stream, a, variant, cfg, cv_area(h_base ? *h_base : *h_queries)) : launch_trace(a, variant, cfg, num_sms, stream)) != cudaSuccess)
     return cuda_fail(e, "trace kernel");
   if ((e = launch_finalize(d_queries, d_acc, nq, nq, nullptr, d_out, stream)) != cudaSuccess)
     return cuda_fail(e, "finalize kernel");
@@ -448,13 +481,11 @@ Ctx::~Ctx() {
   if (serve) stop_serving(this);
   for (auto& kv : panels) release(kv.second.d_panel);
   for (auto& kv : meshes) release(kv.second.d_block);
-  for (Scratch* s : {&s_queries, &s_acc, &s_items, &s_misc, &s_base, &s_out, &s_in, &s_pool})
+  for (Scratch* s : {&s_queries, &s_acc, &s_items, &s_misc, &s_base, &s_out, &s_in})
     release(s->ptr);
   release(vn_table);
   if (h_pinned) cudaFreeHost(h_pinned);
-  if (side_stream) cudaStreamDestroy(side_stream);
-  for (cudaEvent_t ev : {fork, join})
-    if (ev) cudaEventDestroy(ev);
+  destroy_pool(pool);
   if (own_stream) cudaStreamDestroy(own_stream);
 }
 

@@ -42,6 +42,16 @@ struct Scratch {
   size_t cap = 0;
 };
 
+// Seeded particles of a launch's batches (Ctx::grow_pool, Ctx::trace_pool), the
+// second stream of the launch and where it leaves and rejoins the first.  Freed
+// when another allocation needs the room, after `done`.
+struct Pool {
+  void* ptr = nullptr;
+  size_t cap = 0;
+  cudaStream_t side = nullptr;
+  cudaEvent_t fork = nullptr, join = nullptr, done = nullptr;
+};
+
 struct ServeState;  // serve.cpp
 
 // BVH width of mesh loads that neither tpmc_set_launch nor tpmc_tune decided.
@@ -57,6 +67,7 @@ constexpr uint64_t kPoolMin = 1u << 23;
 // Particles of a batch, at most and at least (32 bytes each, two batches).
 constexpr uint64_t kPoolBatch = 1ull << 26, kPoolSmallest = 1ull << 20;
 
+float cv_area(const QueryDev& q);
 tpmc_status fill_query(const MeshRec& m, const tpmc_params* p, uint64_t N, QueryDev* q);
 
 inline uint64_t tune_key(uint32_t n_tri, uint32_t variant) {
@@ -71,9 +82,6 @@ struct Ctx {
   int num_sms = 1;
   cudaStream_t own_stream = nullptr;
   cudaStream_t stream = nullptr;
-  // trace_pool: the second stream of a launch, and where it leaves and rejoins the first
-  cudaStream_t side_stream = nullptr;
-  cudaEvent_t fork = nullptr, join = nullptr;
   size_t budget = 0, used = 0;
   uint64_t n_allocs = 0;       // device allocations made since creation
   std::map<void*, size_t> sizes;
@@ -92,7 +100,8 @@ struct Ctx {
   std::map<uint64_t, LaunchCfg> tuned;
   std::map<uint64_t, int> max_blocks;  // trace_max_blocks_per_sm by variant, block and shared memory
   Scratch s_queries, s_acc, s_items, s_misc, s_base, s_out, s_in;
-  Scratch s_pool;              // seeded particles of a batch (grow_pool); released when other allocations need room
+  Pool pool;                   // of the calls on `stream`
+  std::vector<Pool*> pools{&pool};  // all of them (the serving steps have their own)
   float* vn_table = nullptr;   // start tables (normal speed, latitude knots), built once at creation
   void* h_pinned = nullptr;
   int* h_err_word = nullptr;
@@ -108,8 +117,11 @@ struct Ctx {
   tpmc_status run(const MeshRec& m, const QueryDev* h_queries, uint32_t nq, const QueryDev* h_base,
                   const double* d_dirs, const double* d_S, const ItemDev* h_items, uint32_t n_items,
                   uint64_t total, uint32_t variant, tpmc_result* d_out, const RecordsDev* rec);
-  bool grow_pool(uint64_t total);
-  cudaError_t trace_pool(TraceArgs a, uint32_t variant, const LaunchCfg& cfg, float cv_area);
+  bool grow_pool(Pool& pool, uint64_t total, uint64_t max_batch);
+  void release_pool(Pool& pool);
+  bool release_pools();
+  void destroy_pool(Pool& pool);
+  cudaError_t trace_pool(Pool& pool, cudaStream_t stream, TraceArgs a, uint32_t variant, const LaunchCfg& cfg, float area);
   tpmc_status check_error_word();
   ~Ctx();
 };

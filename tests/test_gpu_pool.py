@@ -151,3 +151,38 @@ def test_empty_mesh_counts_every_particle(T):
             assert r["n_particles"] == N and r["n_hits"] == 0 and r["CD"] == 0.0
     finally:
         T.tpmc_destroy(c)
+
+
+@pytest.mark.parametrize("budget_mib", [96, 700, 0])
+def test_served_large_queries_match_direct_calls(T, budget_mib):
+    """Served queries large enough for the steps' pools, among small ones and direct calls that use the context's own
+    pool and make the others give their memory back: every result as alone."""
+    bodies = [M.cylinder(0.5, 2.0, 32, 7), M.satellite(3_000)]
+    sizes = [(0, (1 << 23) + 1), (1, 30_000_001), (0, 100_003), (1, (1 << 23) + 77), (1, 5_000_000), (0, 40_000_000)]
+    c = T.tpmc_create(0, budget_mib << 20)
+    try:
+        meshes = [T.tpmc_mesh_load(c, *b) for b in bodies]
+        params = [_base(T, stream_id=k, want_panels=k % 2 == 1) for k in range(len(sizes))]
+        alone = []
+        for (m, N), p in zip(sizes, params):
+            r = T.tpmc_trace(c, meshes[m], p, N)
+            if p.want_panels:
+                r["panels"] = T.tpmc_panel_sums(c, r["query_id"], len(bodies[m][1]))
+                T.tpmc_panels(c, r["query_id"], len(bodies[m][1]))
+            alone.append(r)
+        for _ in range(2):
+            ids = [T.tpmc_submit(c, meshes[m], p, N) for (m, N), p in zip(sizes, params)]
+            extra = T.tpmc_mesh_load(c, *M.satellite(60_000))
+            direct = T.tpmc_trace(c, meshes[1], params[0], 20_000_000)
+            T.tpmc_mesh_unload(c, extra)
+            for i, a, (m, N) in zip(ids, alone, sizes):
+                r = T.tpmc_poll(c, i)
+                assert [r[k] for k in KEYS] == [a[k] for k in KEYS]
+                if "panels" in a:
+                    assert (T.tpmc_panel_sums(c, i, len(bodies[m][1])) == a["panels"]).all()
+                    T.tpmc_panels(c, i, len(bodies[m][1]))
+            assert direct["n_particles"] == 20_000_000
+        if budget_mib:
+            assert T.tpmc_memory_info(c)["used"] <= budget_mib << 20
+    finally:
+        T.tpmc_destroy(c)
