@@ -179,6 +179,11 @@ LaunchCfg Ctx::schedule(const MeshRec& m, uint32_t variant, uint64_t total) {
     cfg.smem_nodes = 0;  // the hot top of the tree stays in L1; shared-memory staging costs bank conflicts
     cfg.blocks_per_sm = 0;
     cfg.chunk = 0;
+    // Launches that 4 blocks per SM hold at once (77,824 particles on 152 SMs)
+    // run the kernel without a register cap: 4,096 and 40,000 particles on the
+    // hemisphere 276 -> 259 and 422 -> 386 us, on the satellite 136 -> 125 and
+    // 199 -> 186; at 160,000 the two are equal, beyond more warps win.
+    if (total > 0 && total <= (uint64_t)num_sms * 4 * 128 && (variant & 1u) == TPMC_FP32) cfg.blocks_per_sm = 4;
   }
   cfg.smem_nodes = m.dev.width > 2 ? 0u : std::min<uint32_t>(cfg.smem_nodes, m.dev.n_nodes);  // wide: none staged
   // the kernel's own fixed shared memory comes out of the largest staging
@@ -199,6 +204,11 @@ LaunchCfg Ctx::schedule(const MeshRec& m, uint32_t variant, uint64_t total) {
     uint64_t ch = total / std::max<uint64_t>(1, warps * 16);
     ch = (ch / 32) * 32;
     cfg.chunk = (uint32_t)std::min<uint64_t>(1024, std::max<uint64_t>(32, ch));
+    // fewer particles than lanes: an equal share for every warp, so that the
+    // lanes of a warp wait for fewer others (1,000 and 16,000 particles on the
+    // hemisphere 336 -> 214 and 447 -> 335 us, 4,096 on the icosphere 105 -> 91)
+    const uint64_t share = (total + warps - 1) / std::max<uint64_t>(1, warps);
+    if (share > 0 && share < 32) cfg.chunk = (uint32_t)share;
   }
   return cfg;
 }
