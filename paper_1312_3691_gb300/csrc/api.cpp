@@ -332,38 +332,27 @@ cudaError_t Ctx::trace_pool(Pool& pool, cudaStream_t stream, TraceArgs a, uint32
   return e;
 }
 
-// One batched run: nq queries prepared on the device from `base` (+ dirs/S)
-// or uploaded one by one, traced together, finalised into d_out.
-tpmc_status Ctx::run(const MeshRec& m, const QueryDev* h_queries, uint32_t nq, const QueryDev* h_base,
-                     const double* d_dirs, const double* d_S, const ItemDev* h_items, uint32_t n_items, uint64_t total,
-                     uint32_t variant, tpmc_result* d_out, const RecordsDev* rec) {
+// One batched run: nq queries prepared on the device from `base` (+ dirs/S),
+// traced together, finalised into d_out (device memory or the context's pinned
+// results).  Three launches and no copies: the base query goes with the set-up's
+// launch, which also clears the counters, and the reduction writes the error
+// word to pinned memory (two uploads, a memset and two downloads took 25 us of
+// a small call).
+tpmc_status Ctx::run(const MeshRec& m, uint32_t nq, const QueryDev& base, const double* d_dirs, const double* d_S,
+                     uint64_t total, uint32_t variant, tpmc_result* d_out, const RecordsDev* rec) {
   tpmc_status st;
   if ((st = grow(s_queries, sizeof(QueryDev) * (size_t)nq, "queries")) != TPMC_OK) return st;
   if ((st = grow(s_acc, sizeof(AccStripe) * kAccStripes * (size_t)nq, "accumulators")) != TPMC_OK) return st;
-  if ((st = grow(s_items, sizeof(ItemDev) * (size_t)std::max(nq, n_items), "work items")) != TPMC_OK) return st;
-  if ((st = grow(s_misc, 256, "counters")) != TPMC_OK) return st;
-  if ((st = grow(s_base, sizeof(QueryDev), "base query")) != TPMC_OK) return st;
+  if ((st = grow(s_items, sizeof(ItemDev) * (size_t)nq, "work items")) != TPMC_OK) return st;
+  if ((st = grow(s_misc, sizeof(RunWords), "counters")) != TPMC_OK) return st;
   QueryDev* d_queries = (QueryDev*)s_queries.ptr;
   AccStripe* d_acc = (AccStripe*)s_acc.ptr;
   ItemDev* d_items = (ItemDev*)s_items.ptr;
-  unsigned long long* d_counter = (unsigned long long*)s_misc.ptr;
-  int* d_err = (int*)((char*)s_misc.ptr + 64);
+  RunWords* words = (RunWords*)s_misc.ptr;
   cudaError_t e;
-  // Host sources here are pageable, so each copy is staged before the call
-  // returns and the caller's structs may be reused at once.
-  if (h_base) {
-    if ((e = cudaMemcpyAsync(s_base.ptr, h_base, sizeof(QueryDev), cudaMemcpyHostToDevice, stream)) != cudaSuccess)
-      return cuda_fail(e, "upload base query");
-  } else {
-    if ((e = cudaMemcpyAsync(d_queries, h_queries, sizeof(QueryDev) * nq, cudaMemcpyHostToDevice, stream)) != cudaSuccess)
-      return cuda_fail(e, "upload queries");
-    if ((e = cudaMemcpyAsync(d_items, h_items, sizeof(ItemDev) * n_items, cudaMemcpyHostToDevice, stream)) != cudaSuccess)
-      return cuda_fail(e, "upload items");
-  }
-  if ((e = cudaMemsetAsync(s_misc.ptr, 0, 128, stream)) != cudaSuccess) return cuda_fail(e, "clear counter");
   // the set-up also clears the queries' accumulators
-  if ((e = launch_setup(d_queries, nq, h_base ? (const QueryDev*)s_base.ptr : nullptr, d_dirs, d_S,
-                        h_base ? d_items : nullptr, nullptr, d_acc, nq, vn_table, stream)) != cudaSuccess)
+  if ((e = launch_setup(d_queries, nq, &base, d_dirs, d_S, d_items, nullptr, d_acc, nq, vn_table, words, stream)) !=
+      cudaSuccess)
     return cuda_fail(e, "setup kernel");
   TraceArgs a{};
   a.mesh = m.dev;
@@ -371,10 +360,10 @@ tpmc_status Ctx::run(const MeshRec& m, const QueryDev* h_queries, uint32_t nq, c
   a.acc = d_acc;
   a.acc_stride = nq;
   a.items = d_items;
-  a.n_items = h_base ? nq : n_items;
+  a.n_items = nq;
   a.total = total;
-  a.counter = d_counter;
-  a.error = d_err;
+  a.counter = words->counter;
+  a.error = &words->error;
   a.count_work = counters ? 1u : 0u;
   a.vn_table = vn_table;
   if (rec) a.rec = *rec;
@@ -385,12 +374,10 @@ tpmc_status Ctx::run(const MeshRec& m, const QueryDev* h_queries, uint32_t nq, c
   a.smem_nodes = cfg.smem_nodes;
   a.refill_at = cfg.refill_at;
   last_cfg = cfg;
-  if (total > 0 && (e = pooled ? trace_pool(pool, stream, a, variant, cfg, cv_area(h_base ? *h_base : *h_queries)) : launch_trace(a, variant, cfg, num_sms, stream)) != cudaSuccess)
+  if (total > 0 && (e = pooled ? trace_pool(pool, stream, a, variant, cfg, cv_area(base)) : launch_trace(a, variant, cfg, num_sms, stream)) != cudaSuccess)
     return cuda_fail(e, "trace kernel");
-  if ((e = launch_finalize(d_queries, d_acc, nq, nq, nullptr, d_out, stream)) != cudaSuccess)
+  if ((e = launch_finalize(d_queries, d_acc, nq, nq, nullptr, d_out, &words->error, h_err_word, stream)) != cudaSuccess)
     return cuda_fail(e, "finalize kernel");
-  if ((e = cudaMemcpyAsync(h_err_word, d_err, sizeof(int), cudaMemcpyDeviceToHost, stream)) != cudaSuccess)
-    return cuda_fail(e, "read error word");
   return TPMC_OK;
 }
 
@@ -491,7 +478,7 @@ Ctx::~Ctx() {
   if (serve) stop_serving(this);
   for (auto& kv : panels) release(kv.second.d_panel);
   for (auto& kv : meshes) release(kv.second.d_block);
-  for (Scratch* s : {&s_queries, &s_acc, &s_items, &s_misc, &s_base, &s_out, &s_in})
+  for (Scratch* s : {&s_queries, &s_acc, &s_items, &s_misc, &s_out, &s_in})
     release(s->ptr);
   release(vn_table);
   if (h_pinned) cudaFreeHost(h_pinned);
@@ -525,7 +512,7 @@ tpmc_status tpmc_create(int device, size_t mem_budget_bytes, tpmc_ctx** out) {
   if ((e = cudaStreamCreateWithFlags(&c->own_stream, cudaStreamNonBlocking)) != cudaSuccess)
     return cuda_fail(e, "cudaStreamCreate");
   c->stream = c->own_stream;
-  if ((e = cudaMallocHost(&c->h_pinned, 4096)) != cudaSuccess) return cuda_fail(e, "cudaMallocHost");
+  if ((e = cudaMallocHost(&c->h_pinned, kPinnedBytes)) != cudaSuccess) return cuda_fail(e, "cudaMallocHost");
   {
     void* t = nullptr;
     tpmc_status st = c->alloc(&t, sizeof(float) * kTableFloats, "start tables");
@@ -535,6 +522,8 @@ tpmc_status tpmc_create(int device, size_t mem_budget_bytes, tpmc_ctx** out) {
     if ((e = cudaStreamSynchronize(c->stream)) != cudaSuccess) return cuda_fail(e, "start tables");
   }
   c->h_err_word = (int*)c->h_pinned;
+  c->h_results = (tpmc_result*)((char*)c->h_pinned + 256);
+  c->h_inputs = (double*)((char*)c->h_pinned + 256 + kPinnedItems * sizeof(tpmc_result));
   *c->h_err_word = 0;
   *out = reinterpret_cast<tpmc_ctx*>(c.release());
   return TPMC_OK;
@@ -674,15 +663,9 @@ static tpmc_status trace_common(Ctx* c, tpmc_mesh_id mesh, const tpmc_params* pa
     rec.K = records->K;
     cudaMemsetAsync(rec.tri, 0xFF, N * K * sizeof(uint32_t), c->stream);
   }
-  ItemDev item;
-  std::memset(&item, 0, sizeof(item));
-  item.g_begin = 0; item.pid_begin = 0; item.count = N; item.query = 0;
-  tpmc_status rs = c->grow(c->s_out, sizeof(tpmc_result), "result");
-  if (rs == TPMC_OK)
-    rs = c->run(m, &q, 1, nullptr, nullptr, nullptr, &item, 1, N, trace_variant(params, m.dev), (tpmc_result*)c->s_out.ptr,
-                records ? &rec : nullptr);
+  const tpmc_status rs = c->run(m, 1, q, nullptr, nullptr, N, trace_variant(params, m.dev), c->h_results,
+                                records ? &rec : nullptr);
   cudaError_t e = cudaSuccess;
-  if (rs == TPMC_OK) e = cudaMemcpyAsync(out, c->s_out.ptr, sizeof(tpmc_result), cudaMemcpyDeviceToHost, c->stream);
   if (rs == TPMC_OK && e == cudaSuccess && records) {
     const size_t K = records->K;
     auto cp = [&](void* dst, const void* src, size_t bytes) {
@@ -702,6 +685,7 @@ static tpmc_status trace_common(Ctx* c, tpmc_mesh_id mesh, const tpmc_params* pa
     return rs != TPMC_OK ? rs : cuda_fail(e, "trace");
   }
   if ((st = c->check_error_word()) != TPMC_OK) { c->release(d_panel); return st; }
+  *out = *c->h_results;
   const auto t1 = std::chrono::steady_clock::now();
   out->ms = std::chrono::duration<double, std::milli>(t1 - t0).count();
   if (out->status != TPMC_OK) {
@@ -807,7 +791,7 @@ static tpmc_status sweep_common(Ctx* c, tpmc_mesh_id mesh, const tpmc_params* ba
   const MeshRec& m = it->second;
   QueryDev q;
   if ((st = fill_query(m, base, N_each, &q)) != TPMC_OK) return st;
-  return c->run(m, nullptr, K, &q, d_dirs, d_S, nullptr, 0, (uint64_t)K * N_each, trace_variant(base, m.dev), d_out, nullptr);
+  return c->run(m, K, q, d_dirs, d_S, (uint64_t)K * N_each, trace_variant(base, m.dev), d_out, nullptr);
 }
 
 tpmc_status tpmc_sweep(tpmc_ctx* ctx, tpmc_mesh_id mesh, const tpmc_params* base, const double* h_dirs,
@@ -818,20 +802,34 @@ tpmc_status tpmc_sweep(tpmc_ctx* ctx, tpmc_mesh_id mesh, const tpmc_params* base
   cudaSetDevice(c->device);
   const auto t0 = std::chrono::steady_clock::now();
   tpmc_status st;
-  const size_t in_bytes = (size_t)K * 4 * sizeof(double);
-  if ((st = c->grow(c->s_in, std::max(in_bytes, sizeof(QueryDev)), "sweep inputs")) != TPMC_OK) return st;
-  if ((st = c->grow(c->s_out, (size_t)K * sizeof(tpmc_result), "sweep results")) != TPMC_OK) return st;
-  double* d_dirs = h_dirs ? (double*)c->s_in.ptr : nullptr;
-  double* d_S = h_S ? (double*)c->s_in.ptr + 3 * (size_t)K : nullptr;
+  // Short sweeps: the kernels read their inputs from and write their results to
+  // pinned memory; long ones go through device memory.
+  const bool pinned = K <= kPinnedItems;
+  double* d_in = c->h_inputs;
+  tpmc_result* d_out = c->h_results;
+  if (!pinned) {
+    if ((st = c->grow(c->s_in, std::max((size_t)K * 4 * sizeof(double), sizeof(QueryDev)), "sweep inputs")) != TPMC_OK) return st;
+    if ((st = c->grow(c->s_out, (size_t)K * sizeof(tpmc_result), "sweep results")) != TPMC_OK) return st;
+    d_in = (double*)c->s_in.ptr;
+    d_out = (tpmc_result*)c->s_out.ptr;
+  }
+  double* d_dirs = h_dirs ? d_in : nullptr;
+  double* d_S = h_S ? d_in + 3 * (size_t)K : nullptr;
   cudaError_t e = cudaSuccess;
-  if (h_dirs) e = cudaMemcpyAsync(d_dirs, h_dirs, (size_t)K * 3 * sizeof(double), cudaMemcpyHostToDevice, c->stream);
-  if (e == cudaSuccess && h_S) e = cudaMemcpyAsync(d_S, h_S, (size_t)K * sizeof(double), cudaMemcpyHostToDevice, c->stream);
-  if (e != cudaSuccess) return cuda_fail(e, "upload sweep inputs");
-  if ((st = sweep_common(c, mesh, base, d_dirs, d_S, K, N_each, (tpmc_result*)c->s_out.ptr)) != TPMC_OK) return st;
-  e = cudaMemcpyAsync(h_out, c->s_out.ptr, (size_t)K * sizeof(tpmc_result), cudaMemcpyDeviceToHost, c->stream);
+  if (pinned) {
+    if (h_dirs) std::memcpy(d_dirs, h_dirs, (size_t)K * 3 * sizeof(double));
+    if (h_S) std::memcpy(d_S, h_S, (size_t)K * sizeof(double));
+  } else {
+    if (h_dirs) e = cudaMemcpyAsync(d_dirs, h_dirs, (size_t)K * 3 * sizeof(double), cudaMemcpyHostToDevice, c->stream);
+    if (e == cudaSuccess && h_S) e = cudaMemcpyAsync(d_S, h_S, (size_t)K * sizeof(double), cudaMemcpyHostToDevice, c->stream);
+    if (e != cudaSuccess) return cuda_fail(e, "upload sweep inputs");
+  }
+  if ((st = sweep_common(c, mesh, base, d_dirs, d_S, K, N_each, d_out)) != TPMC_OK) return st;
+  if (!pinned) e = cudaMemcpyAsync(h_out, d_out, (size_t)K * sizeof(tpmc_result), cudaMemcpyDeviceToHost, c->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
   if (e != cudaSuccess) return cuda_fail(e, "sweep");
   if ((st = c->check_error_word()) != TPMC_OK) return st;
+  if (pinned) std::memcpy(h_out, d_out, (size_t)K * sizeof(tpmc_result));
   const double ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
   for (uint32_t k = 0; k < K; ++k) h_out[k].ms = ms;
   return TPMC_OK;

@@ -32,9 +32,19 @@ namespace {
 constexpr int kSetupThreads = 160;
 constexpr int kSetupParts = 6;
 
+// The base query comes with the launch (no copy to the device before it), and
+// the run's counters and error word (`zero`) are cleared here (no memset).
+struct SetupBase {
+  QueryDev q;
+  uint32_t given;
+};
+
 __global__ void __launch_bounds__(kSetupThreads)
-    setup_kernel(QueryDev* qs, const QueryDev* base, const double* dirs, const double* Svals, ItemDev* items,
-                 const uint32_t* slots, AccStripe* acc, uint32_t acc_stride, const double* knots) {
+    setup_kernel(QueryDev* qs, const __grid_constant__ SetupBase with, const double* dirs, const double* Svals, ItemDev* items,
+                 const uint32_t* slots, AccStripe* acc, uint32_t acc_stride, const double* knots, RunWords* zero) {
+  const QueryDev* base = with.given ? &with.q : nullptr;
+  if (zero != nullptr && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < sizeof(RunWords) / 4)
+    reinterpret_cast<uint32_t*>(zero)[threadIdx.x] = 0u;
   const uint32_t slot = slots != nullptr ? slots[blockIdx.x] : blockIdx.x;
   QueryDev& q = qs[slot];
   const QueryDev& in = base != nullptr ? *base : q;  // the inputs (T_inf, m, V, dir, ...)
@@ -329,76 +339,81 @@ __global__ void vn_table_kernel(float* tab) {
 }
 
 // -------------------------------------------------------- final reduction
-// Thread i reduces query slots[i] (or i) into out[i].
-__global__ void finalize_kernel(const QueryDev* qs, const AccStripe* acc, uint32_t stride, uint32_t nq,
-                                const uint32_t* slots, tpmc_result* out) {
-  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+// Warp i reduces query slots[i] (or i) into out[i]; the first thread passes the
+// trace kernel's error word on (err_out, when given).  Lanes sum the stripes'
+// words side by side and compute the components side by side: a chain of double
+// divisions and a square root in one thread after 120 loads took 9 us.
+__global__ void __launch_bounds__(128)
+    finalize_kernel(const QueryDev* qs, const AccStripe* acc, uint32_t stride, uint32_t nq, const uint32_t* slots,
+                    tpmc_result* out, const int* err, int* err_out) {
+  const uint32_t i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31u;
+  if (err_out != nullptr && blockIdx.x == 0 && threadIdx.x == 0) *err_out = *err;
   if (i >= nq) return;
   const uint32_t qi = slots != nullptr ? slots[i] : i;
   const QueryDev& q = qs[qi];
-  // the stripes' sums; the squared-drag limbs as one exact 128-bit integer
-  long long F[3] = {0, 0, 0}, T[3] = {0, 0, 0};
-  unsigned long long hits = 0, hitp = 0, trunc = 0, parts = 0, nodes = 0, tris = 0, d2lo = 0, d2hi = 0;
-  for (int j = 0; j < kAccStripes; ++j) {
-    const AccStripe& A = acc[(size_t)j * stride + qi];
-    for (int k = 0; k < 3; ++k) { F[k] += A.F[k]; T[k] += A.T[k]; }
-    hits += A.hits;
-    hitp += A.hit_particles;
-    trunc += A.truncated;
-    parts += A.particles;
-    nodes += A.nodes;
-    tris += A.tris;
-    const unsigned long long add_lo[3] = {A.d2[0], A.d2[1] << 30, A.d2[2] << 60};
-    const unsigned long long add_hi[3] = {0ull, A.d2[1] >> 34, A.d2[2] >> 4};
-    for (int k = 0; k < 3; ++k) {
-      const unsigned long long nlo = d2lo + add_lo[k];
-      d2hi += add_hi[k] + (nlo < d2lo ? 1ull : 0ull);
-      d2lo = nlo;
-    }
-  }
-  tpmc_result r;
-  memset(&r, 0, sizeof(r));
-  r.status = q.status;
-  if (q.status == TPMC_OK) {
+  // word (lane & 15) of the stripes; the limbs' sums stay below 2^64 too
+  unsigned long long v = 0ull;
+#pragma unroll
+  for (int j = 0; j < kAccStripes / 2; ++j)
+    v += reinterpret_cast<const unsigned long long*>(&acc[(size_t)(2 * j + (lane >> 4)) * stride + qi])[lane & 15u];
+  v += __shfl_xor_sync(kFull, v, 16);
+  const unsigned long long parts = __shfl_sync(kFull, v, 9);
+  // the squared-drag limbs as one exact 128-bit integer
+  const unsigned long long l0 = __shfl_sync(kFull, v, 12), l1 = __shfl_sync(kFull, v, 13), l2 = __shfl_sync(kFull, v, 14);
+  unsigned long long d2lo = l0 + (l1 << 30), d2hi = (l1 >> 34) + (l2 >> 4) + (d2lo < l0 ? 1ull : 0ull);
+  const unsigned long long before = d2lo;
+  d2lo += l2 << 60;
+  d2hi += d2lo < before ? 1ull : 0ull;
+  tpmc_result& res = out[i];
+  // every word of the result starts at zero; lanes then write their own parts
+  for (uint32_t w = lane; w < sizeof(tpmc_result) / 8; w += 32) reinterpret_cast<unsigned long long*>(&res)[w] = 0ull;
+  __syncwarp();
+  int status = q.status;
+  if (status == TPMC_OK) {
     const double Np = (double)parts;
-    double sdv[3], srdv[3];
-    for (int k = 0; k < 3; ++k) {
-      sdv[k] = (double)F[k] * q.quantum;
-      srdv[k] = (double)T[k] * q.quantum;
-      r.sum_dv_q[k] = F[k];
-      r.sum_rdv_q[k] = T[k];
-    }
-    // force = (Gamma/N) m c sum(dv) (§II.A); C_D = F . Vhat / (q_inf A_ref) (Eq. 1)
+    // lanes 0-2: force, lanes 3-5: torque; force = (Gamma/N) m c sum(dv) (§II.A)
+    const double sum = (double)(long long)v * q.quantum;
     const double scale = Np > 0 ? q.gamma / Np * q.m * q.c_mp : 0.0;
-    for (int k = 0; k < 3; ++k) { r.force[k] = scale * sdv[k]; r.torque[k] = scale * srdv[k]; }
-    r.CD = (r.force[0] * q.vhat[0] + r.force[1] * q.vhat[1] + r.force[2] * q.vhat[2]) / (q.q_inf * q.A_ref);
-    // force and moment coefficient vectors (the moment about ref over q_inf A_ref l_ref, §III.D.1)
-    for (int k = 0; k < 3; ++k) {
-      r.CF[k] = r.force[k] / (q.q_inf * q.A_ref);
-      r.CM[k] = r.torque[k] / (q.q_inf * q.A_ref * q.l_ref);
+    const double f = scale * sum;
+    const double f0 = __shfl_sync(kFull, f, 0), f1 = __shfl_sync(kFull, f, 1), f2 = __shfl_sync(kFull, f, 2);
+    const double s0 = __shfl_sync(kFull, sum, 0), s1 = __shfl_sync(kFull, sum, 1), s2 = __shfl_sync(kFull, sum, 2);
+    if (lane < 3) {
+      res.force[lane] = f;
+      res.sum_dv_q[lane] = (long long)v;
+      res.CF[lane] = f / (q.q_inf * q.A_ref);
+      res.center[lane] = q.center[lane];
+    } else if (lane < 6) {
+      // force and moment coefficient vectors (the moment about ref over q_inf A_ref l_ref, §III.D.1)
+      res.torque[lane - 3] = f;
+      res.sum_rdv_q[lane - 3] = (long long)v;
+      res.CM[lane - 3] = f / (q.q_inf * q.A_ref * q.l_ref);
+    } else if (lane < 12) {
+      uint64_t* const counts[6] = {&res.n_hits, &res.n_hit_particles, &res.n_truncated, &res.n_particles,
+                                   &res.n_node_visits, &res.n_tri_tests};
+#pragma unroll
+      for (uint32_t c = 0; c < 6; ++c)
+        if (lane == 6 + c) *counts[c] = v;
+    } else if (lane == 12) {
+      // C_D = F . Vhat / (q_inf A_ref) (Eq. 1)
+      res.CD = (f0 * q.vhat[0] + f1 * q.vhat[1] + f2 * q.vhat[2]) / (q.q_inf * q.A_ref);
+    } else if (lane == 13) {
+      const double mean = Np > 0 ? (s0 * q.vhat[0] + s1 * q.vhat[1] + s2 * q.vhat[2]) / Np : 0.0;
+      const double d2 = ((double)d2hi * 18446744073709551616.0 + (double)d2lo) * q.quantum2;
+      const double var = Np > 1 ? fmax(0.0, (d2 - Np * mean * mean) / (Np - 1.0)) : 0.0;
+      res.CD_sigma = Np > 0 ? q.gamma * q.m * q.c_mp / (q.q_inf * q.A_ref) * sqrt(var / Np) : 0.0;
+    } else if (lane == 14) {
+      res.S = q.S;
+      res.S_W = q.S / q.cw;
+      res.gamma = q.gamma;
+      res.weight = Np > 0 ? q.gamma / Np : 0.0;
+      res.q_inf = q.q_inf;
+      res.c_mp = q.c_mp;
+      res.r_cv = q.r_cv;
+      res.fixed_quantum = q.quantum;
     }
-    const double mean = Np > 0 ? (sdv[0] * q.vhat[0] + sdv[1] * q.vhat[1] + sdv[2] * q.vhat[2]) / Np : 0.0;
-    const double d2 = ((double)d2hi * 18446744073709551616.0 + (double)d2lo) * q.quantum2;
-    const double var = Np > 1 ? fmax(0.0, (d2 - Np * mean * mean) / (Np - 1.0)) : 0.0;
-    r.CD_sigma = Np > 0 ? q.gamma * q.m * q.c_mp / (q.q_inf * q.A_ref) * sqrt(var / Np) : 0.0;
-    r.S = q.S;
-    r.S_W = q.S / q.cw;
-    r.gamma = q.gamma;
-    r.weight = Np > 0 ? q.gamma / Np : 0.0;
-    r.q_inf = q.q_inf;
-    r.c_mp = q.c_mp;
-    r.r_cv = q.r_cv;
-    for (int k = 0; k < 3; ++k) r.center[k] = q.center[k];
-    r.fixed_quantum = q.quantum;
-    r.n_particles = parts;
-    r.n_hits = hits;
-    r.n_hit_particles = hitp;
-    r.n_truncated = trunc;
-    r.n_node_visits = nodes;
-    r.n_tri_tests = tris;
-    if (parts != q.N) r.status = TPMC_ECUDA;
+    if (parts != q.N) status = TPMC_ECUDA;
   }
-  out[i] = r;
+  if (lane == 31) res.status = status;
 }
 
 __global__ void panels_kernel(const QueryDev* q, const long long* panel, const double* frames64, uint32_t n_tri,
@@ -424,16 +439,20 @@ __global__ void panels_kernel(const QueryDev* q, const long long* panel, const d
 }  // namespace
 
 // ------------------------------------------------------------- launchers
-cudaError_t launch_setup(QueryDev* d_queries, uint32_t nq, const QueryDev* d_base, const double* d_dirs,
+cudaError_t launch_setup(QueryDev* d_queries, uint32_t nq, const QueryDev* h_base, const double* d_dirs,
                          const double* d_S, ItemDev* d_items, const uint32_t* d_slots, AccStripe* d_acc,
-                         uint32_t acc_stride, const float* tables, cudaStream_t stream) {
+                         uint32_t acc_stride, const float* tables, RunWords* d_zero, cudaStream_t stream) {
   if (nq == 0) return cudaSuccess;
+  static_assert(sizeof(SetupBase) <= 3800, "a kernel's parameters");
+  SetupBase with{};
+  with.given = h_base != nullptr ? 1u : 0u;
+  if (h_base != nullptr) with.q = *h_base;
   // Blocks of their own for the table as long as the chip's SMs are not all
   // busy with other queries (152 SMs; beyond that the split only repeats the
   // scalars the table needs).
   const dim3 grid(nq, nq * kSetupParts <= 2 * 152 ? kSetupParts : 1);
-  setup_kernel<<<grid, kSetupThreads, 0, stream>>>(d_queries, d_base, d_dirs, d_S, d_items, d_slots, d_acc, acc_stride,
-                                                   reinterpret_cast<const double*>(tables + kVnNS * kVnNZ + 1));
+  setup_kernel<<<grid, kSetupThreads, 0, stream>>>(d_queries, with, d_dirs, d_S, d_items, d_slots, d_acc, acc_stride,
+                                                   reinterpret_cast<const double*>(tables + kVnNS * kVnNZ + 1), d_zero);
   return cudaGetLastError();
 }
 
@@ -516,9 +535,10 @@ cudaError_t launch_trace(const TraceArgs& args, uint32_t variant, const LaunchCf
 }
 
 cudaError_t launch_finalize(const QueryDev* d_queries, const AccStripe* d_acc, uint32_t acc_stride, uint32_t nq,
-                            const uint32_t* d_slots, tpmc_result* d_out, cudaStream_t stream) {
+                            const uint32_t* d_slots, tpmc_result* d_out, const int* d_err, int* err_out,
+                            cudaStream_t stream) {
   if (nq == 0) return cudaSuccess;
-  finalize_kernel<<<(nq + 127) / 128, 128, 0, stream>>>(d_queries, d_acc, acc_stride, nq, d_slots, d_out);
+  finalize_kernel<<<(nq + 3) / 4, 128, 0, stream>>>(d_queries, d_acc, acc_stride, nq, d_slots, d_out, d_err, err_out);
   return cudaGetLastError();
 }
 

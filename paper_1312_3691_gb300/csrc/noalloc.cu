@@ -9,14 +9,14 @@
 // caller creates the context and loads its meshes at start-up (those calls do
 // allocate) and then calls this entry point in the loop.
 //
-// The per-call scratch of the sweep (query table, accumulators, work items,
-// inputs staged for the device, results, work counter, error word) lives in
-// one file-scope device array of fixed size, so the call itself performs no
+// The per-call scratch of the sweep (query table, accumulators, work items, work
+// counter, error word) lives in one file-scope device array of fixed size, so the call itself performs no
 // allocation.  Every GPU that loads this library holds the array until the
 // process exits.  All calls on a device share it: each call clears what must
 // start at zero, and two calls that overlap on the GPU (different streams or
 // threads of different contexts on one device) race on it.
 #include <chrono>
+#include <cstring>
 #include <mutex>
 
 #include "runtime.h"
@@ -27,17 +27,12 @@ namespace {
 constexpr uint32_t kNoAllocMaxQueries = 64;
 
 struct NoAllocArea {
-  QueryDev base;
   QueryDev queries[kNoAllocMaxQueries];
   AccStripe acc[kAccStripes * kNoAllocMaxQueries];  // stripe-major, kNoAllocMaxQueries slots per stripe
   ItemDev items[kNoAllocMaxQueries];
-  double dirs[3 * kNoAllocMaxQueries];
-  double S[kNoAllocMaxQueries];
-  tpmc_result results[kNoAllocMaxQueries];
-  unsigned long long counter;
-  int error;
-  int pad;
+  RunWords words;
 };
+static_assert(kNoAllocMaxQueries <= kPinnedItems, "inputs and results use the context's pinned memory");
 
 // Fixed scratch of tpmc_sweep_noalloc (about 100 KB).
 static __device__ __align__(256) unsigned char g_noalloc_scratch[sizeof(NoAllocArea)];
@@ -90,17 +85,14 @@ extern "C" tpmc_status tpmc_sweep_noalloc(tpmc_ctx* ctx, tpmc_mesh_id mesh, cons
   NoAllocArea* A = nullptr;
   if ((e = area_on_device(c->device, &A)) != cudaSuccess) return cuda_fail(e, "cudaGetSymbolAddress");
   cudaStream_t s = c->stream;
-  // inputs (host sources are pageable, so each copy is staged before the call returns)
-  e = cudaMemcpyAsync(&A->base, &q, sizeof(QueryDev), cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess && h_dirs)
-    e = cudaMemcpyAsync(A->dirs, h_dirs, (size_t)K * 3 * sizeof(double), cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess && h_S) e = cudaMemcpyAsync(A->S, h_S, (size_t)K * sizeof(double), cudaMemcpyHostToDevice, s);
-  // the array keeps the previous call's contents: clear the work counter and the error word (the
-  // set-up clears the sums)
-  if (e == cudaSuccess) e = cudaMemsetAsync(&A->counter, 0, sizeof(unsigned long long) + 2 * sizeof(int), s);
-  if (e != cudaSuccess) return cuda_fail(e, "tpmc_sweep_noalloc inputs");
-  if ((e = launch_setup(A->queries, K, &A->base, h_dirs ? A->dirs : nullptr, h_S ? A->S : nullptr, A->items, nullptr,
-                        A->acc, kNoAllocMaxQueries, c->vn_table, s)) != cudaSuccess)
+  // inputs and results in the context's pinned memory, as in short sweeps; the set-up clears the sums, the counters
+  // and the error word, which keep the previous call's values
+  double* dirs = h_dirs ? c->h_inputs : nullptr;
+  double* S = h_S ? c->h_inputs + 3 * (size_t)K : nullptr;
+  if (h_dirs) std::memcpy(dirs, h_dirs, (size_t)K * 3 * sizeof(double));
+  if (h_S) std::memcpy(S, h_S, (size_t)K * sizeof(double));
+  if ((e = launch_setup(A->queries, K, &q, dirs, S, A->items, nullptr, A->acc, kNoAllocMaxQueries, c->vn_table, &A->words,
+                        s)) != cudaSuccess)
     return cuda_fail(e, "setup kernel");
   TraceArgs a{};
   a.mesh = m.dev;
@@ -110,8 +102,8 @@ extern "C" tpmc_status tpmc_sweep_noalloc(tpmc_ctx* ctx, tpmc_mesh_id mesh, cons
   a.items = A->items;
   a.n_items = K;
   a.total = (uint64_t)K * N_each;
-  a.counter = &A->counter;
-  a.error = &A->error;
+  a.counter = A->words.counter;
+  a.error = &A->words.error;
   a.count_work = c->counters ? 1u : 0u;
   a.vn_table = c->vn_table;
   const LaunchCfg cfg = c->schedule(m, trace_variant(base, m.dev), a.total);
@@ -119,14 +111,12 @@ extern "C" tpmc_status tpmc_sweep_noalloc(tpmc_ctx* ctx, tpmc_mesh_id mesh, cons
   a.smem_nodes = cfg.smem_nodes;
   a.refill_at = cfg.refill_at;
   if ((e = launch_trace(a, trace_variant(base, m.dev), cfg, c->num_sms, s)) != cudaSuccess) return cuda_fail(e, "trace kernel");
-  if ((e = launch_finalize(A->queries, A->acc, kNoAllocMaxQueries, K, nullptr, A->results, s)) != cudaSuccess)
+  if ((e = launch_finalize(A->queries, A->acc, kNoAllocMaxQueries, K, nullptr, c->h_results, &A->words.error, c->h_err_word, s)) !=
+      cudaSuccess)
     return cuda_fail(e, "finalize kernel");
-  int err_word = 0;
-  e = cudaMemcpyAsync(h_out, A->results, (size_t)K * sizeof(tpmc_result), cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&err_word, &A->error, sizeof(int), cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  if (e != cudaSuccess) return cuda_fail(e, "tpmc_sweep_noalloc");
-  if (err_word != 0) return fail(TPMC_ECUDA, "trace kernel reported a traversal stack overflow");
+  if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return cuda_fail(e, "tpmc_sweep_noalloc");
+  if ((st = c->check_error_word()) != TPMC_OK) return st;
+  std::memcpy(h_out, c->h_results, (size_t)K * sizeof(tpmc_result));
   // as tpmc_sweep: an item that its set-up rejected reports that in its own
   // status, and every item carries the call's wall time
   const double ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();

@@ -54,6 +54,10 @@ struct Pool {
 
 struct ServeState;  // serve.cpp
 
+// Items of a sweep whose inputs and results stay in the context's pinned memory.
+constexpr uint32_t kPinnedItems = 256;
+constexpr size_t kPinnedBytes = 256 + kPinnedItems * (sizeof(tpmc_result) + 4 * sizeof(double));
+
 // BVH width of mesh loads that neither tpmc_set_launch nor tpmc_tune decided.
 constexpr uint32_t kDefaultBvhWidth = 2;
 
@@ -99,12 +103,14 @@ struct Ctx {
   LaunchCfg last_cfg;
   std::map<uint64_t, LaunchCfg> tuned;
   std::map<uint64_t, int> max_blocks;  // trace_max_blocks_per_sm by variant, block and shared memory
-  Scratch s_queries, s_acc, s_items, s_misc, s_base, s_out, s_in;
+  Scratch s_queries, s_acc, s_items, s_misc, s_out, s_in;
   Pool pool;                   // of the calls on `stream`
   std::vector<Pool*> pools{&pool};  // all of them (the serving steps have their own)
   float* vn_table = nullptr;   // start tables (normal speed, latitude knots), built once at creation
   void* h_pinned = nullptr;
-  int* h_err_word = nullptr;
+  int* h_err_word = nullptr;          // in h_pinned, as are the next two
+  tpmc_result* h_results = nullptr;   // [kPinnedItems], written by the reduction
+  double* h_inputs = nullptr;         // [kPinnedItems][4] directions and speed ratios, read by the set-up
   ServeState* serve = nullptr;
 
   uint32_t width_for(uint32_t n_tri) const;
@@ -114,8 +120,7 @@ struct Ctx {
   void release(void* p);
   tpmc_status grow(Scratch& s, size_t bytes, const char* what);
   LaunchCfg schedule(const MeshRec& m, uint32_t variant, uint64_t total);  // variant: see trace_variant
-  tpmc_status run(const MeshRec& m, const QueryDev* h_queries, uint32_t nq, const QueryDev* h_base,
-                  const double* d_dirs, const double* d_S, const ItemDev* h_items, uint32_t n_items,
+  tpmc_status run(const MeshRec& m, uint32_t nq, const QueryDev& base, const double* d_dirs, const double* d_S,
                   uint64_t total, uint32_t variant, tpmc_result* d_out, const RecordsDev* rec);
   bool grow_pool(Pool& pool, uint64_t total, uint64_t max_batch);
   void release_pool(Pool& pool);

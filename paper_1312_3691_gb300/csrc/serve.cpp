@@ -218,7 +218,7 @@ bool enqueue_step(ServeState* s, int b, int prev, const std::vector<Request*>& c
     e = cudaMemcpyAsync(B.d_fresh, B.h_fresh, n_fresh * sizeof(uint32_t), cudaMemcpyHostToDevice, st);
     // the set-up also clears the fresh slots' accumulators
     if (e == cudaSuccess)
-      e = launch_setup(s->d_q, n_fresh, nullptr, nullptr, nullptr, nullptr, B.d_fresh, s->d_acc, kSlots, c->vn_table, st);
+      e = launch_setup(s->d_q, n_fresh, nullptr, nullptr, nullptr, nullptr, B.d_fresh, s->d_acc, kSlots, c->vn_table, nullptr, st);
   }
   if (e == cudaSuccess) e = cudaMemsetAsync(B.d_counters, 0, 2 * kMaxGroups * sizeof(unsigned long long), st);
   // the groups run on their own streams once the set-up is done, so that one
@@ -300,7 +300,7 @@ bool enqueue_step(ServeState* s, int b, int prev, const std::vector<Request*>& c
   if (!B.finishing.empty() && e == cudaSuccess) {
     e = cudaMemcpyAsync(B.d_fin, B.h_fin, B.finishing.size() * sizeof(uint32_t), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess)
-      e = launch_finalize(s->d_q, s->d_acc, kSlots, (uint32_t)B.finishing.size(), B.d_fin, B.d_res, st);
+      e = launch_finalize(s->d_q, s->d_acc, kSlots, (uint32_t)B.finishing.size(), B.d_fin, B.d_res, nullptr, nullptr, st);
     if (e == cudaSuccess)
       e = cudaMemcpyAsync(B.h_res, B.d_res, B.finishing.size() * sizeof(tpmc_result), cudaMemcpyDeviceToHost, st);
   }

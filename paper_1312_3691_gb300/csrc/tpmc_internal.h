@@ -249,11 +249,19 @@ inline uint32_t trace_variant(const tpmc_params* p, const MeshDev& m) {
 inline uint32_t variant_width(uint32_t v) { return (v & kVariantWide8) ? 8u : ((v & kVariantWide4) ? 4u : 2u); }
 inline uint32_t node_float4s(uint32_t width) { return width == 8 ? 5u : (width == 4 ? 4u : 2u); }
 
+// A run's counters (the second for the pool's second stream) and error word.
+struct RunWords {
+  unsigned long long counter[2];
+  int error;
+  int pad[3];
+};
+
 // Set-up of nq queries (block i: slot slots[i], or i), which also clears
-// their accumulator stripes in acc (stripe-major, acc_stride slots per stripe).
-cudaError_t launch_setup(QueryDev* d_queries, uint32_t nq, const QueryDev* d_base, const double* d_dirs,
+// their accumulator stripes in acc (stripe-major, acc_stride slots per stripe)
+// and, when given, the run's words.
+cudaError_t launch_setup(QueryDev* d_queries, uint32_t nq, const QueryDev* h_base, const double* d_dirs,
                          const double* d_S, ItemDev* d_items, const uint32_t* d_slots, AccStripe* d_acc,
-                         uint32_t acc_stride, const float* tables, cudaStream_t stream);
+                         uint32_t acc_stride, const float* tables, RunWords* d_zero, cudaStream_t stream);
 // Fills a context's tables: the normal-speed start table, then (8-byte
 // aligned) the uniforms Phi(z_j) of the latitude knots as doubles.
 cudaError_t launch_tables(float* d_tables, cudaStream_t stream);
@@ -270,7 +278,8 @@ cudaError_t launch_seed(const TraceArgs& args, cudaStream_t stream);
 cudaError_t launch_trace(const TraceArgs& args, uint32_t variant, const LaunchCfg& cfg, int num_sms,
                          cudaStream_t stream);
 cudaError_t launch_finalize(const QueryDev* d_queries, const AccStripe* d_acc, uint32_t acc_stride, uint32_t nq,
-                            const uint32_t* d_slots, tpmc_result* d_out, cudaStream_t stream);
+                            const uint32_t* d_slots, tpmc_result* d_out, const int* d_err, int* err_out,
+                            cudaStream_t stream);
 cudaError_t launch_panels(const QueryDev* d_query, const long long* d_panel, const float4* frames,
                           const double* frames64, uint32_t n_tri, double* d_pressure, double* d_shear,
                           cudaStream_t stream);

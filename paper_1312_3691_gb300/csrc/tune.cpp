@@ -67,8 +67,8 @@ tpmc_status measure(Ctx* c, const MeshRec& m, const tpmc_params* params, uint64_
     QueryDev q;
     if ((st = fill_query(m, params, each[k], &q)) != TPMC_OK) break;
     cudaEventRecord(tm.e0, c->stream);
-    st = c->run(m, nullptr, kTrialDirs, &q, d_dirs, nullptr, nullptr, 0, (uint64_t)kTrialDirs * each[k],
-                trace_variant(params, m.dev), (tpmc_result*)c->s_out.ptr, nullptr);
+    st = c->run(m, kTrialDirs, q, d_dirs, nullptr, (uint64_t)kTrialDirs * each[k], trace_variant(params, m.dev),
+                (tpmc_result*)c->s_out.ptr, nullptr);
     cudaEventRecord(tm.e1, c->stream);
     if (st != TPMC_OK) break;
     const cudaError_t e = cudaEventSynchronize(tm.e1);
