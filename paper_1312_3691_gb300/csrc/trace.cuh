@@ -819,8 +819,8 @@ __device__ __forceinline__ int trav_pop(Trav<R, B>& t, SP stack) {
 // below n_stage come from the copy in shared memory.
 template <bool STAGE, typename R, typename B, typename SP>
 __device__ __forceinline__ void trav_inner(const MeshDev& m, const float4* __restrict__ s_nodes, uint32_t n_stage,
-                                           const Ray<R, B>& r, Trav<R, B>& t, SP stack, uint32_t& n_nodes,
-                                           int* err) {
+                                           const Ray<R, B>& r, Trav<R, B>& t, SP stack,
+                                           uint32_t& n_nodes) {
   ++n_nodes;
   float4 n0, n1;
   if (STAGE && (uint32_t)t.cur < n_stage) {
@@ -852,26 +852,16 @@ __device__ __forceinline__ void trav_inner(const MeshDev& m, const float4* __res
     tmax1 = fma(fabs(tmax1), (B)1e-6, tmax1);
   }
   const bool h0 = tmin0 <= tmax0, h1 = tmin1 <= tmax1;
-  int c0 = __float_as_int(n1.z), c1 = __float_as_int(n1.w);
+  const int c0 = __float_as_int(n1.z), c1 = __float_as_int(n1.w);
+  // the nearer hit child next, the farther one of two on the stack (which holds
+  // at most one entry a level: the builder keeps the depth below its size)
+  const bool second = h0 && h1 ? tmin1 < tmin0 : h1;
   if (h0 && h1) {
-    B tfar = tmin1;
-    if (tmin1 < tmin0) { const int x = c0; c0 = c1; c1 = x; tfar = tmin0; }
-    if (t.sp >= kMaxStack) {
-      atomicOr(err, 1);
-      t.cur = kDone;
-      t.leaf = 0;
-      return;
-    }
-    stack_put(stack, t.sp, c1, tfar);
+    stack_put(stack, t.sp, second ? c0 : c1, second ? tmin0 : tmin1);
     ++t.sp;
-    t.cur = c0;
-  } else if (h0) {
-    t.cur = c0;
-  } else if (h1) {
-    t.cur = c1;
-  } else {
-    t.cur = trav_pop(t, stack);
   }
+  t.cur = second ? c1 : c0;
+  if (!h0 && !h1) t.cur = trav_pop(t, stack);
   if (t.cur < 0 && t.cur != kDone && t.leaf == 0) {
     t.leaf = t.cur;
     t.cur = trav_pop(t, stack);
@@ -881,7 +871,7 @@ __device__ __forceinline__ void trav_inner(const MeshDev& m, const float4* __res
 // The postponed leaf: test its triangles; then a leaf found meanwhile becomes
 // the postponed one.  Returns true when the ray's traversal is finished.
 template <typename R, typename B, typename SP>
-__device__ __forceinline__ bool trav_leaf(const MeshDev& m, const Ray<R, B>& r, uint32_t last, Trav<R, B>& t,
+__device__ __forceinline__ void trav_leaf(const MeshDev& m, const Ray<R, B>& r, uint32_t last, Trav<R, B>& t,
                                           SP stack, uint32_t& n_tris) {
   const uint32_t code = ~(uint32_t)t.leaf;
   const uint32_t first = code & 0xFFFFFFu, count = code >> 24;
@@ -902,7 +892,6 @@ __device__ __forceinline__ bool trav_leaf(const MeshDev& m, const Ray<R, B>& r, 
     t.leaf = t.cur;
     t.cur = trav_pop(t, stack);
   }
-  return t.leaf == 0 && t.cur == kDone;
 }
 
 // ------------------------------------- compressed wide BVH traversal
@@ -1746,6 +1735,8 @@ __global__ void __launch_bounds__(MINB > 0 ? 128 : 256, MINB > 0 ? MINB : (sizeo
   uint32_t it_q = 0;
 
   // lane's particle
+  // tdone: the ray is finished (binary trees: no postponed leaf and nothing to
+  // visit, which holds for lanes without a particle too)
   bool has = false, tdone = true;
   int qi = -1;
   uint32_t last = 0xFFFFFFFFu;
@@ -1756,6 +1747,7 @@ __global__ void __launch_bounds__(MINB > 0 ? 128 : 256, MINB > 0 ? MINB : (sizeo
   using TV = std::conditional_t<(W > 2), TravW<R>, Trav<R, B>>;
   using SE = std::conditional_t<(W > 2), uint2, StackE<B>>;
   TV tv{};
+  if constexpr (W == 2) tv.cur = kDone;  // nothing to do
   SE local_stack[W > 2 ? kMaxStackW : kMaxStack];
   constexpr bool kSplit = POOL && W == 2 && sizeof(R) == 4 && MINB > 0;
   __shared__ int2 s_stack[kSplit ? 4 * kSharedStack * 32 : 1];
@@ -1768,6 +1760,7 @@ __global__ void __launch_bounds__(MINB > 0 ? 128 : 256, MINB > 0 ? MINB : (sizeo
 
   for (;;) {
     // ---- 1. lanes whose ray is finished: re-emit, or finish the particle
+    if constexpr (W == 2) tdone = tv.leaf == 0 && tv.cur == kDone;
     if (has && tdone) {
       const QueryDev& q = a.queries[qi];
       const uint64_t pid = acc.pb & ((1ull << kSlotPidBits) - 1);
@@ -1999,27 +1992,25 @@ __global__ void __launch_bounds__(MINB > 0 ? 128 : 256, MINB > 0 ? MINB : (sizeo
       // without staged nodes, the shared-memory check leaves the node loop
       if (n_stage == 0) {
         for (;;) {
-          const unsigned searching = __ballot_sync(kFull, has && !tdone && tv.cur >= 0 && tv.leaf == 0);
+          const unsigned searching = __ballot_sync(kFull, tv.cur >= 0 && tv.leaf == 0);
           if (searching == 0u) break;
           // the last few lanes wait while as many others test their leaves: cylinder
           // sweep 98.3 -> 97.5 ms, hemisphere 7.38 -> 7.17, attitude sweep 204.5 -> 197.4
           // (6 lanes: 98.9, 7.14, 197.4; 8: 101.0, 7.21, 198.7)
-          if (__popc(searching) < 4 && __popc(__ballot_sync(kFull, has && !tdone && tv.leaf != 0)) >= 4) break;
-          if (has && !tdone && tv.cur >= 0)
-            trav_inner<false>(a.mesh, s_nodes, n_stage, ray, tv, stack, n_nodes, a.error);
+          if (__popc(searching) < 4 && __popc(__ballot_sync(kFull, tv.leaf != 0)) >= 4) break;
+          if (tv.cur >= 0)
+            trav_inner<false>(a.mesh, s_nodes, n_stage, ray, tv, stack, n_nodes);
         }
       } else {
-        while (__any_sync(kFull, has && !tdone && tv.cur >= 0 && tv.leaf == 0)) {
-          if (has && !tdone && tv.cur >= 0)
-            trav_inner<true>(a.mesh, s_nodes, n_stage, ray, tv, stack, n_nodes, a.error);
+        while (__any_sync(kFull, tv.cur >= 0 && tv.leaf == 0)) {
+          if (tv.cur >= 0)
+            trav_inner<true>(a.mesh, s_nodes, n_stage, ray, tv, stack, n_nodes);
         }
       }
-      if (has && !tdone) {
-        if (tv.leaf != 0) tdone = trav_leaf(a.mesh, ray, last, tv, stack, n_tris);
-        else if (tv.cur == kDone) tdone = true;
-      }
-      const unsigned fin = __ballot_sync(kFull, has && tdone);
-      const unsigned run = __ballot_sync(kFull, has && !tdone);
+      if (tv.leaf != 0) trav_leaf(a.mesh, ray, last, tv, stack, n_tris);
+      const bool ended = tv.leaf == 0 && tv.cur == kDone;  // also lanes without a particle
+      const unsigned fin = __ballot_sync(kFull, has && ended);
+      const unsigned run = __ballot_sync(kFull, !ended);
       if (run == 0u || (uint32_t)__popc(fin) >= a.refill_at) break;
     }
   }
