@@ -42,6 +42,7 @@ struct SetupBase {
 __global__ void __launch_bounds__(kSetupThreads)
     setup_kernel(QueryDev* qs, const __grid_constant__ SetupBase with, const double* dirs, const double* Svals, ItemDev* items,
                  const uint32_t* slots, AccStripe* acc, uint32_t acc_stride, const double* knots, RunWords* zero) {
+  cudaTriggerProgrammaticLaunchCompletion();  // see launch_after
   const QueryDev* base = with.given ? &with.q : nullptr;
   if (zero != nullptr && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < sizeof(RunWords) / 4)
     reinterpret_cast<uint32_t*>(zero)[threadIdx.x] = 0u;
@@ -347,6 +348,7 @@ __global__ void __launch_bounds__(128)
     finalize_kernel(const QueryDev* qs, const AccStripe* acc, uint32_t stride, uint32_t nq, const uint32_t* slots,
                     tpmc_result* out, const int* err, int* err_out) {
   const uint32_t i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31u;
+  cudaGridDependencySynchronize();  // every thread, before its first read: see launch_after
   if (err_out != nullptr && blockIdx.x == 0 && threadIdx.x == 0) *err_out = *err;
   if (i >= nq) return;
   const uint32_t qi = slots != nullptr ? slots[i] : i;
@@ -439,6 +441,30 @@ __global__ void panels_kernel(const QueryDev* q, const long long* panel, const d
 }  // namespace
 
 // ------------------------------------------------------------- launchers
+// A launch that may start once every block of the stream's previous kernel has
+// started (cudaTriggerProgrammaticLaunchCompletion in it; at its end otherwise), so
+// that its launch latency passes under that kernel.  Its threads wait in
+// cudaGridDependencySynchronize for that kernel's end, and its writes, before they
+// read what it wrote; as all of them do, the end of this kernel means the end of
+// that one, and a chain of these is as ordered as plain launches for what follows.
+// Waiting blocks hold only what the running ones left free.  A call of 4,096
+// particles on the 1,280-triangle sphere: 90 -> 86 us, eight attitudes of 20,000 on the
+// cylinder: 156 -> 152.  Not from the pool: those launches take milliseconds.
+template <typename... P, typename... A>
+cudaError_t launch_after(void (*f)(P...), uint32_t grid, uint32_t block, size_t smem, cudaStream_t stream, A... args) {
+  cudaLaunchAttribute overlap{};
+  overlap.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  overlap.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = dim3(grid);
+  c.blockDim = dim3(block);
+  c.dynamicSmemBytes = smem;
+  c.stream = stream;
+  c.attrs = &overlap;
+  c.numAttrs = 1;
+  return cudaLaunchKernelEx(&c, f, P(args)...);
+}
+
 cudaError_t launch_setup(QueryDev* d_queries, uint32_t nq, const QueryDev* h_base, const double* d_dirs,
                          const double* d_S, ItemDev* d_items, const uint32_t* d_slots, AccStripe* d_acc,
                          uint32_t acc_stride, const float* tables, RunWords* d_zero, cudaStream_t stream) {
@@ -530,16 +556,19 @@ cudaError_t launch_trace(const TraceArgs& args, uint32_t variant, const LaunchCf
   const TraceKernel f = pick_trace(variant, cfg.block, cfg.blocks_per_sm);
   cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  f<<<grid, cfg.block, smem, stream>>>(args);
-  return cudaGetLastError();
+  if (variant & kVariantPool) {
+    f<<<grid, cfg.block, smem, stream>>>(args);
+    return cudaGetLastError();
+  }
+  return launch_after(f, grid, cfg.block, smem, stream, args);
 }
 
 cudaError_t launch_finalize(const QueryDev* d_queries, const AccStripe* d_acc, uint32_t acc_stride, uint32_t nq,
                             const uint32_t* d_slots, tpmc_result* d_out, const int* d_err, int* err_out,
                             cudaStream_t stream) {
   if (nq == 0) return cudaSuccess;
-  finalize_kernel<<<(nq + 3) / 4, 128, 0, stream>>>(d_queries, d_acc, acc_stride, nq, d_slots, d_out, d_err, err_out);
-  return cudaGetLastError();
+  return launch_after(finalize_kernel, (nq + 3) / 4, 128, 0, stream, d_queries, d_acc, acc_stride, nq, d_slots, d_out,
+                      d_err, err_out);
 }
 
 cudaError_t launch_panels(const QueryDev* d_query, const long long* d_panel, const float4*, const double* frames64,

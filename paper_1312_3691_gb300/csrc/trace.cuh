@@ -162,13 +162,14 @@ __device__ __forceinline__ R latitude_pdf(R x, R S, R Dinv) {
   return (Fn<R>::exp(-Sx * Sx) + (R)kSqrtPiD * Sx * Fn<R>::erfc(-Sx)) * Dinv;
 }
 
-// Interpolated start from a table laid out in z = Phi^-1(u).
+// Interpolated start from a query's table laid out in z = Phi^-1(u).  Plain loads:
+// the set-up may write the table after the trace kernel has been launched.
 __device__ __forceinline__ float z_table_start(const float* tab, int n, float z, float z_lo, float z_step) {
   const float f = (z - z_lo) / z_step;
   float fl;
   const int j = min(max(floor_bits(f, fl), 0), n - 2);
   const float w = fminf(fmaxf(f - fminf(fmaxf(fl, 0.0f), (float)(n - 2)), 0.0f), 1.0f);
-  return (1.0f - w) * __ldg(&tab[j]) + w * __ldg(&tab[j + 1]);
+  return (1.0f - w) * tab[j] + w * tab[j + 1];
 }
 
 // Float latitude solve near a pole, in w = 1 - x (up) or w = 1 + x (down).
@@ -1305,12 +1306,13 @@ __device__ __forceinline__ void work_flush(AccStripe* acc, uint32_t stride, int 
   if (n_tris) atomicAdd(&A.tris, (unsigned long long)n_tris);
 }
 
-// Work index g -> item (binary search over item starts).
+// Work index g -> item (binary search over item starts).  Plain loads: the
+// set-up may write the items after this kernel has been launched.
 __device__ __forceinline__ uint32_t find_item(const ItemDev* items, uint32_t n_items, uint64_t g) {
   uint32_t lo = 0, hi = n_items;
   while (hi - lo > 1) {
     const uint32_t mid = (lo + hi) >> 1;
-    if (__ldg(&items[mid].g_begin) <= g) lo = mid; else hi = mid;
+    if (items[mid].g_begin <= g) lo = mid; else hi = mid;
   }
   return lo;
 }
@@ -1719,6 +1721,12 @@ __global__ void __launch_bounds__(MINB > 0 ? 128 : 256, MINB > 0 ? MINB : (sizeo
   }
   lane_reset(acc, -1);
   __syncthreads();
+  // The set-up may still run (its launch_after, kernels.cu): the mesh's arrays
+  // above are complete, queries, items, tables and sums only from here on.
+  if constexpr (!POOL) {
+    cudaTriggerProgrammaticLaunchCompletion();
+    cudaGridDependencySynchronize();
+  }
 
   const unsigned lane = threadIdx.x & 31u;
   const unsigned lt_mask = (1u << lane) - 1u;

@@ -93,3 +93,36 @@ def test_containment_at_its_limit(T, offset):
                     assert e.value.status == T.TPMC_EINVAL
     finally:
         T.tpmc_destroy(c)
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("N", [1, 33, 4096, 20_000])
+def test_calls_in_turn_read_their_own_set_up(T, precision, N):
+    """Short calls one after another on one context, each with its own speed ratio, direction and seed, so with tables,
+    items and sums that the next call's set-up writes over: each gives the bits it gives on a context of its own."""
+    xyz, tri = M.icosphere(2, 1.0)
+    base = dict(eps_diffuse=0.9, A_ref=math.pi, r_cv=1.5, max_bounces=8, precision=precision)
+    calls = [dict(**W.base_state(S=S), **base, dir=d, seed=int(10 * S))
+             for S, d in ((0.05, (0, 0, 1)), (50.0, (1, 0.2, 0)), (7.0, (-1, 2, 0.5)), (1.0, (0, -1, 0)))]
+    keys = ("sum_dv_q", "sum_rdv_q", "n_hits", "n_hit_particles", "n_particles", "CD", "CD_sigma", "gamma")
+    want = []
+    for kw in calls:
+        c = T.tpmc_create(0)
+        try:
+            mesh, p = T.tpmc_mesh_load(c, xyz, tri), T.make_params(**kw)
+            rs = T.tpmc_trace(c, mesh, p, N), T.tpmc_sweep(c, mesh, p, np.array([kw["dir"]], float), None, N)[0]
+            want.append([[r[k] for k in keys] for r in rs])
+        finally:
+            T.tpmc_destroy(c)
+    c = T.tpmc_create(0)
+    try:
+        mesh = T.tpmc_mesh_load(c, xyz, tri)
+        params = [T.make_params(**kw) for kw in calls]
+        for _ in range(25):
+            for p, kw, w in zip(params, calls, want):
+                r = T.tpmc_trace(c, mesh, p, N)
+                assert [r[k] for k in keys] == w[0]
+                r = T.tpmc_sweep_noalloc(c, mesh, p, np.array([kw["dir"]], float), None, N)[0]
+                assert [r[k] for k in keys] == w[1]
+    finally:
+        T.tpmc_destroy(c)
