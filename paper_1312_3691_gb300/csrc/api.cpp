@@ -283,12 +283,13 @@ void Ctx::destroy_pool(Pool& pool) {
 // a.counter: two counters.
 cudaError_t Ctx::trace_pool(Pool& pool, cudaStream_t stream, TraceArgs a, uint32_t variant, const LaunchCfg& cfg,
                             float area) {
-  // Rough rays first where at most a quarter of the particles is expected to
-  // meet the front (its mean projected area over the control volume's).  They
-  // cost 55 % of an exact seeding: the satellite (12 % pass) 6.74 -> 6.09 ms for
-  // 1e8 particles; the plate sweep (36 %) 33.7 -> 33.6, the cylinder's (55 %) 98.7
-  // -> 101.9, so those seed exactly at once.
-  a.prefilter = a.mesh.front_area < 0.25f * area ? 1u : 0u;
+  // Rough rays first where less than 45 % of the particles are expected to meet
+  // the front (its mean projected area over the control volume's).  They cost
+  // 55 % of an exact seeding and what passes is seeded exactly after them: the
+  // satellite (12 % pass) 6.74 -> 6.09 ms for 1e8 particles, the plate sweep
+  // (36 %) 32.7 -> 31.6; the cylinder's (55 %) would take 94.9 for 92.9, so it
+  // seeds exactly at once.
+  a.prefilter = a.mesh.front_area < 0.45f * area ? 1u : 0u;
   cudaError_t e = cudaSuccess;
   if (!pool.side) e = cudaStreamCreateWithFlags(&pool.side, cudaStreamNonBlocking);
   for (cudaEvent_t* ev : {&pool.fork, &pool.join, &pool.done})
