@@ -283,7 +283,7 @@ cudaError_t launch_finalize(const QueryDev* d_queries, const AccStripe* d_acc, u
 cudaError_t launch_panels(const QueryDev* d_query, const long long* d_panel, const float4* frames,
                           const double* frames64, uint32_t n_tri, double* d_pressure, double* d_shear,
                           cudaStream_t stream);
-constexpr uint32_t kTraceStaticSmem = 4224;  // the trace kernel's fixed shared memory (stacks, front, counts of misses), at most
+constexpr uint32_t kTraceStaticSmem = 384;  // the trace kernel's fixed shared memory (front, counts of misses), at most
 size_t trace_smem_bytes(const LaunchCfg& cfg, uint32_t n_nodes, uint32_t variant);
 int trace_max_blocks_per_sm(uint32_t variant, const LaunchCfg& cfg, uint32_t n_nodes);
 

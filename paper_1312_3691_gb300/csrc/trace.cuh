@@ -734,31 +734,12 @@ constexpr int kDone = (int)0x80000000;  // no valid leaf code: first + count wou
 
 // Traversal stack entry: a stacked child and its entry distance.  In float
 // the pair is one 8-byte local-memory access per push and per pop (two 4-byte
-// arrays took two).
+// arrays took two).  The pool kernel with its first four entries in shared memory
+// instead, and so a branch at each access and less L1: cylinder sweep 91.8 -> 92.7
+// ms, hemisphere 6.55 -> 6.59, moments 3.44 -> 3.48, attitude sweep 185.4 -> 186.8.
 template <typename R> struct StackE;
 template <> struct __align__(8) StackE<float> { int node; float t; };
 template <> struct __align__(16) StackE<double> { double t; int node; int pad; };
-// The pool kernel's stack: its first kSharedStack entries in shared memory, a
-// column of the warp's block for each lane (so lanes at different depths use
-// different banks), the rest in local memory.  Most pushes and pops of a lane
-// are within the first four, and they no longer miss the L1 or write lines of
-// the 90 MB that the grid's local stacks span back through the L2: cylinder
-// sweep 97.4 -> 96.4 ms, hemisphere 7.17 -> 7.00, attitude sweep 197.3 -> 195.7
-// (6 and 8 entries take the L1 as much as they save).
-constexpr int kSharedStack = 4;
-struct SplitStack {
-  int2* shared;
-  StackE<float>* local;
-};
-__device__ __forceinline__ void stack_put(SplitStack s, int i, int node, float t) {
-  if (i < kSharedStack) s.shared[i * 32] = make_int2(node, __float_as_int(t));
-  else *reinterpret_cast<int2*>(s.local + i) = make_int2(node, __float_as_int(t));
-}
-__device__ __forceinline__ void stack_get(SplitStack s, int i, int& node, float& t) {
-  const int2 v = i < kSharedStack ? s.shared[i * 32] : *reinterpret_cast<const int2*>(s.local + i);
-  node = v.x;
-  t = __int_as_float(v.y);
-}
 __device__ __forceinline__ void stack_put(StackE<float>* s, int i, int node, float t) {
   *reinterpret_cast<int2*>(s + i) = make_int2(node, __float_as_int(t));
 }
@@ -803,8 +784,8 @@ __device__ __forceinline__ void trav_begin(Trav<R, B>& t) {
 }
 
 // Next stacked candidate whose entry distance is still below the best hit.
-template <typename R, typename B, typename SP>
-__device__ __forceinline__ int trav_pop(Trav<R, B>& t, SP stack) {
+template <typename R, typename B>
+__device__ __forceinline__ int trav_pop(Trav<R, B>& t, StackE<B>* stack) {
   while (t.sp > 0) {
     --t.sp;
     int node;
@@ -818,9 +799,9 @@ __device__ __forceinline__ int trav_pop(Trav<R, B>& t, SP stack) {
 // One inner node: test both children, continue with the nearer hit child,
 // stack the farther one; the first leaf reached is postponed.  STAGE: nodes
 // below n_stage come from the copy in shared memory.
-template <bool STAGE, typename R, typename B, typename SP>
+template <bool STAGE, typename R, typename B>
 __device__ __forceinline__ void trav_inner(const MeshDev& m, const float4* __restrict__ s_nodes, uint32_t n_stage,
-                                           const Ray<R, B>& r, Trav<R, B>& t, SP stack,
+                                           const Ray<R, B>& r, Trav<R, B>& t, StackE<B>* stack,
                                            uint32_t& n_nodes) {
   ++n_nodes;
   float4 n0, n1;
@@ -862,18 +843,36 @@ __device__ __forceinline__ void trav_inner(const MeshDev& m, const float4* __res
     ++t.sp;
   }
   t.cur = second ? c1 : c0;
-  if (!h0 && !h1) t.cur = trav_pop(t, stack);
-  if (t.cur < 0 && t.cur != kDone && t.leaf == 0) {
+  // A leaf is postponed when none is; then, or when nothing was hit, the next
+  // candidate of the stack whose entry distance is still below the best hit.  One
+  // loop for both, which ends as each turn takes an entry off: two calls of
+  // trav_pop took the hemisphere 6.67 ms instead of 6.59, moments 3.51 and 3.49
+  // (branches and their barriers are a quarter of the trace kernel's instructions).
+  bool next = !h0 && !h1;
+  if (!next && t.cur < 0 && t.leaf == 0) {
     t.leaf = t.cur;
-    t.cur = trav_pop(t, stack);
+    next = true;
+  }
+  while (next) {
+    if (t.sp == 0) {
+      t.cur = kDone;
+      break;
+    }
+    --t.sp;
+    B te;
+    stack_get(stack, t.sp, t.cur, te);
+    if (te <= trav_cull(t)) {
+      next = t.cur < 0 && t.leaf == 0;
+      if (next) t.leaf = t.cur;
+    }
   }
 }
 
 // The postponed leaf: test its triangles; then a leaf found meanwhile becomes
 // the postponed one.  Returns true when the ray's traversal is finished.
-template <typename R, typename B, typename SP>
+template <typename R, typename B>
 __device__ __forceinline__ void trav_leaf(const MeshDev& m, const Ray<R, B>& r, uint32_t last, Trav<R, B>& t,
-                                          SP stack, uint32_t& n_tris) {
+                                          StackE<B>* stack, uint32_t& n_tris) {
   const uint32_t code = ~(uint32_t)t.leaf;
   const uint32_t first = code & 0xFFFFFFu, count = code >> 24;
   const Shear<R> sh = make_shear<R>(r.d);
@@ -1756,14 +1755,7 @@ __global__ void __launch_bounds__(MINB > 0 ? 128 : 256, MINB > 0 ? MINB : (sizeo
   using SE = std::conditional_t<(W > 2), uint2, StackE<B>>;
   TV tv{};
   if constexpr (W == 2) tv.cur = kDone;  // nothing to do
-  SE local_stack[W > 2 ? kMaxStackW : kMaxStack];
-  constexpr bool kSplit = POOL && W == 2 && sizeof(R) == 4 && MINB > 0;
-  __shared__ int2 s_stack[kSplit ? 4 * kSharedStack * 32 : 1];
-  std::conditional_t<kSplit, SplitStack, SE*> stack;
-  if constexpr (kSplit)
-    stack = SplitStack{s_stack + (threadIdx.x >> 5) * kSharedStack * 32 + (threadIdx.x & 31u), local_stack};
-  else
-    stack = local_stack;
+  SE stack[W > 2 ? kMaxStackW : kMaxStack];
   uint32_t n_nodes = 0, n_tris = 0;
 
   for (;;) {
