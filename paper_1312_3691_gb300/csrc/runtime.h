@@ -64,9 +64,9 @@ constexpr uint32_t kDefaultBvhWidth = 2;
 // FP32 launches of at least this many particles go through the pool.  Below, the
 // second launch and two tails cost more than the leaner kernels save.  One
 // attitude at S = 7, us through the pool / fused, at 2^22, 2^23 and 2^24
-// particles: plate 261/219, 363/356, 574/640; icosphere 1075/1189, 1966/2283,
-// 3769/4463; cylinder 717/705, 1169/1319, 2119/2493; hemisphere 3475/3769,
-// 6495/7152, 12500/13919; satellite 1001/929, 1316/1381, 1731/1928.
+// particles: plate 235/191, 337/328, 543/597; icosphere 1019/1082, 1865/2090,
+// 3559/4102; cylinder 674/630, 1108/1190, 1985/2271; hemisphere 3159/3432,
+// 5851/6536, 11259/12703; satellite 873/742, 1148/1207, 1470/1722.
 constexpr uint64_t kPoolMin = 1u << 23;
 // Particles of a batch, at most and at least (32 bytes each, two batches).
 constexpr uint64_t kPoolBatch = 1ull << 26, kPoolSmallest = 1ull << 20;
@@ -96,6 +96,7 @@ struct Ctx {
   tpmc_query_id next_query = 1;
   bool counters = false;
   bool manual_launch = false;
+  uint64_t pool_min = kPoolMin;  // lower while the tuner compares schedules (tune.cpp: measure)
   uint32_t bvh_leaf = 4;       // largest leaf of the BVHs built by later mesh loads
   uint32_t bvh_width = 0;      // children per node of later mesh loads (0: tuned or default)
   std::map<uint64_t, uint32_t> tuned_width;  // BVH width chosen by tpmc_tune per size class

@@ -53,13 +53,14 @@ void trial_dirs(const tpmc_params* p, double out[kTrialDirs * 3]) {
 // all, and the rate is the difference in particles over the difference in
 // time, so that the fixed costs of a launch (set-up, reduction, the tail of
 // its last warps) drop out and the choice holds for the long launches of
-// sweeps.  `used` receives the schedule as completed by Ctx::schedule.
+// sweeps.  Both go the way of the longer one, through the pool or not.  `used` receives the schedule as completed by Ctx::schedule.
 tpmc_status measure(Ctx* c, const MeshRec& m, const tpmc_params* params, uint64_t N_trial, const double* d_dirs,
                     const LaunchCfg& cfg, bool manual, Timer& tm, double* rate, LaunchCfg* used) {
   const bool had_manual = c->manual_launch;
   const LaunchCfg old_manual = c->manual;
   c->manual_launch = manual;
   c->manual = cfg;
+  if (N_trial >= kPoolMin) c->pool_min = 0;
   const uint64_t each[2] = {std::max<uint64_t>(1, N_trial / (4 * kTrialDirs)), std::max<uint64_t>(1, N_trial / kTrialDirs)};
   float ms[2] = {0.0f, 0.0f};
   tpmc_status st = TPMC_OK;
@@ -78,6 +79,7 @@ tpmc_status measure(Ctx* c, const MeshRec& m, const tpmc_params* params, uint64_
   }
   c->manual_launch = had_manual;
   c->manual = old_manual;
+  c->pool_min = kPoolMin;
   if (st != TPMC_OK) return st;
   if ((st = c->check_error_word()) != TPMC_OK) return st;
   const double dt = (double)ms[1] - (double)ms[0];
@@ -127,6 +129,14 @@ extern "C" tpmc_status tpmc_tune(tpmc_ctx* ctx, tpmc_mesh_id mesh, const tpmc_pa
   Timer tm;
   const uint32_t n_tri = m.dev.n_tri;
 
+  // Trials through the pool are four times as long, which takes the time that they
+  // took in one kernel: at 2^24 particles half the time is the tail of the longest
+  // paths, and a tail that shrinks with N reads as rate.  On the satellite such
+  // trials kept 4-wide nodes, and the attitude sweep ran at 1.14e10 particles/s
+  // where the untuned schedule gives 1.65e10.
+  const uint64_t N_long = std::min<uint64_t>(4 * N_trial, 1ull << 30);
+  const uint64_t N_short = params->precision == TPMC_FP32 && N_trial >= kPoolMin ? N_long : N_trial;
+
   // 1. BVH width, each layout with its untuned schedule
   uint32_t best_width = m.dev.width;
   {
@@ -147,7 +157,7 @@ extern "C" tpmc_status tpmc_tune(tpmc_ctx* ctx, tpmc_mesh_id mesh, const tpmc_pa
         run_on = &cand;
       }
       double rate = 0.0;
-      st = measure2(c, *run_on, params, N_trial, d_dirs, LaunchCfg(), false, tm, &rate, nullptr);
+      st = measure2(c, *run_on, params, N_short, d_dirs, LaunchCfg(), false, tm, &rate, nullptr);
       if (st != TPMC_OK) {
         if (run_on == &cand) c->release(cand.d_block);
         return st;
@@ -201,15 +211,14 @@ extern "C" tpmc_status tpmc_tune(tpmc_ctx* ctx, tpmc_mesh_id mesh, const tpmc_pa
   for (const LaunchCfg& cfg : cands) {
     double rate = 0.0;
     LaunchCfg used;
-    if ((st = measure2(c, m, params, N_trial, d_dirs, cfg, true, tm, &rate, &used)) != TPMC_OK) return st;
+    if ((st = measure2(c, m, params, N_short, d_dirs, cfg, true, tm, &rate, &used)) != TPMC_OK) return st;
     used.chunk = 0;
     scored.push_back({rate, used});
   }
-  // the three best and the untuned schedule again on a four times longer
-  // trial, so that a short trial's noise does not decide; the untuned
+  // the three best and the untuned schedule again on a trial of N_long,
+  // so that a short trial's noise does not decide; the untuned
   // schedule is the one to beat, by 1 %
   std::sort(scored.begin(), scored.end(), [](const auto& x, const auto& y) { return x.first > y.first; });
-  const uint64_t N_long = std::min<uint64_t>(4 * N_trial, 1ull << 30);
   {
     double r = 0.0;
     LaunchCfg used;
