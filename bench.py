@@ -55,8 +55,8 @@ BYTES_PER_TRI_TEST = 48      # three float4 vertices
 # source, its build flags and the BVH builder it was taken with (keyed by the
 # SHA-256 of trace.cuh, trace_w2.cu, kernels.cu, bvh.cpp and build.py, in that order).
 # Mean over the four bench groups of dram__bytes_read.sum + dram__bytes_write.sum
-# for one full-size launch (9.6e8 particles).
-TRACE_TRAFFIC = {"5b65220644608b79c040240ed0f05ff920b17b62b72549f59ddb14d9d7524451": 38_543_872}
+# over the seeding and trace launches of one full-size call (9.6e8 particles).
+TRACE_TRAFFIC = {"4316ee444d768ede4a5a2180fe36f8f5a3cbd9e77383d7a9ae8ac9ebd93a9cea": 25_501_210_240}
 
 
 def kernel_source_hash() -> str:
@@ -901,7 +901,7 @@ def run_ours(args):
 
 def run_profile_launch(args):
     """One warm-up and one measured sweep launch of one group of the workload at a
-    reduced particle count, for profiler captures (ncu -k regex:trace_kernel -s 1 -c 1)."""
+    reduced particle count, for profiler captures (ncu -k "regex:(seed|trace)_kernel": a pair per batch of 2^26)."""
     import torch
 
     from paper_1312_3691_gb300 import tpmc as T

@@ -34,7 +34,7 @@ struct NoAllocArea {
 };
 static_assert(kNoAllocMaxQueries <= kPinnedItems, "inputs and results use the context's pinned memory");
 
-// Fixed scratch of tpmc_sweep_noalloc (about 100 KB).
+// Fixed scratch of tpmc_sweep_noalloc (about 150 KB).
 static __device__ __align__(256) unsigned char g_noalloc_scratch[sizeof(NoAllocArea)];
 
 constexpr int kMaxDevices = 64;

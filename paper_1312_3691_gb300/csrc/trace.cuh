@@ -1526,14 +1526,14 @@ __device__ __forceinline__ bool may_hit(const QueryDev& q, const TraceArgs& a, c
 // temporaries and the queue's state cost the traversal loop its registers (84
 // bytes of spills at 64, none now at 56), and warps of one SM in different
 // phases evicted each other's instructions (no_instruction was 1.5 to 3.7 of the
-// stall cycles per issue, now 0.3).  Here every lane seeds, 750 instructions a
-// particle at 85 % of the issue slots: 3.9e10 particles/s, where the fused
-// kernel on an empty mesh reaches 3.2e10.
+// stall cycles per issue, now 0.3).  Here every lane seeds, 745 instructions a
+// particle at 85 % of the issue slots, which bound it: 4.1e10 particles/s, where
+// the fused kernel on an empty mesh reaches 3.2e10.
 //
 // PRE: a rough ray (may_hit) decides first, and only the particles that it lets
 // through, gathered in shared memory until they fill a warp, are seeded exactly.
-// The host takes it when it expects that few pass (Ctx::trace_pool): 7.3e10
-// particles/s when none does.
+// The host takes it when it expects less than 45 % to pass (Ctx::trace_pool):
+// 7.4e10 particles/s when none does.
 template <int W, typename R, bool PRE>
 __global__ void __launch_bounds__(128, 8) seed_kernel(const __grid_constant__ TraceArgs a) {
   __shared__ __align__(16) float s_front[kMaxFront * 8];
@@ -1681,6 +1681,11 @@ __device__ __noinline__ unsigned seed_into(const TraceArgs& a, uint32_t qi, uint
 // Lanes then trace in rounds of resumable traversal steps; a round ends when
 // refill_at lanes have finished their rays, and those lanes re-emit (next
 // bounce) or finish their particle and take the next one from the queue.
+// What bounds it, from the pool: on the cylinder sweep the issue slots (79 % full
+// at 35 warps per SM; a round is 15 node steps at 22 lanes, two leaf phases at 15
+// and one hit phase at 23), on concave meshes the latency of node loads as well
+// (the hemisphere 17 lanes a node step).  Occupancy decides: 8 and 10 blocks per SM
+// (64 and 48 registers) take the cylinder sweep 95.5 and 92.7 ms, 9 blocks 91.7.
 // MINB > 0: a register-capped instantiation for 128-thread blocks with at
 // least MINB resident blocks per SM (more warps to hide latency, at the cost
 // of spills inside the out-of-line seeding).  MINB = 0: 256-thread blocks,
