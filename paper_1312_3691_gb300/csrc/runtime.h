@@ -70,6 +70,7 @@ constexpr uint32_t kDefaultBvhWidth = 2;
 constexpr uint64_t kPoolMin = 1u << 23;
 // Particles of a batch, at most and at least (32 bytes each, two batches).
 constexpr uint64_t kPoolBatch = 1ull << 26, kPoolSmallest = 1ull << 20;
+constexpr uint32_t kPoolSegment = 2048;  // work indices of a segment, at most (a batch is a multiple)
 
 float cv_area(const QueryDev& q);
 tpmc_status fill_query(const MeshRec& m, const tpmc_params* p, uint64_t N, QueryDev* q);

@@ -1851,7 +1851,7 @@ __global__ void __launch_bounds__(MINB > 0 ? 128 : 256, MINB > 0 ? MINB : (sizeo
         while (q_count == 0 && !drained) {  // the next segment, of a run of them
           // A run of segments at a time, as many as would let every warp fetch four
           // more times (64 at most): with single segments a warp met another query
-          // at every fetch of an attitude sweep (its queries hold 2,000 segments,
+          // at every fetch of an attitude sweep (its queries held 2,000 segments,
           // the grid 5,472 warps), which took 306 ms instead of 239.
           if (seg_left == 0) {
             unsigned sg = 0;

@@ -66,6 +66,25 @@ def test_pool_gives_the_fused_sums(T, K, N, width, gsi):
         T.tpmc_destroy(c)
 
 
+# lengths of segments, from 64 work indices on: powers of two up to 2,048 behind rough rays (the satellite), 1,024
+# without (the cylinder in a tight control volume); ragged ends in each
+@pytest.mark.parametrize("N", [(1 << 23) + 2047, 12_000_001, 23_000_003, 47_000_033, (1 << 26) + 1])
+@pytest.mark.parametrize("body", ["satellite", "cylinder"])
+def test_segment_lengths(T, body, N):
+    xyz, tri = M.satellite(3_000) if body == "satellite" else M.cylinder(0.5, 2.0, 24, 5)
+    c = T.tpmc_create(0)
+    try:
+        mesh = T.tpmc_mesh_load(c, xyz, tri)
+        p = _base(T, r_cv=1.01 * float(np.sqrt((xyz ** 2).sum(axis=1).max())))
+        pooled = T.tpmc_trace(c, mesh, p, N)
+        T.tpmc_set_counters(c, True)
+        fused = T.tpmc_trace(c, mesh, p, N)
+        assert pooled["n_particles"] == N
+        assert {k: pooled[k] for k in KEYS} == {k: fused[k] for k in KEYS}
+    finally:
+        T.tpmc_destroy(c)
+
+
 @pytest.mark.parametrize("cv", ["tight", "wide", "box", "maxwell box"])
 @pytest.mark.parametrize("body", ["satellite", "cylinder", "plate"])
 def test_rough_rays_drop_no_particle_that_hits(T, body, cv):
