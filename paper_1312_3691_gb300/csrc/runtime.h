@@ -61,13 +61,16 @@ constexpr size_t kPinnedBytes = 256 + kPinnedItems * (sizeof(tpmc_result) + 4 * 
 // BVH width of mesh loads that neither tpmc_set_launch nor tpmc_tune decided.
 constexpr uint32_t kDefaultBvhWidth = 2;
 
-// FP32 launches of at least this many particles go through the pool.  Below, the
-// second launch and two tails cost more than the leaner kernels save.  One
-// attitude at S = 7, us through the pool / fused, at 2^22, 2^23 and 2^24
-// particles: plate 235/191, 337/328, 543/597; icosphere 1019/1082, 1865/2090,
-// 3559/4102; cylinder 674/630, 1108/1190, 1985/2271; hemisphere 3159/3432,
-// 5851/6536, 11259/12703; satellite 873/742, 1148/1207, 1470/1722.
-constexpr uint64_t kPoolMin = 1u << 23;
+// FP32 launches of at least this many particles go through the pool, those of one
+// query from kPoolMinOne on.  Below, the second launch and two tails cost more
+// than the leaner kernels save.  us through the pool / fused at S = 7: one query of
+// 2^22 and 2^23 particles, then 16 and 512 queries of 2^22 in all:
+//   plate       153/188    242/325     256/335    1685/1834
+//   icosphere   963/1053   1771/2041   1076/1376  2555/2950
+//   cylinder    656/617    1079/1173   711/832    2142/2318
+//   hemisphere  3062/3322  5746/6273   1832/2176  3309/3638
+//   satellite   660/717    1029/1179   787/956    2359/2538
+constexpr uint64_t kPoolMin = 1u << 22, kPoolMinOne = 6u << 20;
 // Particles of a batch, at most and at least (32 bytes each, two batches).
 constexpr uint64_t kPoolBatch = 1ull << 26, kPoolSmallest = 1ull << 20;
 constexpr uint32_t kPoolSegment = 2048;  // work indices of a segment, at most (a batch is a multiple)
@@ -97,7 +100,7 @@ struct Ctx {
   tpmc_query_id next_query = 1;
   bool counters = false;
   bool manual_launch = false;
-  uint64_t pool_min = kPoolMin;  // lower while the tuner compares schedules (tune.cpp: measure)
+  bool pool_always = false;    // while the tuner times both sizes of a long trial (tune.cpp: measure)
   uint32_t bvh_leaf = 4;       // largest leaf of the BVHs built by later mesh loads
   uint32_t bvh_width = 0;      // children per node of later mesh loads (0: tuned or default)
   std::map<uint64_t, uint32_t> tuned_width;  // BVH width chosen by tpmc_tune per size class

@@ -53,6 +53,7 @@ constexpr int kInFlight = 2;                     // steps enqueued ahead of the 
 constexpr int kMaxGroups = 64;                   // trace launches per step
 constexpr int kGroupStreams = 4;                 // streams the groups of a step run on
 constexpr uint64_t kServePoolBatch = 1ull << 25;  // particles of a pool batch (a pool for each step in flight)
+constexpr uint64_t kServePoolMin = 1u << 23;       // groups from here on: smaller ones run beside each other anyway
 }  // namespace
 
 struct Request {
@@ -275,7 +276,7 @@ bool enqueue_step(ServeState* s, int b, int prev, const std::vector<Request*>& c
     // goes through the step's pool: a burst of 32 queries of 1e5 to 1e8 particles
     // on three meshes 77.8 -> 63.0 ms
     bool pooled = false;
-    if (e == cudaSuccess && g >= kPoolMin && (groups[gi].first.second & 1u) == TPMC_FP32 && a.count_work == 0u) {
+    if (e == cudaSuccess && g >= kServePoolMin && (groups[gi].first.second & 1u) == TPMC_FP32 && a.count_work == 0u) {
       std::lock_guard<std::recursive_mutex> ck(c->mu);  // until the pool's `done` is recorded
       if (c->grow_pool(B.pool, g, kServePoolBatch)) {
         pooled = true;

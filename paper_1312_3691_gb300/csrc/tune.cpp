@@ -60,7 +60,7 @@ tpmc_status measure(Ctx* c, const MeshRec& m, const tpmc_params* params, uint64_
   const LaunchCfg old_manual = c->manual;
   c->manual_launch = manual;
   c->manual = cfg;
-  if (N_trial >= kPoolMin) c->pool_min = 0;
+  c->pool_always = N_trial >= kPoolMin;
   const uint64_t each[2] = {std::max<uint64_t>(1, N_trial / (4 * kTrialDirs)), std::max<uint64_t>(1, N_trial / kTrialDirs)};
   float ms[2] = {0.0f, 0.0f};
   tpmc_status st = TPMC_OK;
@@ -79,7 +79,7 @@ tpmc_status measure(Ctx* c, const MeshRec& m, const tpmc_params* params, uint64_
   }
   c->manual_launch = had_manual;
   c->manual = old_manual;
-  c->pool_min = kPoolMin;
+  c->pool_always = false;
   if (st != TPMC_OK) return st;
   if ((st = c->check_error_word()) != TPMC_OK) return st;
   const double dt = (double)ms[1] - (double)ms[0];
