@@ -27,15 +27,17 @@ tpmc_status cuda_fail(cudaError_t e, const char* where) {
 }
 
 // ------------------------------------------------------------ allocation
-tpmc_status Ctx::alloc(void** p, size_t bytes, const char* what) {
+// take_pools: the pools of seeded particles give way when their memory is what is
+// missing, which waits for the launches that use them.
+tpmc_status Ctx::alloc(void** p, size_t bytes, const char* what, bool take_pools) {
   *p = nullptr;
   if (bytes == 0) return TPMC_OK;
-  if (used + bytes > budget) release_pools();
+  if (take_pools && used + bytes > budget && used + bytes <= budget + pooled()) release_pools();
   if (used + bytes > budget)
     return fail(TPMC_ENOMEM, std::string(what) + ": memory budget exceeded (" + std::to_string(used + bytes) +
                                  " > " + std::to_string(budget) + " bytes)");
   cudaError_t e = cudaMalloc(p, bytes);
-  if (e != cudaSuccess && release_pools()) {
+  if (e != cudaSuccess && take_pools && release_pools()) {
     cudaGetLastError();
     e = cudaMalloc(p, bytes);
   }
@@ -240,7 +242,7 @@ bool Ctx::grow_pool(Pool& pool, uint64_t total, uint64_t max_batch) {
   if (pool.cap >= need) return true;
   release_pool(pool);
   const std::string last = g_last_error;
-  if (alloc(&pool.ptr, need, "seeded particles") == TPMC_OK) {
+  if (alloc(&pool.ptr, need, "seeded particles", false) == TPMC_OK) {
     pool.cap = need;
     return true;
   }
@@ -257,7 +259,7 @@ void Ctx::release_pool(Pool& pool) {
   pool.cap = 0;
 }
 
-// Pools give way to everything else that needs the memory.
+// Pools give way to everything else that needs the memory (Ctx::alloc, where it helps).
 bool Ctx::release_pools() {
   bool any = false;
   for (Pool* p : pools) {
@@ -265,6 +267,12 @@ bool Ctx::release_pools() {
     release_pool(*p);
   }
   return any;
+}
+
+size_t Ctx::pooled() const {
+  size_t n = 0;
+  for (const Pool* p : pools) n += p->cap;
+  return n;
 }
 
 void Ctx::destroy_pool(Pool& pool) {

@@ -44,7 +44,8 @@ struct Scratch {
 
 // Seeded particles of a launch's batches (Ctx::grow_pool, Ctx::trace_pool), the
 // second stream of the launch and where it leaves and rejoins the first.  Freed
-// when another allocation needs the room, after `done`.
+// when another allocation needs the room, after `done` (the serving loop, whose
+// locks nobody should wait for, does so between its steps: give_back_pools).
 struct Pool {
   void* ptr = nullptr;
   size_t cap = 0;
@@ -121,7 +122,7 @@ struct Ctx {
   uint32_t width_for(uint32_t n_tri) const;
   tpmc_status upload_mesh(const double* xyz, uint32_t n_vert, const uint32_t* tri, uint32_t n_tri, uint32_t width,
                           MeshRec* out);
-  tpmc_status alloc(void** p, size_t bytes, const char* what);
+  tpmc_status alloc(void** p, size_t bytes, const char* what, bool take_pools = true);
   void release(void* p);
   tpmc_status grow(Scratch& s, size_t bytes, const char* what);
   LaunchCfg schedule(const MeshRec& m, uint32_t variant, uint64_t total);  // variant: see trace_variant
@@ -130,6 +131,7 @@ struct Ctx {
   bool grow_pool(Pool& pool, uint64_t total, uint64_t max_batch);
   void release_pool(Pool& pool);
   bool release_pools();
+  size_t pooled() const;
   void destroy_pool(Pool& pool);
   cudaError_t trace_pool(Pool& pool, cudaStream_t stream, TraceArgs a, uint32_t variant, const LaunchCfg& cfg, float area);
   tpmc_status check_error_word();

@@ -92,6 +92,7 @@ struct StepBuf {
   cudaEvent_t ready = nullptr;                   // set-up done
   cudaEvent_t traces_done = nullptr;             // every trace launch of the step done
   Pool pool;                                     // of the step's large group
+  bool pooled = false;                           // the step in flight uses it
   std::vector<Request*> members, finishing;
 };
 
@@ -102,6 +103,8 @@ struct ServeState {
   std::condition_variable cv_work, cv_done;
   bool stop = false;
   bool mem_wait = false;       // queued queries wait for device memory to be released
+  bool want_pools = false;     // a queued query waits for the memory of pools
+  bool no_pools = false;       // steps take no pool (loop thread only; see give_back_pools)
   std::deque<Request*> queue;
   std::map<tpmc_query_id, Request*> all;
   std::vector<Request*> slots;
@@ -118,12 +121,16 @@ namespace {
 
 // Admits queued requests into free slots (caller holds s->m), in arrival
 // order.  A request whose panel buffer does not fit now stays queued while
-// memory may still be released (queries in flight, or panel loads not yet
+// memory may still be released (pools, queries in flight, or panel loads not yet
 // read by tpmc_panels), and the requests behind it are admitted meanwhile; it
-// fails with ENOMEM only when nothing can free memory.
+// fails with ENOMEM only when nothing can free memory.  Pools are not freed here:
+// a step in flight may use them, and with both locks held tpmc_submit and
+// tpmc_poll would wait for its end as well (0.6 s behind a query of 1.2e10
+// particles).
 void admit(ServeState* s) {
   Ctx* c = s->ctx;
   s->mem_wait = false;
+  s->want_pools = false;
   for (auto qit = s->queue.begin(); qit != s->queue.end();) {
     Request* r = *qit;
     int slot = -1;
@@ -131,8 +138,12 @@ void admit(ServeState* s) {
     if (slot < 0) return;
     if (r->want_panels && r->n_tri > 0) {
       std::lock_guard<std::recursive_mutex> ck(c->mu);
-      if (c->alloc(&r->d_panel, (size_t)r->n_tri * 3 * sizeof(long long), "serving panel loads") != TPMC_OK) {
-        bool may_free = !s->inflight.empty() || !c->panels.empty();
+      const size_t bytes = (size_t)r->n_tri * 3 * sizeof(long long);
+      if (c->alloc(&r->d_panel, bytes, "serving panel loads", false) != TPMC_OK) {
+        const size_t pooled = c->pooled();
+        const bool behind_pools = pooled > 0 && c->used + bytes <= c->budget + pooled;
+        s->want_pools = s->want_pools || behind_pools;
+        bool may_free = behind_pools || !s->inflight.empty() || !c->panels.empty();
         for (Request* a : s->slots) may_free = may_free || a;
         if (may_free) {  // wait for memory; later queries may still fit
           s->mem_wait = true;
@@ -156,6 +167,45 @@ void admit(ServeState* s) {
   }
 }
 
+// Frees the pools for queued queries that wait for their memory (loop thread, no
+// lock held): freeing waits for the device, so only once no step in flight uses a
+// pool, and the locks are taken only to let go of the pools and to count them off.
+// Whoever submits or polls meanwhile does not wait.  The steps after it do without
+// pools: a context that had to give them back is short of memory, and every step
+// would take gigabytes that the next such query has to wait for again.
+void give_back_pools(ServeState* s) {
+  Ctx* c = s->ctx;
+  s->no_pools = true;
+  for (int b : s->inflight)
+    if (s->buf[b].pooled) return;
+  std::vector<void*> gone;
+  size_t bytes = 0;
+  {
+    std::lock_guard<std::recursive_mutex> ck(c->mu);
+    for (Pool* p : c->pools) {
+      if (!p->ptr) continue;
+      if (p->done && cudaEventQuery(p->done) != cudaSuccess) {  // a direct call's, still running
+        cudaGetLastError();
+        continue;
+      }
+      gone.push_back(p->ptr);
+      bytes += p->cap;
+      c->sizes.erase(p->ptr);
+      p->ptr = nullptr;
+      p->cap = 0;
+    }
+  }
+  for (void* p : gone) cudaFree(p);
+  if (gone.empty()) {
+    std::this_thread::sleep_for(std::chrono::microseconds(200));
+  } else {
+    std::lock_guard<std::recursive_mutex> ck(c->mu);
+    c->used -= bytes;
+  }
+  std::lock_guard<std::mutex> lk(s->m);
+  s->mem_wait = false;  // those queries are admitted next, or wait again
+}
+
 // Builds and enqueues one step in buffer b (caller does not hold s->m).
 // Returns false when there was nothing to run.
 bool enqueue_step(ServeState* s, int b, int prev, const std::vector<Request*>& cand, cudaError_t& e) {
@@ -163,6 +213,7 @@ bool enqueue_step(ServeState* s, int b, int prev, const std::vector<Request*>& c
   StepBuf& B = s->buf[b];
   B.members.clear();
   B.finishing.clear();
+  B.pooled = false;
   // Shortest remaining work first, aged: a query's key is its remaining work
   // in GPU time (at a nominal rate) minus kAging times the time it has
   // waited, so small queries overtake young large ones, and a large query that
@@ -276,10 +327,11 @@ bool enqueue_step(ServeState* s, int b, int prev, const std::vector<Request*>& c
     // goes through the step's pool: a burst of 32 queries of 1e5 to 1e8 particles
     // on three meshes 77.8 -> 63.0 ms
     bool pooled = false;
-    if (e == cudaSuccess && g >= kServePoolMin && (groups[gi].first.second & 1u) == TPMC_FP32 && a.count_work == 0u) {
+    if (e == cudaSuccess && !s->no_pools && g >= kServePoolMin && (groups[gi].first.second & 1u) == TPMC_FP32 &&
+        a.count_work == 0u) {
       std::lock_guard<std::recursive_mutex> ck(c->mu);  // until the pool's `done` is recorded
       if (c->grow_pool(B.pool, g, kServePoolBatch)) {
-        pooled = true;
+        pooled = B.pooled = true;
         const uint32_t variant = groups[gi].first.second | kVariantPool;
         const LaunchCfg pcfg = c->schedule(c->meshes.at(groups[gi].first.first), variant, g);
         a.smem_nodes = pcfg.smem_nodes;
@@ -379,6 +431,7 @@ void loop(ServeState* s) {
   std::vector<Request*> cand;
   for (;;) {
     int free_buf = -1;
+    bool give = false;
     {
       std::unique_lock<std::mutex> lk(s->m);
       auto has_work = [&] {
@@ -387,10 +440,11 @@ void loop(ServeState* s) {
         return false;
       };
       s->cv_work.wait(lk, [&] {
-        return s->stop || !s->inflight.empty() || (!s->queue.empty() && !s->mem_wait) || has_work();
+        return s->stop || !s->inflight.empty() || s->want_pools || (!s->queue.empty() && !s->mem_wait) || has_work();
       });
       if (s->stop) break;
       admit(s);
+      give = s->want_pools;
       cand.clear();
       for (Request* r : s->slots)
         if (r && !r->done && r->next_pid < r->N) cand.push_back(r);
@@ -399,6 +453,7 @@ void loop(ServeState* s) {
           if (std::find(s->inflight.begin(), s->inflight.end(), b) == s->inflight.end()) { free_buf = b; break; }
       }
     }
+    if (give) give_back_pools(s);
     cudaError_t e = cudaSuccess;
     if (free_buf >= 0) {
       // inflight is changed only by this thread, so it can be read here unlocked

@@ -1,0 +1,78 @@
+"""Pools of seeded particles and the memory around them: who waits for it, how often it is taken, on the GPU."""
+import time
+
+import pytest
+
+from tpmc_inputs import meshes as M
+from tpmc_inputs import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+KEYS = ("sum_dv_q", "sum_rdv_q", "n_particles", "n_hits", "n_hit_particles", "n_truncated", "CD_sigma", "status")
+
+
+@pytest.fixture(scope="module")
+def T():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1312_3691_gb300.build import build
+
+    build()
+    from paper_1312_3691_gb300 import tpmc
+
+    return tpmc
+
+
+def _base(T, **kw):
+    return T.make_params(**{**W.base_state(S=7.0), "dir": (0.3, -0.2, 1.0), "eps_diffuse": 0.9, "A_ref": 1.0,
+                            "max_bounces": 64, "seed": 7, **kw})
+
+
+def _room(T, c):
+    i = T.tpmc_memory_info(c)
+    return i["budget"] - i["used"]
+
+
+def test_panel_query_waits_for_pool_memory_and_nobody_waits_with_it(T):
+    """A served query whose panel loads find the budget taken by the pools of a running step is left queued until that
+    step is over; submitting and polling (without a time-out) go on meanwhile, and the query is served in the end."""
+    xyz, tri = M.satellite(60_000)
+    budget = 4 << 30
+    c = T.tpmc_create(0, budget)
+    try:
+        mesh = T.tpmc_mesh_load(c, xyz, tri)
+        for _ in range(2):  # the pools of both steps in flight
+            for i in [T.tpmc_submit(c, mesh, _base(T), 1 << 24) for _ in range(2)]:
+                T.tpmc_poll(c, i)
+        p = _base(T, want_panels=True, stream_id=3)
+        alone = T.tpmc_trace(c, mesh, p, 1000)
+        panels = T.tpmc_panel_sums(c, alone["query_id"], len(tri))
+        while _room(T, c) >= 24 * len(tri):  # panel loads nobody reads fill the rest
+            T.tpmc_trace(c, mesh, p, 1000)
+        t0 = time.perf_counter()
+        # two steps in flight: queries are admitted again when the first is over, while the large one runs
+        first, big = T.tpmc_submit(c, mesh, _base(T), 1_000_000_000), T.tpmc_submit(c, mesh, _base(T), 12_000_000_000)
+        time.sleep(0.02)
+        longest, waiting = 0.0, []
+        while True:
+            a = time.perf_counter()
+            if len(waiting) < 4:
+                waiting.append(T.tpmc_submit(c, mesh, p, 1000))
+            done = T.tpmc_poll(c, big, 0)
+            longest = max(longest, time.perf_counter() - a)
+            if done is not None:
+                break
+            time.sleep(0.002)
+        assert time.perf_counter() - t0 > 0.4  # the large query ran for long enough to tell
+        assert longest < 0.1, longest
+        assert T.tpmc_poll(c, first)["n_particles"] == 1_000_000_000
+        for i in waiting:
+            r = T.tpmc_poll(c, i)
+            assert [r[k] for k in KEYS] == [alone[k] for k in KEYS]
+            assert (T.tpmc_panel_sums(c, i, len(tri)) == panels).all()
+        assert T.tpmc_memory_info(c)["used"] <= budget
+        again = T.tpmc_submit(c, mesh, _base(T), (1 << 23) + 5)  # large queries are served as before
+        assert T.tpmc_poll(c, again)["n_particles"] == (1 << 23) + 5
+    finally:
+        T.tpmc_destroy(c)
