@@ -215,11 +215,6 @@ LaunchCfg Ctx::schedule(const MeshRec& m, uint32_t variant, uint64_t total) {
   return cfg;
 }
 
-// Entries for `batch` particles (a multiple of kPoolSegment) and a count for each segment of 32 or more.
-static size_t pool_bytes(uint64_t batch) {
-  return (size_t)batch * kPoolEntryBytes + (size_t)(batch / 32) * sizeof(uint32_t) + 256;
-}
-
 // Mean projected area over pi, m^2, of a query's control volume.
 float cv_area(const QueryDev& q) {
   if (q.cv_kind == TPMC_CV_SPHERE) return (float)(q.r_cv * q.r_cv);
@@ -228,17 +223,13 @@ float cv_area(const QueryDev& q) {
 }
 
 // A pool for launches of `total` particles: twice the entries of a batch (at most
-// max_batch) and a count for each of its segments.  It takes at most half of the
-// memory the context's budget leaves and halves the batch until that holds; false
-// when less than a small batch fits (the launch then seeds inside the trace kernel).
+// max_batch) and a count for each of its segments, in the memory the context's
+// budget leaves (pool_batch); false when it has no room (the launch then seeds
+// inside the trace kernel).
 bool Ctx::grow_pool(Pool& pool, uint64_t total, uint64_t max_batch) {
-  const size_t left = budget - std::min(budget, used - pool.cap);
-  // whole segments, so that a launch no longer than a batch is one batch
-  auto whole = [](uint64_t n) { return (n + kPoolSegment - 1) / kPoolSegment * kPoolSegment; };
-  uint64_t batch = std::min<uint64_t>(max_batch, whole(total));
-  while (batch > kPoolSmallest && 2 * pool_bytes(batch) > left / 2) batch = whole(batch / 2);
+  const uint64_t batch = pool_batch(total, max_batch, budget - std::min(budget, used - pool.cap));
+  if (batch == 0) return false;
   const size_t need = 2 * pool_bytes(batch);
-  if (need > left / 2) return false;
   if (pool.cap >= need) return true;
   release_pool(pool);
   const std::string last = g_last_error;

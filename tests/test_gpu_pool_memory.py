@@ -76,3 +76,33 @@ def test_panel_query_waits_for_pool_memory_and_nobody_waits_with_it(T):
         assert T.tpmc_poll(c, again)["n_particles"] == (1 << 23) + 5
     finally:
         T.tpmc_destroy(c)
+
+
+def test_rising_counts_take_a_pool_for_each_power_of_two(T):
+    """Forty calls, each of 2^20 particles more than the last: the pool is taken for 2^24, 2^25 and 2^26 particles."""
+    c = T.tpmc_create(0)
+    try:
+        mesh = T.tpmc_mesh_load(c, *M.plate(1.0))
+        T.tpmc_trace(c, mesh, _base(T), 1000)
+        before = T.tpmc_memory_info(c)["n_allocs"]
+        for k in range(40):
+            N = (1 << 24) - 5 + (k << 20)
+            assert T.tpmc_trace(c, mesh, _base(T), N)["n_particles"] == N
+        assert T.tpmc_memory_info(c)["n_allocs"] - before <= 3
+    finally:
+        T.tpmc_destroy(c)
+
+
+def test_serving_takes_a_pool_for_each_step_in_flight_once(T):
+    """Large queries of rising size, served smallest first: one allocation for each of the two steps."""
+    c = T.tpmc_create(0)
+    try:
+        mesh = T.tpmc_mesh_load(c, *M.plate(1.0))
+        T.tpmc_poll(c, T.tpmc_submit(c, mesh, _base(T), 1000))
+        before = T.tpmc_memory_info(c)["n_allocs"]
+        sizes = [(1 << 23) + 7 + (k << 21) for k in range(12)]
+        ids = [T.tpmc_submit(c, mesh, _base(T), N) for N in sizes]
+        assert [T.tpmc_poll(c, i)["n_particles"] for i in ids] == sizes
+        assert T.tpmc_memory_info(c)["n_allocs"] - before <= 2
+    finally:
+        T.tpmc_destroy(c)
