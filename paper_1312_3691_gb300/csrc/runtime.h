@@ -72,8 +72,16 @@ constexpr uint32_t kDefaultBvhWidth = 2;
 //   hemisphere  3062/3322  5746/6273   1832/2176  3309/3638
 //   satellite   660/717    1029/1179   787/956    2359/2538
 constexpr uint64_t kPoolMin = 1u << 22, kPoolMinOne = 6u << 20;
-// Particles of a batch, at most and at least (32 bytes each, two batches).
-constexpr uint64_t kPoolBatch = 1ull << 26, kPoolSmallest = 1ull << 20;
+// Particles of a batch, at most and, in a launch of several, at least (32 bytes
+// each, two batches).  Every batch has a tail of its own, the fused launch one for
+// all.  ms for 1e8 particles of one query and for 96 queries of 1e6, fused, then
+// in batches of 2^20, 2^22, 2^23 and 2^26:
+//   plate       5.1 4.8    6.5 5.3    4.7 3.7    4.4 3.4    4.2 3.2
+//   icosphere   22.6 24.0  21.8 22.8  19.3 20.4  18.4 19.3  18.0 18.6
+//   cylinder    12.1 13.6  19.3 16.3  11.7 13.0  10.7 11.3  9.6 10.2
+//   hemisphere  71.1 31.2  79.6 40.1  65.8 31.2  63.0 28.2  61.4 27.6
+//   satellite   7.3 9.7    23.5 26.8  9.4 11.5   6.9 8.7    5.2 6.2
+constexpr uint64_t kPoolBatch = 1ull << 26, kPoolSmallest = 1ull << 23;
 constexpr uint32_t kPoolSegment = 2048;  // work indices of a segment, at most (a batch is a multiple)
 
 // Bytes of half a pool: entries for `batch` particles (a multiple of kPoolSegment) and a count for each segment of
@@ -90,6 +98,7 @@ constexpr size_t pool_bytes(uint64_t batch) {
 constexpr uint64_t pool_batch(uint64_t total, uint64_t max_batch, size_t room) {
   uint64_t batch = kPoolSegment;
   while (batch < total && batch < max_batch) batch *= 2;
+  // a launch of one batch may be smaller than kPoolSmallest, as long as it stays one
   while (batch > kPoolSmallest && 2 * pool_bytes(batch) > room / 2) batch /= 2;
   return 2 * pool_bytes(batch) > room / 2 ? 0 : batch;
 }

@@ -114,7 +114,7 @@ def test_rough_rays_drop_no_particle_that_hits(T, body, cv):
         T.tpmc_destroy(c)
 
 
-@pytest.mark.parametrize("budget_mib", [24, 80, 300, 2048])
+@pytest.mark.parametrize("budget_mib", [24, 80, 300, 1200, 2048])
 def test_pool_yields_to_the_memory_budget(T, budget_mib):
     """A pool of any size gives the same sums; meshes loaded after it find the room they would have had."""
     xyz, tri = M.cylinder(0.5, 2.0, 32, 7)
@@ -173,7 +173,7 @@ def test_empty_mesh_counts_every_particle(T):
         T.tpmc_destroy(c)
 
 
-@pytest.mark.parametrize("budget_mib", [96, 700, 0])
+@pytest.mark.parametrize("budget_mib", [96, 700, 2500, 0])
 def test_served_large_queries_match_direct_calls(T, budget_mib):
     """Served queries large enough for the steps' pools, among small ones and direct calls that use the context's own
     pool and make the others give their memory back: every result as alone."""
