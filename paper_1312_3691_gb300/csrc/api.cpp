@@ -281,9 +281,10 @@ void Ctx::destroy_pool(Pool& pool) {
 // kernels fill it.  One stream and batches of 2^26, 2^27 particles: the attitude
 // sweep 236 and 226 ms; two streams of 2^26: 217 (of 2^27: 211, for
 // twice the memory).
-// a.counter: two counters.
+// a.counter: kRunCounters counters.  Particles beyond max_batches batches are traced
+// by one launch that seeds them itself.
 cudaError_t Ctx::trace_pool(Pool& pool, cudaStream_t stream, TraceArgs a, uint32_t variant, const LaunchCfg& cfg,
-                            float area) {
+                            const MeshRec& m, float area, uint64_t max_batches) {
   // Rough rays first where less than 45 % of the particles are expected to meet
   // the front (its mean projected area over the control volume's).  They cost
   // 55 % of an exact seeding and what passes is seeded exactly after them: the
@@ -296,7 +297,7 @@ cudaError_t Ctx::trace_pool(Pool& pool, cudaStream_t stream, TraceArgs a, uint32
   for (cudaEvent_t* ev : {&pool.fork, &pool.join, &pool.done})
     if (e == cudaSuccess && !*ev) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
   if (e != cudaSuccess) return e;
-  const uint64_t total = a.total;
+  uint64_t total = a.total;
   uint64_t batch = std::min<uint64_t>(kPoolBatch, (pool.cap - 512) / (2 * (32 * kPoolEntryBytes + sizeof(uint32_t))) * 32);
   // Segments of 32 to 2,048 work indices (a power of two): as long as the trace
   // grid still gets eight a warp to even out its work, or two behind rough rays,
@@ -311,6 +312,7 @@ cudaError_t Ctx::trace_pool(Pool& pool, cudaStream_t stream, TraceArgs a, uint32
   a.segment = 32;
   while (2 * a.segment <= per_warp && a.segment < kPoolSegment) a.segment *= 2;
   batch = batch / a.segment * a.segment;
+  if (max_batches < total / batch) total = max_batches * batch;
   bool forked = false;
   uint64_t i = 0;
   for (a.g0 = 0; a.g0 < total && e == cudaSuccess; a.g0 += batch, ++i) {
@@ -338,6 +340,17 @@ cudaError_t Ctx::trace_pool(Pool& pool, cudaStream_t stream, TraceArgs a, uint32
   }
   const cudaError_t e3 = cudaEventRecord(pool.done, stream);
   if (e == cudaSuccess) e = e3;
+  if (e == cudaSuccess && total < a.total) {
+    TraceArgs r = a;
+    r.pool = nullptr;
+    r.g0 = total;
+    r.counter = a.counter + kRunCounters - 1;
+    const LaunchCfg c = schedule(m, variant & ~kVariantPool, a.total - total);
+    r.chunk = c.chunk;
+    r.smem_nodes = c.smem_nodes;
+    r.refill_at = c.refill_at;
+    e = launch_trace(r, variant & ~kVariantPool, c, num_sms, stream);
+  }
   return e;
 }
 
@@ -348,7 +361,7 @@ cudaError_t Ctx::trace_pool(Pool& pool, cudaStream_t stream, TraceArgs a, uint32
 // word to pinned memory (two uploads, a memset and two downloads took 25 us of
 // a small call).
 tpmc_status Ctx::run(const MeshRec& m, uint32_t nq, const QueryDev& base, const double* d_dirs, const double* d_S,
-                     uint64_t total, uint32_t variant, tpmc_result* d_out, const RecordsDev* rec) {
+                     uint64_t total, uint32_t variant, tpmc_result* d_out, const RecordsDev* rec, uint64_t max_batches) {
   tpmc_status st;
   if ((st = grow(s_queries, sizeof(QueryDev) * (size_t)nq, "queries")) != TPMC_OK) return st;
   if ((st = grow(s_acc, sizeof(AccStripe) * kAccStripes * (size_t)nq, "accumulators")) != TPMC_OK) return st;
@@ -384,7 +397,8 @@ tpmc_status Ctx::run(const MeshRec& m, uint32_t nq, const QueryDev& base, const 
   a.smem_nodes = cfg.smem_nodes;
   a.refill_at = cfg.refill_at;
   last_cfg = cfg;
-  if (total > 0 && (e = pooled ? trace_pool(pool, stream, a, variant, cfg, cv_area(base)) : launch_trace(a, variant, cfg, num_sms, stream)) != cudaSuccess)
+  if (total > 0 && (e = pooled ? trace_pool(pool, stream, a, variant, cfg, m, cv_area(base), max_batches)
+                               : launch_trace(a, variant, cfg, num_sms, stream)) != cudaSuccess)
     return cuda_fail(e, "trace kernel");
   if ((e = launch_finalize(d_queries, d_acc, nq, nq, nullptr, d_out, &words->error, h_err_word, stream)) != cudaSuccess)
     return cuda_fail(e, "finalize kernel");
@@ -790,7 +804,8 @@ tpmc_status tpmc_panel_sums(tpmc_ctx* ctx, tpmc_query_id query, int64_t* dv_q, u
 }
 
 static tpmc_status sweep_common(Ctx* c, tpmc_mesh_id mesh, const tpmc_params* base, const double* d_dirs,
-                                const double* d_S, uint32_t K, uint64_t N_each, tpmc_result* d_out) {
+                                const double* d_S, uint32_t K, uint64_t N_each, tpmc_result* d_out,
+                                uint64_t max_batches = ~0ull) {
   tpmc_status st = validate_params(base);
   if (st != TPMC_OK) return st;
   if (K == 0 || K > kMaxLaunchQueries) return fail(TPMC_EINVAL, "K must be in [1, 2^24]");
@@ -801,7 +816,7 @@ static tpmc_status sweep_common(Ctx* c, tpmc_mesh_id mesh, const tpmc_params* ba
   const MeshRec& m = it->second;
   QueryDev q;
   if ((st = fill_query(m, base, N_each, &q)) != TPMC_OK) return st;
-  return c->run(m, K, q, d_dirs, d_S, (uint64_t)K * N_each, trace_variant(base, m.dev), d_out, nullptr);
+  return c->run(m, K, q, d_dirs, d_S, (uint64_t)K * N_each, trace_variant(base, m.dev), d_out, nullptr, max_batches);
 }
 
 tpmc_status tpmc_sweep(tpmc_ctx* ctx, tpmc_mesh_id mesh, const tpmc_params* base, const double* h_dirs,
@@ -851,7 +866,7 @@ tpmc_status tpmc_sweep_device(tpmc_ctx* ctx, tpmc_mesh_id mesh, const tpmc_param
   Ctx* c = reinterpret_cast<Ctx*>(ctx);
   std::lock_guard<std::recursive_mutex> lk(c->mu);
   cudaSetDevice(c->device);
-  return sweep_common(c, mesh, base, d_dirs, d_S, K, N_each, d_out);
+  return sweep_common(c, mesh, base, d_dirs, d_S, K, N_each, d_out, kPoolBatchesQueued);
 }
 
 tpmc_status tpmc_set_launch(tpmc_ctx* ctx, const tpmc_launch* cfg) {

@@ -82,6 +82,12 @@ constexpr uint64_t kPoolMin = 1u << 22, kPoolMinOne = 6u << 20;
 //   hemisphere  71.1 31.2  79.6 40.1  65.8 31.2  63.0 28.2  61.4 27.6
 //   satellite   7.3 9.7    23.5 26.8  9.4 11.5   6.9 8.7    5.2 6.2
 constexpr uint64_t kPoolBatch = 1ull << 26, kPoolSmallest = 1ull << 23;
+// Batches that a call which only enqueues (tpmc_sweep_device, a serving step) puts
+// into its two streams, each of which gets as many launches: a stream's queue holds
+// about 1,024, and beyond that the host waits for the GPU with the context's lock
+// held (2^35 particles in batches of 2^23 on no mesh: 346 of 461 ms; now 4).  What is
+// left is one launch.
+constexpr uint64_t kPoolBatchesQueued = 896;
 constexpr uint32_t kPoolSegment = 2048;  // work indices of a segment, at most (a batch is a multiple)
 
 // Bytes of half a pool: entries for `batch` particles (a multiple of kPoolSegment) and a count for each segment of
@@ -154,13 +160,15 @@ struct Ctx {
   tpmc_status grow(Scratch& s, size_t bytes, const char* what);
   LaunchCfg schedule(const MeshRec& m, uint32_t variant, uint64_t total);  // variant: see trace_variant
   tpmc_status run(const MeshRec& m, uint32_t nq, const QueryDev& base, const double* d_dirs, const double* d_S,
-                  uint64_t total, uint32_t variant, tpmc_result* d_out, const RecordsDev* rec);
+                  uint64_t total, uint32_t variant, tpmc_result* d_out, const RecordsDev* rec,
+                  uint64_t max_batches = ~0ull);
   bool grow_pool(Pool& pool, uint64_t total, uint64_t max_batch);
   void release_pool(Pool& pool);
   bool release_pools();
   size_t pooled() const;
   void destroy_pool(Pool& pool);
-  cudaError_t trace_pool(Pool& pool, cudaStream_t stream, TraceArgs a, uint32_t variant, const LaunchCfg& cfg, float area);
+  cudaError_t trace_pool(Pool& pool, cudaStream_t stream, TraceArgs a, uint32_t variant, const LaunchCfg& cfg,
+                         const MeshRec& m, float area, uint64_t max_batches);
   tpmc_status check_error_word();
   ~Ctx();
 };

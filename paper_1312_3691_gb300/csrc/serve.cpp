@@ -272,7 +272,7 @@ bool enqueue_step(ServeState* s, int b, int prev, const std::vector<Request*>& c
     if (e == cudaSuccess)
       e = launch_setup(s->d_q, n_fresh, nullptr, nullptr, nullptr, nullptr, B.d_fresh, s->d_acc, kSlots, c->vn_table, nullptr, st);
   }
-  if (e == cudaSuccess) e = cudaMemsetAsync(B.d_counters, 0, 2 * kMaxGroups * sizeof(unsigned long long), st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(B.d_counters, 0, kRunCounters * kMaxGroups * sizeof(unsigned long long), st);
   // the groups run on their own streams once the set-up is done, so that one
   // launch's tail overlaps the next launch's start
   if (e == cudaSuccess) e = cudaEventRecord(B.ready, st);
@@ -316,7 +316,7 @@ bool enqueue_step(ServeState* s, int b, int prev, const std::vector<Request*>& c
     a.items = B.d_items + first_item;
     a.n_items = n_items - first_item;
     a.total = g;
-    a.counter = B.d_counters + 2 * gi;  // two: the pool's streams have one each
+    a.counter = B.d_counters + kRunCounters * gi;
     a.error = B.d_err;
     a.count_work = c->counters ? 1u : 0u;
     a.vn_table = c->vn_table;
@@ -336,10 +336,11 @@ bool enqueue_step(ServeState* s, int b, int prev, const std::vector<Request*>& c
       if (B.pool.ptr || c->grow_pool(B.pool, kServePoolBatch, kServePoolBatch)) {
         pooled = B.pooled = true;
         const uint32_t variant = groups[gi].first.second | kVariantPool;
-        const LaunchCfg pcfg = c->schedule(c->meshes.at(groups[gi].first.first), variant, g);
+        const MeshRec& mr = c->meshes.at(groups[gi].first.first);
+        const LaunchCfg pcfg = c->schedule(mr, variant, g);
         a.smem_nodes = pcfg.smem_nodes;
         a.refill_at = pcfg.refill_at;
-        e = c->trace_pool(B.pool, gst, a, variant, pcfg, cv_area(groups[gi].second.front()->q));
+        e = c->trace_pool(B.pool, gst, a, variant, pcfg, mr, cv_area(groups[gi].second.front()->q), kPoolBatchesQueued);
       }
     }
     if (e == cudaSuccess && !pooled) e = launch_trace(a, groups[gi].first.second, cfg, c->num_sms, gst);
@@ -521,7 +522,7 @@ tpmc_status start_serving(Ctx* c) {
     return cuda_fail(e, "serving stream");
   }
   const size_t per_buf_dev = kSlots * (sizeof(ItemDev) + 2 * sizeof(uint32_t) + sizeof(tpmc_result)) +
-                             2 * kMaxGroups * sizeof(unsigned long long) + 256;
+                             kRunCounters * kMaxGroups * sizeof(unsigned long long) + 256;
   const size_t dev_bytes = kSlots * (sizeof(QueryDev) + kAccStripes * sizeof(AccStripe)) + kInFlight * per_buf_dev + 256;
   tpmc_status st = c->alloc(&s->d_block, dev_bytes, "serving slots");
   if (st != TPMC_OK) {
@@ -545,7 +546,7 @@ tpmc_status start_serving(Ctx* c) {
     StepBuf& B = s->buf[b];
     B.d_items = (ItemDev*)p; p += kSlots * sizeof(ItemDev);
     B.d_res = (tpmc_result*)p; p += kSlots * sizeof(tpmc_result);
-    B.d_counters = (unsigned long long*)p; p += 2 * kMaxGroups * sizeof(unsigned long long);
+    B.d_counters = (unsigned long long*)p; p += kRunCounters * kMaxGroups * sizeof(unsigned long long);
     B.d_fresh = (uint32_t*)p; p += kSlots * sizeof(uint32_t);
     B.d_fin = (uint32_t*)p; p += kSlots * sizeof(uint32_t);
     B.d_err = (int*)p; p += 256;

@@ -209,13 +209,13 @@ struct TraceArgs {
   unsigned long long* counter;  // global work counter (zeroed before launch)
   int* error;                 // device error word (stack overflow)
   const float* vn_table;      // [kVnNS][kVnNZ] normal-speed start table
+  uint64_t g0 = 0;                // first work index of the launch
   // pool path (kVariantPool): the particles of work indices g0 ... total - 1,
   // seeded beforehand in n_seg segments of `segment` indices
   void* pool = nullptr;           // Seeded<float>[n_seg][segment]: a segment's particles that may hit, closed up
   uint32_t* seg_count = nullptr;  // [n_seg] how many
   uint32_t n_seg = 0, segment = 0;
   uint32_t prefilter = 0;         // 1: rough rays first (may_hit)
-  uint64_t g0 = 0;
   RecordsDev rec;
 };
 constexpr size_t kPoolEntryBytes = 32;
@@ -249,11 +249,13 @@ inline uint32_t trace_variant(const tpmc_params* p, const MeshDev& m) {
 inline uint32_t variant_width(uint32_t v) { return (v & kVariantWide8) ? 8u : ((v & kVariantWide4) ? 4u : 2u); }
 inline uint32_t node_float4s(uint32_t width) { return width == 8 ? 5u : (width == 4 ? 4u : 2u); }
 
-// A run's counters (the second for the pool's second stream) and error word.
+// A run's work counters (the second for the pool's second stream, the third for
+// what follows the pool, Ctx::trace_pool) and error word.
+constexpr int kRunCounters = 3;
 struct RunWords {
-  unsigned long long counter[2];
+  unsigned long long counter[kRunCounters];
   int error;
-  int pad[3];
+  int pad;
 };
 
 // Set-up of nq queries (block i: slot slots[i], or i), which also clears

@@ -1873,7 +1873,7 @@ __global__ void __launch_bounds__(MINB > 0 ? 128 : 256, MINB > 0 ? MINB : (sizeo
         if (pool_rem == 0) {
           unsigned long long base = 0;
           if (lane == 0) base = atomicAdd(a.counter, (unsigned long long)a.chunk);
-          base = __shfl_sync(kFull, base, 0);
+          base = a.g0 + __shfl_sync(kFull, base, 0);
           if (base >= a.total) {
             drained = true;
             break;

@@ -1,6 +1,7 @@
 """Pools of seeded particles and the memory around them: who waits for it, how often it is taken, on the GPU."""
 import time
 
+import numpy as np
 import pytest
 
 from tpmc_inputs import meshes as M
@@ -104,5 +105,57 @@ def test_serving_takes_a_pool_for_each_step_in_flight_once(T):
         ids = [T.tpmc_submit(c, mesh, _base(T), N) for N in sizes]
         assert [T.tpmc_poll(c, i)["n_particles"] for i in ids] == sizes
         assert T.tpmc_memory_info(c)["n_allocs"] - before <= 2
+    finally:
+        T.tpmc_destroy(c)
+
+
+def test_device_sweep_of_thousands_of_batches_only_enqueues(T):
+    """2^35 particles (on no mesh) with room for batches of 2^23: the call returns while most of them are to come, and
+    every item counts its particles, those traced after the pool's batches as well."""
+    import torch
+
+    K, N = 64, 1 << 29
+    c = T.tpmc_create(0, 1200 << 20)
+    try:
+        mesh = T.tpmc_mesh_load(c, np.zeros((0, 3)), np.zeros((0, 3), np.uint32))
+        out = torch.zeros(K * T.RESULT_BYTES // 8, dtype=torch.int64, device="cuda")
+        p = _base(T, r_cv=1.0)
+        T.tpmc_sweep_device(c, mesh, p, None, None, K, 1 << 20, out)
+        torch.cuda.synchronize()
+        assert T.tpmc_memory_info(c)["used"] > 64 << 23  # the pool is there
+        t0 = time.perf_counter()
+        T.tpmc_sweep_device(c, mesh, p, None, None, K, N, out)
+        enqueued = time.perf_counter() - t0
+        torch.cuda.synchronize()
+        whole = time.perf_counter() - t0
+        # a host that waits for room in the queue is there to the last few thousand of 8,192 launches
+        assert enqueued < 0.25 * whole, (enqueued, whole)
+        assert bool((out.view(K, -1)[:, 31] == N).all())  # n_particles: 25 doubles and six sums before it
+    finally:
+        T.tpmc_destroy(c)
+
+
+def test_what_follows_the_pool_gives_the_same_sums(T):
+    """2^33 particles and some, with room for batches of 2^23: 896 of them go through the pool, 128 and a ragged rest do
+    not; the sums are the fused launch's."""
+    import torch
+
+    K, N = 3, (1 << 33) // 3 + 12_345
+    xyz, tri = M.plate(1.0)
+    c = T.tpmc_create(0, 1200 << 20)
+    try:
+        mesh = T.tpmc_mesh_load(c, xyz, tri)
+        rows = []
+        for counting in (False, True):
+            T.tpmc_set_counters(c, counting)
+            out = torch.zeros(K * T.RESULT_BYTES // 8, dtype=torch.int64, device="cuda")
+            d = torch.from_numpy(np.random.default_rng(2).normal(size=(K, 3))).cuda()
+            torch.cuda.synchronize()
+            T.tpmc_sweep_device(c, mesh, _base(T), d, None, K, N, out)
+            torch.cuda.synchronize()
+            got = out.view(K, -1).cpu()
+            rows.append(torch.cat([got[:, :35], got[:, 39:]], dim=1))  # all but the work counters, the id and ms
+        assert bool((rows[0] == rows[1]).all())
+        assert bool((rows[0][:, 31] == N).all())
     finally:
         T.tpmc_destroy(c)
