@@ -205,9 +205,15 @@ tpmc_status tpmc_set_stream(tpmc_ctx* ctx, void* cuda_stream);
 const char* tpmc_last_error(const tpmc_ctx* ctx);
 
 /* Device memory of the context: *used, the bytes it holds through its own
- * allocations (meshes and their BVHs, scratch, panel buffers, serving slots),
- * *budget, the limit set at creation, and *n_allocs, the number of device
- * allocations it has made since creation.  Any pointer may be NULL. */
+ * allocations (meshes and their BVHs, scratch, panel buffers, serving slots,
+ * pools of seeded particles), *budget, the limit set at creation, and *n_allocs,
+ * the number of device allocations it has made since creation.  Any pointer may be
+ * NULL.
+ * A pool serves FP32 calls of 2^22 particles and more and is kept for the next one
+ * until the context is destroyed or another of its allocations needs the room: up
+ * to 4.3 GB for direct calls and 2.1 GB for each of the two serving steps, at most
+ * half of what the budget leaves and a quarter of the device's free memory when it
+ * is taken.  A context with a smaller budget has smaller pools, or none. */
 tpmc_status tpmc_memory_info(tpmc_ctx* ctx, size_t* used, size_t* budget, uint64_t* n_allocs);
 
 /* Enables (1) or disables (0) the traversal counters n_node_visits and

@@ -225,9 +225,21 @@ float cv_area(const QueryDev& q) {
 // A pool for launches of `total` particles: twice the entries of a batch (at most
 // max_batch) and a count for each of its segments, in the memory the context's
 // budget leaves (pool_batch); false when it has no room (the launch then seeds
-// inside the trace kernel).
+// inside the trace kernel).  A pool outlives its call, so a new one also takes at
+// most a quarter of the device's free memory: three quarters stay for whoever
+// shares the device and cannot ask for the pool back.
 bool Ctx::grow_pool(Pool& pool, uint64_t total, uint64_t max_batch) {
-  const uint64_t batch = pool_batch(total, max_batch, budget - std::min(budget, used - pool.cap));
+  size_t room = budget - std::min(budget, used - pool.cap);
+  uint64_t batch = pool_batch(total, max_batch, room);
+  if (batch > 0 && pool.cap < 2 * pool_bytes(batch)) {
+    size_t free_b = 0, total_b = 0;
+    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    room = std::min(room, (free_b + pool.cap) / 2);
+    batch = pool_batch(total, max_batch, room);
+  }
   if (batch == 0) return false;
   const size_t need = 2 * pool_bytes(batch);
   if (pool.cap >= need) return true;

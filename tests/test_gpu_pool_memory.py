@@ -159,3 +159,29 @@ def test_what_follows_the_pool_gives_the_same_sums(T):
         assert bool((rows[0][:, 31] == N).all())
     finally:
         T.tpmc_destroy(c)
+
+
+def test_pools_leave_the_device_to_others(T):
+    """With 8 GB of the device free, a context whose budget allows more takes at most a quarter for its pools, each
+    time; another user of the device finds what is left."""
+    import torch
+
+    c = T.tpmc_create(0)
+    try:
+        mesh = T.tpmc_mesh_load(c, *M.plate(1.0))
+        torch.cuda.empty_cache()
+        free = torch.cuda.mem_get_info()[0]
+        rest = 8 << 30
+        if free < 2 * rest:
+            pytest.skip("the device is in use")
+        others = torch.empty(free - rest, dtype=torch.uint8, device="cuda")
+        before = T.tpmc_memory_info(c)["used"]
+        assert T.tpmc_trace(c, mesh, _base(T), 1 << 27)["n_particles"] == 1 << 27
+        assert 0 < T.tpmc_memory_info(c)["used"] - before <= rest // 4 + (1 << 20)
+        ids = [T.tpmc_submit(c, mesh, _base(T), 1 << 25) for _ in range(3)]
+        assert [T.tpmc_poll(c, i)["n_particles"] for i in ids] == [1 << 25] * 3
+        more = torch.empty(rest // 3, dtype=torch.uint8, device="cuda")
+        del others, more
+    finally:
+        T.tpmc_destroy(c)
+        torch.cuda.empty_cache()
