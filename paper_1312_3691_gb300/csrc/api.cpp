@@ -402,7 +402,7 @@ tpmc_status Ctx::run(const MeshRec& m, uint32_t nq, const QueryDev& base, const 
   a.vn_table = vn_table;
   if (rec) a.rec = *rec;
   const bool pooled = !counters && !rec && (variant & 1u) == TPMC_FP32 && total > 0 &&
-                      (pool_always || total >= (nq > 1 ? kPoolMin : kPoolMinOne)) && grow_pool(pool, total, kPoolBatch);
+                      (pool_always || total >= kPoolMin) && grow_pool(pool, total, kPoolBatch);
   if (pooled) variant |= kVariantPool;
   const LaunchCfg cfg = schedule(m, variant, total);
   a.chunk = cfg.chunk;

@@ -62,16 +62,18 @@ constexpr size_t kPinnedBytes = 256 + kPinnedItems * (sizeof(tpmc_result) + 4 * 
 // BVH width of mesh loads that neither tpmc_set_launch nor tpmc_tune decided.
 constexpr uint32_t kDefaultBvhWidth = 2;
 
-// FP32 launches of at least this many particles go through the pool, those of one
-// query from kPoolMinOne on.  Below, the second launch and two tails cost more
-// than the leaner kernels save.  us through the pool / fused at S = 7: one query of
-// 2^22 and 2^23 particles, then 16 and 512 queries of 2^22 in all:
-//   plate       153/188    242/325     256/335    1685/1834
-//   icosphere   963/1053   1771/2041   1076/1376  2555/2950
-//   cylinder    656/617    1079/1173   711/832    2142/2318
-//   hemisphere  3062/3322  5746/6273   1832/2176  3309/3638
-//   satellite   660/717    1029/1179   787/956    2359/2538
-constexpr uint64_t kPoolMin = 1u << 22, kPoolMinOne = 6u << 20;
+// FP32 launches of at least this many particles go through the pool.  Below, the
+// second launch and two tails cost what the leaner kernels save.  us fused / through
+// the pool at S = 7, eps = 0.9: one query of 2^21 and 2^22 particles, then 16 queries
+// of 2^20 and 2^22 in all:
+//   plate       169/178    277/263     162/161  339/245
+//   icosphere   548/513    1013/890    448/377  1362/1023
+//   cylinder    337/470    582/558     316/299  829/680
+//   hemisphere  1886/1711  3358/3001   875/787  2159/1772
+//   satellite   532/518    674/597     761/758  1154/946
+// (one query of 2^22 at three S and directions: the cylinder 5 % faster to 2 %
+// slower, the other bodies 3 to 21 % faster)
+constexpr uint64_t kPoolMin = 1u << 22;
 // Particles of a batch, at most and, in a launch of several, at least (32 bytes
 // each, two batches).  Every batch has a tail of its own, the fused launch one for
 // all.  ms for 1e8 particles of one query and for 96 queries of 1e6, fused, then

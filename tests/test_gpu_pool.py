@@ -34,7 +34,7 @@ def _base(T, **kw):
 
 # (items, particles each): the pool's smallest launches, of several items and of one; several items a batch with ragged ends; over two
 # batches of 2^26 (both streams, and the first pool again); many items inside one segment of 256 work indices
-@pytest.mark.parametrize("K,N", [(2, (1 << 21) + 5), (1, 6 << 20), (1, (1 << 23) + 1), (3, 12_000_017), (7, 25_000_003),
+@pytest.mark.parametrize("K,N", [(2, (1 << 21) + 5), (1, (1 << 22) + 3), (1, 6 << 20), (1, (1 << 23) + 1), (3, 12_000_017), (7, 25_000_003),
                                  (400_000, 97)])
 @pytest.mark.parametrize("width", [2, 4, 8])
 @pytest.mark.parametrize("gsi", ["maxwell", "cll"])
