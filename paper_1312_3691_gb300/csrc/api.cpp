@@ -385,8 +385,8 @@ tpmc_status Ctx::run(const MeshRec& m, uint32_t nq, const QueryDev& base, const 
   RunWords* words = (RunWords*)s_misc.ptr;
   cudaError_t e;
   // the set-up also clears the queries' accumulators
-  if ((e = launch_setup(d_queries, nq, &base, d_dirs, d_S, d_items, nullptr, d_acc, nq, vn_table, words, stream)) !=
-      cudaSuccess)
+  if ((e = launch_setup(d_queries, nq, &base, d_dirs, d_S, d_items, nullptr, d_acc, nq, vn_table, words, num_sms,
+                        stream)) != cudaSuccess)
     return cuda_fail(e, "setup kernel");
   TraceArgs a{};
   a.mesh = m.dev;

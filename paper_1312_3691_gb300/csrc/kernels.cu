@@ -467,16 +467,16 @@ cudaError_t launch_after(void (*f)(P...), uint32_t grid, uint32_t block, size_t 
 
 cudaError_t launch_setup(QueryDev* d_queries, uint32_t nq, const QueryDev* h_base, const double* d_dirs,
                          const double* d_S, ItemDev* d_items, const uint32_t* d_slots, AccStripe* d_acc,
-                         uint32_t acc_stride, const float* tables, RunWords* d_zero, cudaStream_t stream) {
+                         uint32_t acc_stride, const float* tables, RunWords* d_zero, int num_sms, cudaStream_t stream) {
   if (nq == 0) return cudaSuccess;
   static_assert(sizeof(SetupBase) <= 3800, "a kernel's parameters");
   SetupBase with{};
   with.given = h_base != nullptr ? 1u : 0u;
   if (h_base != nullptr) with.q = *h_base;
   // Blocks of their own for the table as long as the chip's SMs are not all
-  // busy with other queries (152 SMs; beyond that the split only repeats the
-  // scalars the table needs).
-  const dim3 grid(nq, nq * kSetupParts <= 2 * 152 ? kSetupParts : 1);
+  // busy with other queries (beyond that the split only repeats the scalars the
+  // table needs).
+  const dim3 grid(nq, (uint64_t)nq * kSetupParts <= 2 * (uint64_t)num_sms ? kSetupParts : 1);
   setup_kernel<<<grid, kSetupThreads, 0, stream>>>(d_queries, with, d_dirs, d_S, d_items, d_slots, d_acc, acc_stride,
                                                    reinterpret_cast<const double*>(tables + kVnNS * kVnNZ + 1), d_zero);
   return cudaGetLastError();

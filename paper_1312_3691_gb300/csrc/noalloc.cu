@@ -92,7 +92,7 @@ extern "C" tpmc_status tpmc_sweep_noalloc(tpmc_ctx* ctx, tpmc_mesh_id mesh, cons
   if (h_dirs) std::memcpy(dirs, h_dirs, (size_t)K * 3 * sizeof(double));
   if (h_S) std::memcpy(S, h_S, (size_t)K * sizeof(double));
   if ((e = launch_setup(A->queries, K, &q, dirs, S, A->items, nullptr, A->acc, kNoAllocMaxQueries, c->vn_table, &A->words,
-                        s)) != cudaSuccess)
+                        c->num_sms, s)) != cudaSuccess)
     return cuda_fail(e, "setup kernel");
   TraceArgs a{};
   a.mesh = m.dev;

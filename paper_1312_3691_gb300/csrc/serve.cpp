@@ -270,7 +270,8 @@ bool enqueue_step(ServeState* s, int b, int prev, const std::vector<Request*>& c
     e = cudaMemcpyAsync(B.d_fresh, B.h_fresh, n_fresh * sizeof(uint32_t), cudaMemcpyHostToDevice, st);
     // the set-up also clears the fresh slots' accumulators
     if (e == cudaSuccess)
-      e = launch_setup(s->d_q, n_fresh, nullptr, nullptr, nullptr, nullptr, B.d_fresh, s->d_acc, kSlots, c->vn_table, nullptr, st);
+      e = launch_setup(s->d_q, n_fresh, nullptr, nullptr, nullptr, nullptr, B.d_fresh, s->d_acc, kSlots, c->vn_table, nullptr,
+                       c->num_sms, st);
   }
   if (e == cudaSuccess) e = cudaMemsetAsync(B.d_counters, 0, kRunCounters * kMaxGroups * sizeof(unsigned long long), st);
   // the groups run on their own streams once the set-up is done, so that one

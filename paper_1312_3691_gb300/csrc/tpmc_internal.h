@@ -263,7 +263,7 @@ struct RunWords {
 // and, when given, the run's words.
 cudaError_t launch_setup(QueryDev* d_queries, uint32_t nq, const QueryDev* h_base, const double* d_dirs,
                          const double* d_S, ItemDev* d_items, const uint32_t* d_slots, AccStripe* d_acc,
-                         uint32_t acc_stride, const float* tables, RunWords* d_zero, cudaStream_t stream);
+                         uint32_t acc_stride, const float* tables, RunWords* d_zero, int num_sms, cudaStream_t stream);
 // Fills a context's tables: the normal-speed start table, then (8-byte
 // aligned) the uniforms Phi(z_j) of the latitude knots as doubles.
 cudaError_t launch_tables(float* d_tables, cudaStream_t stream);
