@@ -732,29 +732,19 @@ __device__ __forceinline__ float grid_q(uint32_t w, uint32_t sel) {
 // while other lanes are still searching.
 constexpr int kDone = (int)0x80000000;  // no valid leaf code: first + count would exceed 2^24
 
-// Traversal stack entry: a stacked child and its entry distance.  In float
-// the pair is one 8-byte local-memory access per push and per pop (two 4-byte
-// arrays took two).  The pool kernel with its first four entries in shared memory
+// Traversal stack entry of binary trees: a stacked child and its entry distance
+// (float in both precisions: it is the box tests'), one 8-byte local-memory access
+// per push and per pop (two 4-byte arrays took two).  The pool kernel with its first four entries in shared memory
 // instead, and so a branch at each access and less L1: cylinder sweep 91.8 -> 92.7
 // ms, hemisphere 6.55 -> 6.59, moments 3.44 -> 3.48, attitude sweep 185.4 -> 186.8.
-template <typename R> struct StackE;
-template <> struct __align__(8) StackE<float> { int node; float t; };
-template <> struct __align__(16) StackE<double> { double t; int node; int pad; };
-__device__ __forceinline__ void stack_put(StackE<float>* s, int i, int node, float t) {
+struct __align__(8) StackE { int node; float t; };
+__device__ __forceinline__ void stack_put(StackE* s, int i, int node, float t) {
   *reinterpret_cast<int2*>(s + i) = make_int2(node, __float_as_int(t));
 }
-__device__ __forceinline__ void stack_put(StackE<double>* s, int i, int node, double t) {
-  s[i].t = t;
-  s[i].node = node;
-}
-__device__ __forceinline__ void stack_get(const StackE<float>* s, int i, int& node, float& t) {
+__device__ __forceinline__ void stack_get(const StackE* s, int i, int& node, float& t) {
   const int2 v = *reinterpret_cast<const int2*>(s + i);
   node = v.x;
   t = __int_as_float(v.y);
-}
-__device__ __forceinline__ void stack_get(const StackE<double>* s, int i, int& node, double& t) {
-  node = s[i].node;
-  t = s[i].t;
 }
 
 template <typename R, typename B = R>
@@ -785,7 +775,7 @@ __device__ __forceinline__ void trav_begin(Trav<R, B>& t) {
 
 // Next stacked candidate whose entry distance is still below the best hit.
 template <typename R, typename B>
-__device__ __forceinline__ int trav_pop(Trav<R, B>& t, StackE<B>* stack) {
+__device__ __forceinline__ int trav_pop(Trav<R, B>& t, StackE* stack) {
   while (t.sp > 0) {
     --t.sp;
     int node;
@@ -801,7 +791,7 @@ __device__ __forceinline__ int trav_pop(Trav<R, B>& t, StackE<B>* stack) {
 // below n_stage come from the copy in shared memory.
 template <bool STAGE, typename R, typename B>
 __device__ __forceinline__ void trav_inner(const MeshDev& m, const float4* __restrict__ s_nodes, uint32_t n_stage,
-                                           const Ray<R, B>& r, Trav<R, B>& t, StackE<B>* stack,
+                                           const Ray<R, B>& r, Trav<R, B>& t, StackE* stack,
                                            uint32_t& n_nodes) {
   ++n_nodes;
   float4 n0, n1;
@@ -872,7 +862,7 @@ __device__ __forceinline__ void trav_inner(const MeshDev& m, const float4* __res
 // the postponed one.  Returns true when the ray's traversal is finished.
 template <typename R, typename B>
 __device__ __forceinline__ void trav_leaf(const MeshDev& m, const Ray<R, B>& r, uint32_t last, Trav<R, B>& t,
-                                          StackE<B>* stack, uint32_t& n_tris) {
+                                          StackE* stack, uint32_t& n_tris) {
   const uint32_t code = ~(uint32_t)t.leaf;
   const uint32_t first = code & 0xFFFFFFu, count = code >> 24;
   const Shear<R> sh = make_shear<R>(r.d);
@@ -1237,10 +1227,10 @@ __device__ __forceinline__ void lane_add_d2(LaneAcc& a, unsigned long long x) {
 
 // Adds the 96-bit sum hi 2^64 + lo of one flush to the three limbs of the
 // stripe's squared-drag sum: bits 0-29, bits 30-59, and hi 2^4 + (lo >> 60).
-// Every flush carries at least one particle and a query has at most 2^34, so
-// each low limb stays below 2^34 2^30 = 2^64; the top limb stays below the
-// exact total over 2^60, which is below 2^36 (each particle's term is below
-// 2^62).
+// A flush whose sum is not 0 carries at least one finished particle and a query
+// has at most 2^34, so each low limb stays below 2^34 2^30 = 2^64; the top limb
+// stays below the exact total over 2^60, which is below 2^36 (each particle's term
+// is below 2^62).
 __device__ __forceinline__ void add_d2(AccStripe& A, unsigned long long lo, unsigned long long hi) {
   constexpr unsigned long long kM30 = (1ull << 30) - 1ull;
   const unsigned long long l0 = lo & kM30, l1 = (lo >> 30) & kM30, l2 = (hi << 4) | (lo >> 60);
@@ -1261,7 +1251,10 @@ __device__ __forceinline__ int acc_stripe() {
 // so the result does not depend on the order.  Lanes that flushed by themselves
 // put 13 atomics each on the query's few lines, and a lane without a particle (a
 // launch's last warps hold many) made all 32 do so: 60 ns a warp, 270 us of a
-// 131,072-particle launch on the cylinder, now 50.
+// 131,072-particle launch on the cylinder, now 50.  Queries are taken one after the
+// other; with very many of a few particles each, where a warp holds up to 32, that
+// is no slower: 65,536 queries of 1, 4, 16 and 63 particles on the cylinder 64.7 to
+// 65.4 -> 7.5 to 8.3 ms a call, 2^20 of 1 and of 8 1,031 -> 120 (set-up included).
 __device__ __noinline__ void warp_flush(AccStripe* acc, uint32_t stride, LaneAcc& a, int stripe) {
   const uint32_t lane = threadIdx.x & 31u;
   unsigned todo = __ballot_sync(kFull, a.q >= 0 && a.particles + a.hits > 0);
@@ -1757,7 +1750,7 @@ __global__ void __launch_bounds__(MINB > 0 ? 128 : 256, MINB > 0 ? MINB : (sizeo
   using B = std::conditional_t<W == 2, float, R>;  // of the box tests
   Ray<R, B> ray;
   using TV = std::conditional_t<(W > 2), TravW<R>, Trav<R, B>>;
-  using SE = std::conditional_t<(W > 2), uint2, StackE<B>>;
+  using SE = std::conditional_t<(W > 2), uint2, StackE>;
   TV tv{};
   if constexpr (W == 2) tv.cur = kDone;  // nothing to do
   SE stack[W > 2 ? kMaxStackW : kMaxStack];
