@@ -137,15 +137,24 @@ def test_pool_yields_to_the_memory_budget(T, budget_mib):
         T.tpmc_destroy(c)
 
 
-@pytest.mark.parametrize("r_cv", [0.75, 40.0, 3000.0])
+# r_cv: spheres from tight to 80 bodies wide; long: flux boxes close around the body and as many metres long upstream,
+# at S = 50, so that rays that hit start beyond the front boxes' reach (256 to 512 extents for binary trees, 8 radii for
+# wide ones) as well as within it
+@pytest.mark.parametrize("r_cv,long", [(0.75, 0), (40.0, 0), (0, 6), (0, 1000)])
 @pytest.mark.parametrize("name", ["plate", "cylinder"])
 @pytest.mark.parametrize("width", [2, 8])
-def test_front_rejects_no_particle_that_hits(T, orc, name, r_cv, width):
-    """Control volumes from tight to thousands of bodies wide (beyond the front boxes' reach): the oracle's hits."""
+def test_front_rejects_no_particle_that_hits(T, orc, name, r_cv, long, width):
+    """Control volumes from tight to beyond the front boxes' reach: the oracle's hits."""
     xyz, tri = M.plate(1.0) if name == "plate" else M.cylinder(0.3, 0.8, 12, 2)
     # aim: particles are seeded on the far volume, so the flow is cold and few of them meet the body
-    N = 20_000 if r_cv < 1 else 400_000
-    kw = dict(**W.base_state(S=8.0), dir=(0.02, 0.01, -1.0), eps_diffuse=0.9, A_ref=1.0, r_cv=r_cv, max_bounces=16, seed=3)
+    N = 20_000 if 0 < r_cv < 1 else 1_000_000
+    kw = dict(eps_diffuse=0.9, A_ref=1.0, max_bounces=16, seed=3)
+    if long:
+        lo, hi = xyz.min(axis=0) - 0.05, xyz.max(axis=0) + 0.05
+        hi[2] += long
+        kw.update(W.base_state(S=50.0), dir=(0.0, 0.0, -1.0), cv_kind=T.TPMC_CV_BOX_FLUX, box_lo=tuple(lo), box_hi=tuple(hi))
+    else:
+        kw.update(W.base_state(S=8.0), dir=(0.02, 0.01, -1.0), r_cv=r_cv)
     c = T.tpmc_create(0)
     try:
         T.tpmc_set_launch(c, block=0, bvh_width=width)
@@ -153,12 +162,15 @@ def test_front_rejects_no_particle_that_hits(T, orc, name, r_cv, width):
         r = T.tpmc_trace(c, mesh, T.make_params(**kw), N)
     finally:
         T.tpmc_destroy(c)
-    o = orc.trace(orc.Mesh(xyz, tri), orc.make_params(**kw), N)[0]
+    o, _, rec = orc.trace(orc.Mesh(xyz, tri), orc.make_params(**kw), N, records=True, K=1)
     assert r["n_particles"] == N
-    # float positions are off by 6e-8 r_cv: particles that near to a silhouette edge may fall on either side
-    edge = 8.0 * 6e-8 * r_cv / 0.5 * max(1.0, float(o["n_hits"]))
+    # float positions are off by 6e-8 of the volume's size: particles that near to a silhouette edge may fall on either side
+    edge = 8.0 * 6e-8 * (r_cv or long) / 0.5 * max(1.0, float(o["n_hits"]))
     assert abs(int(r["n_hits"]) - int(o["n_hits"])) <= 2 + edge, (r["n_hits"], o["n_hits"])
-    if r_cv < 1:
+    assert o["n_hits"] >= 50
+    if long:
+        assert int(((rec["n_hits"] > 0) & (rec["pos"][:, 2] > 0.5 * long)).sum()) >= 10
+    if 0 < r_cv < 1:
         assert r["n_hits"] > 1000 and abs(r["CD"] - o["CD"]) <= 1e-4 * abs(o["CD"]) + 3 * o["CD_sigma"]
 
 
