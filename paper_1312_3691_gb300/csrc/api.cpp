@@ -222,26 +222,26 @@ float cv_area(const QueryDev& q) {
   return (float)((x * y + y * z + z * x) / 6.283185307179586);
 }
 
-// A pool for launches of `total` particles: twice the entries of a batch (at most
-// max_batch) and a count for each of its segments, in the memory the context's
-// budget leaves (pool_batch); false when it has no room (the launch then seeds
+// A pool for launches of `total` particles in batches of at most max_batch, in the
+// memory the context's budget leaves (pool_entries); false when it has no room (the launch then seeds
 // inside the trace kernel).  A pool outlives its call, so a new one also takes at
 // most a quarter of the device's free memory: three quarters stay for whoever
 // shares the device and cannot ask for the pool back.
 bool Ctx::grow_pool(Pool& pool, uint64_t total, uint64_t max_batch) {
+  pool.max_batch = max_batch;
   size_t room = budget - std::min(budget, used - pool.cap);
-  uint64_t batch = pool_batch(total, max_batch, room);
-  if (batch > 0 && pool.cap < 2 * pool_bytes(batch)) {
+  uint64_t entries = pool_entries(total, max_batch, room);
+  if (entries > 0 && pool.cap < pool_bytes(entries)) {
     size_t free_b = 0, total_b = 0;
     if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
       cudaGetLastError();
       return false;
     }
     room = std::min(room, (free_b + pool.cap) / 2);
-    batch = pool_batch(total, max_batch, room);
+    entries = pool_entries(total, max_batch, room);
   }
-  if (batch == 0) return false;
-  const size_t need = 2 * pool_bytes(batch);
+  if (entries == 0) return false;
+  const size_t need = pool_bytes(entries);
   if (pool.cap >= need) return true;
   release_pool(pool);
   const std::string last = g_last_error;
@@ -286,8 +286,8 @@ void Ctx::destroy_pool(Pool& pool) {
   pool = Pool();
 }
 
-// Traces a launch through the pool: batches of half of it, seed_kernel then
-// trace_kernel, in turn on the context's stream and on a second one, which joins
+// Traces a launch through the pool: in one batch, or in batches of half of it,
+// seed_kernel then trace_kernel, in turn on the context's stream and on a second one, which joins
 // it again at the end.  A batch ends in a tail of its longest paths (up to 0.6 ms
 // on the satellite: 64 bounces, one after the other); the other stream's next
 // kernels fill it.  One stream and batches of 2^26, 2^27 particles: the attitude
@@ -310,7 +310,8 @@ cudaError_t Ctx::trace_pool(Pool& pool, cudaStream_t stream, TraceArgs a, uint32
     if (e == cudaSuccess && !*ev) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
   if (e != cudaSuccess) return e;
   uint64_t total = a.total;
-  uint64_t batch = std::min<uint64_t>(kPoolBatch, (pool.cap - 512) / (2 * (32 * kPoolEntryBytes + sizeof(uint32_t))) * 32);
+  const uint64_t entries = (pool.cap - pool_bytes(0)) / (32 * kPoolEntryBytes + sizeof(uint32_t)) * 32;
+  uint64_t batch = pool_batch(entries, total, pool.max_batch);
   // Segments of 32 to 2,048 work indices (a power of two): as long as the trace
   // grid still gets eight a warp to even out its work, or two behind rough rays,
   // where few particles of a segment pass.  Every segment costs a fetch, and behind

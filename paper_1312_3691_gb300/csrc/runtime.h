@@ -1,6 +1,7 @@
 // Host-side context of the TPMC library (not part of the ABI).
 #pragma once
 
+#include <algorithm>
 #include <condition_variable>
 #include <cstdint>
 #include <deque>
@@ -49,6 +50,7 @@ struct Scratch {
 struct Pool {
   void* ptr = nullptr;
   size_t cap = 0;
+  uint64_t max_batch = 0;
   cudaStream_t side = nullptr;
   cudaEvent_t fork = nullptr, join = nullptr, done = nullptr;
 };
@@ -92,23 +94,30 @@ constexpr uint64_t kPoolBatch = 1ull << 26, kPoolSmallest = 1ull << 23;
 constexpr uint64_t kPoolBatchesQueued = 896;
 constexpr uint32_t kPoolSegment = 2048;  // work indices of a segment, at most (a batch is a multiple)
 
-// Bytes of half a pool: entries for `batch` particles (a multiple of kPoolSegment) and a count for each segment of
-// 32 or more.
-constexpr size_t pool_bytes(uint64_t batch) {
-  return (size_t)batch * kPoolEntryBytes + (size_t)(batch / 32) * sizeof(uint32_t) + 256;
+// Bytes of a pool of `entries` particles (a multiple of 2 kPoolSegment), in two halves: the particles and a count for
+// each segment of 32 or more.
+constexpr size_t pool_bytes(uint64_t entries) {
+  return (size_t)entries * kPoolEntryBytes + (size_t)(entries / 32) * sizeof(uint32_t) + 512;
 }
 
-// Particles of a batch in a pool for launches of `total` particles, at most
-// max_batch, that takes at most half of `room` bytes; 0: there is no room for a
-// pool.  Powers of two, so that a program that raises its count from call to call
-// does not free and allocate a pool at each (40 calls of 2^24 particles and 2^20
-// more at each on a 60,000-triangle satellite: 161 -> 93 ms, 89 when repeated).
-constexpr uint64_t pool_batch(uint64_t total, uint64_t max_batch, size_t room) {
-  uint64_t batch = kPoolSegment;
-  while (batch < total && batch < max_batch) batch *= 2;
-  // a launch of one batch may be smaller than kPoolSmallest, as long as it stays one
-  while (batch > kPoolSmallest && 2 * pool_bytes(batch) > room / 2) batch /= 2;
-  return 2 * pool_bytes(batch) > room / 2 ? 0 : batch;
+// Particles of a batch in a pool of `entries`: a launch that fits into it, and into
+// max_batch, is one batch; others take its two halves in turn.
+constexpr uint64_t pool_batch(uint64_t entries, uint64_t total, uint64_t max_batch) {
+  return std::min(total <= entries && total <= max_batch ? entries : entries / 2, max_batch);
+}
+
+// Entries of a pool for launches of `total` particles that takes at most half of
+// `room` bytes; 0: there is no room for one.  Powers of two, so that a program that
+// raises its count from call to call does not free and allocate a pool at each (40
+// calls of 2^24 particles and 2^20 more at each on a 60,000-triangle satellite: 161
+// -> 92 ms, 89 when repeated).  A launch of one batch may be smaller than
+// kPoolSmallest, one of several has batches of at least that.
+constexpr uint64_t pool_entries(uint64_t total, uint64_t max_batch, size_t room) {
+  uint64_t n = 2 * kPoolSegment;
+  while (n < total && n < 2 * max_batch) n *= 2;
+  while (n > kPoolSegment && pool_bytes(n) > room / 2) n /= 2;
+  const bool one = total <= n && total <= max_batch;
+  return n > kPoolSegment && (one || n >= 2 * kPoolSmallest) ? n : 0;
 }
 
 float cv_area(const QueryDev& q);

@@ -334,7 +334,7 @@ bool enqueue_step(ServeState* s, int b, int prev, const std::vector<Request*>& c
       // whole at its first use: queries are served smallest first, and a pool that
       // grew with them was freed, which waits for the device, at every other step
       // (a context's first burst of 32 queries 55.2 -> 47.7 ms, its second 47.2)
-      if (B.pool.ptr || c->grow_pool(B.pool, kServePoolBatch, kServePoolBatch)) {
+      if (B.pool.ptr || c->grow_pool(B.pool, 2 * kServePoolBatch, kServePoolBatch)) {
         pooled = B.pooled = true;
         const uint32_t variant = groups[gi].first.second | kVariantPool;
         const MeshRec& mr = c->meshes.at(groups[gi].first.first);
