@@ -271,8 +271,10 @@ tpmc_status tpmc_trace_records(tpmc_ctx* ctx, tpmc_mesh_id mesh, const tpmc_para
                                tpmc_records* records, tpmc_result* out);
 
 /* Batched sweep: K queries that differ from `base` only in flow direction and
- * speed ratio, in one persistent launch.  h_dirs: host [K][3]; h_S: host [K]
- * speed ratios (V = S c_mp); either may be NULL, and then every item takes
+ * speed ratio, in one call: one persistent launch, or for FP32 sweeps of 2^22
+ * particles and more batches of up to 2^26, each seeded and traced by a launch.
+ * h_dirs: host [K][3]; h_S: host [K] speed ratios (V = S c_mp); either may be
+ * NULL, and then every item takes
  * base's direction or speed.  Item k uses stream_id = base->stream_id + k.
  * Per-panel loads are not kept.  Results in h_out[K].
  * Errors as tpmc_trace; EINVAL for K = 0 or K > 2^24. */
@@ -280,7 +282,8 @@ tpmc_status tpmc_sweep(tpmc_ctx* ctx, tpmc_mesh_id mesh, const tpmc_params* base
                        const double* h_S, uint32_t K, uint64_t N_each, tpmc_result* h_out);
 
 /* Device-resident form of tpmc_sweep: d_dirs, d_S and d_out are device
- * buffers; the call only enqueues work on the context's stream and returns.
+ * buffers; the call only enqueues work on the context's stream and returns
+ * (at most 896 batches; particles beyond them share one launch).
  * Per-item input errors are reported in d_out[k].status. */
 tpmc_status tpmc_sweep_device(tpmc_ctx* ctx, tpmc_mesh_id mesh, const tpmc_params* base, const double* d_dirs,
                               const double* d_S, uint32_t K, uint64_t N_each, tpmc_result* d_out);
@@ -332,7 +335,8 @@ tpmc_status tpmc_poll(tpmc_ctx* ctx, tpmc_query_id query, int timeout_ms, tpmc_r
  * fixed per-launch costs do not decide (N_trial of a few million or more keeps
  * the difference above the noise); a candidate must beat the untuned schedule
  * by 1 %.  The schedule is kept for meshes of the size class and this kernel
- * variant.  `best` (may be NULL) receives it.
+ * variant.  `best` (may be NULL) receives it.  Trials of FP32 queries with
+ * N_trial of 2^22 and more are four times as long.
  * Errors: as tpmc_trace; EINVAL for N_trial = 0 or > 2^30; ENOMEM when a
  * layout does not fit the memory budget (that width is then skipped). */
 tpmc_status tpmc_tune(tpmc_ctx* ctx, tpmc_mesh_id mesh, const tpmc_params* params, uint64_t N_trial,

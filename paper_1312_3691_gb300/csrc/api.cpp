@@ -223,10 +223,10 @@ float cv_area(const QueryDev& q) {
 }
 
 // A pool for launches of `total` particles in batches of at most max_batch, in the
-// memory the context's budget leaves (pool_entries); false when it has no room (the launch then seeds
-// inside the trace kernel).  A pool outlives its call, so a new one also takes at
-// most a quarter of the device's free memory: three quarters stay for whoever
-// shares the device and cannot ask for the pool back.
+// memory the context's budget leaves (pool_entries); false when it has no room (the
+// launch then seeds inside the trace kernel).  A pool outlives its call, so a new one
+// also takes at most a quarter of the device's free memory: three quarters stay for
+// whoever shares the device and cannot ask for the pool back.
 bool Ctx::grow_pool(Pool& pool, uint64_t total, uint64_t max_batch) {
   pool.max_batch = max_batch;
   size_t room = budget - std::min(budget, used - pool.cap);
@@ -287,11 +287,11 @@ void Ctx::destroy_pool(Pool& pool) {
 }
 
 // Traces a launch through the pool: in one batch, or in batches of half of it,
-// seed_kernel then trace_kernel, in turn on the context's stream and on a second one, which joins
-// it again at the end.  A batch ends in a tail of its longest paths (up to 0.6 ms
-// on the satellite: 64 bounces, one after the other); the other stream's next
-// kernels fill it.  One stream and batches of 2^26, 2^27 particles: the attitude
-// sweep 236 and 226 ms; two streams of 2^26: 217 (of 2^27: 211, for
+// seed_kernel then trace_kernel, in turn on the context's stream and on a second
+// one, which joins it again at the end.  A batch ends in a tail of its longest
+// paths (up to 0.6 ms on the satellite: 64 bounces, one after the other); the other
+// stream's next kernels fill it.  One stream and batches of 2^26, 2^27 particles:
+// the attitude sweep 236 and 226 ms; two streams of 2^26: 217 (of 2^27: 211, for
 // twice the memory).
 // a.counter: kRunCounters counters.  Particles beyond max_batches batches are traced
 // by one launch that seeds them itself.

@@ -171,7 +171,7 @@ __global__ void __launch_bounds__(kSetupThreads)
     q.fc[kFcScale] = (float)ldexp(1.0, shift);
     q.fc[kFcS] = (float)S;
     // Rough rays (may_hit): off by `da` radians on the CV, their velocity by da |v|
-    // + dv + S dc; emulated over the uniforms, da and dc are at most 1.6e-3 for S
+    // + dv + S dc; emulated over samples of the uniforms, da and dc are at most 1.6e-3 for S
     // below 3.5 and 4.4e-4 above (tests/test_rough_rays.py), dv 2.6e-3.  They pass the body within two CV radii
     // (or the box's diagonal) of the start.  Half as much again is added.
     const double vmin = fmax(0.5, 0.5 * S), da = S < 4.0 ? 1.7e-3 : 4.5e-4, dv = 2.6e-3;

@@ -10,13 +10,13 @@
 //      split, so nothing overtakes it midway), and queries behind it join the
 //      step while together they stay tiny,
 //   3. enqueues the step -- set-up of newly admitted queries, one persistent
-//      trace launch per (mesh, kernel variant) group over work items from all of
-//      the group's queries, the FP64 reduction of the queries that finish,
-//      the read-back -- while the previous step may still run.  Each of the
-//      two step buffers has its own streams, so a step's trace launches start
-//      on the SMs that the previous step's launch tails free up; the
-//      reduction waits for the traces of both steps, since a finishing query
-//      may have had work in the previous one, and
+//      trace launch (a large group: a pool's batches) per (mesh, kernel variant)
+//      group over work items from all of the group's queries, the FP64 reduction
+//      of the queries that finish, the read-back -- while the previous step may
+//      still run.  Each of the two step buffers has its own streams, so a step's
+//      trace launches start on the SMs that the previous step's launch tails free
+//      up; the reduction waits for the traces of both steps, since a finishing
+//      query may have had work in the previous one, and
 //   4. waits for the older step on the host (a CUDA event; no device-side
 //      wait), publishes its finished results and frees their slots.
 // A query's particles keep their ids 0..N-1 whatever steps they land in, and

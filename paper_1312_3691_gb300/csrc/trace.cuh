@@ -734,9 +734,10 @@ constexpr int kDone = (int)0x80000000;  // no valid leaf code: first + count wou
 
 // Traversal stack entry of binary trees: a stacked child and its entry distance
 // (float in both precisions: it is the box tests'), one 8-byte local-memory access
-// per push and per pop (two 4-byte arrays took two).  The pool kernel with its first four entries in shared memory
-// instead, and so a branch at each access and less L1: cylinder sweep 91.8 -> 92.7
-// ms, hemisphere 6.55 -> 6.59, moments 3.44 -> 3.48, attitude sweep 185.4 -> 186.8.
+// per push and per pop (two 4-byte arrays took two).  The pool kernel with its first
+// four entries in shared memory instead, and so a branch at each access and less L1:
+// cylinder sweep 91.8 -> 92.7 ms, hemisphere 6.55 -> 6.59, moments 3.44 -> 3.48,
+// attitude sweep 185.4 -> 186.8.
 struct __align__(8) StackE { int node; float t; };
 __device__ __forceinline__ void stack_put(StackE* s, int i, int node, float t) {
   *reinterpret_cast<int2*>(s + i) = make_int2(node, __float_as_int(t));
