@@ -6,8 +6,9 @@ Workload (one step): the plate / closed-cylinder sweep -- a 1 x 1 m plate
 over 32 angles of attack in [0, 90] deg x S in {2, 5, 10} x {specular, diffuse}
 re-emission, 1e7 particles per case (384 cases, 3.84e9 particles), atomic
 oxygen at T_inf = 1000 K, T_W = 300 K, FP32 traversal with FP64 set-up and
-reduction.  One step is four batched sweep launches (mesh x re-emission), each
-covering 96 cases in one persistent launch.
+reduction.  One step is four batched sweep calls (mesh x re-emission) of 96 cases
+each: a set-up, batches of 2^26 particles seeded and traced by a persistent launch
+each, and a reduction.
 
 value: traced particles per second with meshes resident on the device (CUDA
 events around each step on the launching stream; a 256 MiB L2 flush between
@@ -51,20 +52,29 @@ FLOPS_PER_TRI_TEST = 35      # watertight test: translate, shear, 3 edge functio
 FLOPS_PER_PARTICLE = 150     # seeding: two inverse-CDF solves, Box-Muller, two rotations
 FLOPS_PER_HIT = 30           # re-emission, momentum difference, torque, quantisation
 BYTES_PER_TRI_TEST = 48      # three float4 vertices
-# DRAM bytes per trace launch from an ncu capture, valid only for the kernel
-# source, its build flags and the BVH builder it was taken with (keyed by the
-# SHA-256 of trace.cuh, trace_w2.cu, kernels.cu, bvh.cpp and build.py, in that order).
+# DRAM bytes per sweep call from an ncu capture, valid only for the kernel source,
+# its build flags, the BVH builder and the host code that decides on the pool, its
+# batches and its entries it was taken with (keyed by the SHA-256 of TRAFFIC_SOURCES
+# in that order).
+TRAFFIC_SOURCES = ("csrc/trace.cuh", "csrc/trace_w2.cu", "csrc/kernels.cu", "csrc/bvh.cpp", "build.py", "csrc/api.cpp",
+                   "csrc/runtime.h", "csrc/tpmc_internal.h")
 # Mean over the four bench groups of dram__bytes_read.sum + dram__bytes_write.sum
 # over the seeding and trace launches of one full-size call (9.6e8 particles).
-TRACE_TRAFFIC = {"80bc31cba96006aebfad128063279869f40f07b4cc6b5495423ff91098c29647": 25_433_692_736}
+TRACE_TRAFFIC = {"98a95d7d657a0f1f2ce67b82a03d21c50748c6b69311e25a83394fe2fed13a5d": 25_431_364_480}
 
 
 def kernel_source_hash() -> str:
     h = hashlib.sha256()
-    for name in ("csrc/trace.cuh", "csrc/trace_w2.cu", "csrc/kernels.cu", "csrc/bvh.cpp", "build.py"):
+    for name in TRAFFIC_SOURCES:
         with open(os.path.join(ROOT, "paper_1312_3691_gb300", name), "rb") as f:
             h.update(f.read())
     return h.hexdigest()
+
+
+def launches_per_call(particles: int) -> int:
+    """Kernels of one sweep call of this size: the set-up, a seeding and a trace launch for every batch of the pool
+    (2^26 particles, the full size, which a device with nothing else on it has room for), and the reduction."""
+    return 2 + 2 * -(-particles // (1 << 26))
 
 
 def rank_stream_base(rank: int, group: int) -> int:
@@ -534,7 +544,7 @@ def measure_box_cv(T, ctx):
 def measure_moment_sweep(T, ctx, torch, stream, dev):
     """Restoring moment about the quarter chord (§III.D.1) on the synthetic
     satellite at the Table 1 conditions: alpha in [-90, 90] step 10 x 8 roll
-    angles = 152 attitudes x 2^22 particles in one persistent launch; the
+    angles = 152 attitudes x 2^22 particles in one sweep call; the
     pitching-moment coefficient C_m = -M.e_p / (q_inf c) (pitch-up positive, area-
     scaled, A_ref = 1 m^2) for the horizontal (beta 0) and vertical (beta 90) rolls."""
     case = W.satellite_moment_case(N=1)
@@ -582,8 +592,8 @@ def measure_moment_sweep(T, ctx, torch, stream, dev):
 
 def measure_attitude_sweep(T, ctx, torch, stream, dev, ceil):
     """32 x 32 yaw/pitch grid x S in {5, 7.5, 10} on the satellite, 2^20 particles per
-    item: one persistent launch against 3,072 one-query launches (same N, so equal
-    C_D error)."""
+    item: one sweep call against 3,072 one-query calls (same N, so equal C_D
+    error)."""
     case = W.satellite_case(N=1)
     grid = W.attitude_grid(32, 32)
     dirs = np.concatenate([grid] * 3)
@@ -852,9 +862,9 @@ def run_ours(args):
     parts = [(w, mesh_info[g["shape"]]["node_bytes"], mesh_info[g["shape"]]["bvh_width"])
              for w, g in zip(group_work, gs)]
     roof = roofline_of(parts, mean_step_s, ceil)
-    roof.update({"traffic": traffic, "kernel": "trace_kernel<float>",
-                 "achieved_definition": "algorithmic L2 bytes (node and triangle reads) per launch / mean launch "
-                                        "duration (CUDA events on the launching stream)",
+    roof.update({"traffic": traffic, "kernel": "seed_kernel<float> and trace_kernel<float>, all batches of a sweep call",
+                 "achieved_definition": "algorithmic L2 bytes (node and triangle reads) per sweep call / mean duration "
+                                        "of a call (CUDA events on the launching stream)",
                  "launch_ms_mean": statistics.mean(launch_ms),
                  "fp32_alu_derived_tflops": alu_peak_tflops,
                  "fp32_alu_basis": f"{props.multi_processor_count} SMs x {FP32_LANES_PER_SM} FP32 lanes x 2 (FMA) x "
@@ -879,11 +889,11 @@ def run_ours(args):
             "vs_baseline": None, "dtype": "f32",
             "data": "synthetic (procedural meshes; paper prints no absolute throughput)",
             "config": {"workload": WORKLOAD, "particles_per_step": particles_step, "cases": 4 * K,
-                       "launches_per_step": len(d_in), "l2": "256 MiB flush between steps, outside timed intervals",
+                       "sweep_calls_per_step": len(d_in), "l2": "256 MiB flush between steps, outside timed intervals",
                        "precision": "FP32 traversal, FP64 set-up and reduction"},
             "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": int(h2d), "d2h_bytes_per_step": int(d2h),
                     "ms_per_step": e2e_t, "includes": "mesh upload + BVH build, host inputs, host results"},
-            "gpu_launches": args.steps * len(d_in) * 3,
+            "gpu_launches": args.steps * len(d_in) * launches_per_call(len(gs[0]["dirs"]) * N_EACH),
             "roofline": roof,
             "clocks": clocks,
             "cpu_baseline": cpu_base,
